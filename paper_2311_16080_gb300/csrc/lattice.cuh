@@ -81,15 +81,24 @@ __host__ __device__ constexpr float weight(int i) {
   return (float)weight_d<Q>(i);
 }
 
+// opp(i): the direction with c = -c_i.  A table: a search through the
+// velocities here is unrolled and folded anew at each of the thousands of
+// places that ask, which took most of the build's time.
 template <int Q>
 __host__ __device__ constexpr int opposite(int i) {
-  int r = 0;
-  for (int k = 0; k < Q; ++k)
-    if (Lattice<Q>::c(k, 0) == -Lattice<Q>::c(i, 0) && Lattice<Q>::c(k, 1) == -Lattice<Q>::c(i, 1) &&
-        Lattice<Q>::c(k, 2) == -Lattice<Q>::c(i, 2))
-      r = k;
-  return r;
+  constexpr int t[27] = {0,  4,  5,  6,  1,  2,  3,  10, 9,  8,  7,  14, 13, 12,
+                         11, 18, 17, 16, 15, 26, 25, 24, 23, 22, 21, 20, 19};
+  constexpr int t9[9] = {0, 3, 4, 1, 2, 8, 7, 6, 5};
+  return Q == 9 ? t9[i < 9 ? i : 0] : t[i];
 }
+template <int Q>
+constexpr bool opposite_holds() {
+  for (int i = 0; i < Q; ++i)
+    for (int a = 0; a < 3; ++a)
+      if (Lattice<Q>::c(opposite<Q>(i), a) != -Lattice<Q>::c(i, a)) return false;
+  return true;
+}
+static_assert(opposite_holds<9>() && opposite_holds<19>() && opposite_holds<27>(), "opposite directions");
 
 // ---------------------------------------------------------------------------
 // Population storage.  Every storage type holds the deviation
