@@ -7,6 +7,7 @@
 //   j   = sum_i c_i df_i, u = j / rho          (Eq. 7; sum_i c_i w_i = 0)
 //   df_i^eq = w_i [drho + rho (3 c.u + 4.5 (c.u)^2 - 1.5 u.u)]   (Eq. 5)
 #pragma once
+#include "lane_math.cuh"
 #include "lattice.cuh"
 #include "xlb_types.h"
 
@@ -59,28 +60,30 @@ __device__ __forceinline__ void moments(const float (&df)[Q], float& drho, float
 // Moments of order 0, 1 and 2 of the deviations in one pass over the pairs
 // (i, opp(i)): their sum carries the even moments, their difference the odd.
 // M = sum_i c_ia c_ib df_i, stored xx yy zz xy xz yz.
-template <int Q>
-__device__ __forceinline__ void moments_kbc(const float (&df)[Q], float& drho, float (&j)[3], float (&M)[6]) {
+template <int Q, typename T>
+__device__ __forceinline__ void moments_kbc(const T (&df)[Q], T& drho, T (&j)[3], T (&M)[6]) {
+  constexpr int D = Lattice<Q>::D;
   drho = df[0];
-  j[0] = j[1] = j[2] = 0.f;
-#pragma unroll
-  for (int a = 0; a < 6; ++a) M[a] = 0.f;
+  bool fj[3] = {true, true, true}, fm[6] = {true, true, true, true, true, true};
+  auto acc = [](T& s, bool& first, int c, T x) {
+    s = first ? x : (c > 0 ? vadd(s, x) : vsub(s, x));
+    first = false;
+  };
 #pragma unroll
   for (int i = 1; i < Q; ++i) {
     if (opposite<Q>(i) > i) {
-      const float sp = df[i] + df[opposite<Q>(i)], dm = df[i] - df[opposite<Q>(i)];
-      constexpr int D = Lattice<Q>::D;
+      const T sp = vadd(df[i], df[opposite<Q>(i)]), dm = vsub(df[i], df[opposite<Q>(i)]);
       const int cx = Lattice<Q>::c(i, 0), cy = Lattice<Q>::c(i, 1), cz = D == 3 ? Lattice<Q>::c(i, 2) : 0;
-      drho += sp;
-      if (cx) j[0] += cx * dm;
-      if (cy) j[1] += cy * dm;
-      if (cz) j[2] += cz * dm;
-      if (cx) M[0] += sp;
-      if (cy) M[1] += sp;
-      if (cz) M[2] += sp;
-      if (cx * cy) M[3] += (float)(cx * cy) * sp;
-      if (cx * cz) M[4] += (float)(cx * cz) * sp;
-      if (cy * cz) M[5] += (float)(cy * cz) * sp;
+      drho = vadd(drho, sp);
+      if (cx) acc(j[0], fj[0], cx, dm);
+      if (cy) acc(j[1], fj[1], cy, dm);
+      if (cz) acc(j[2], fj[2], cz, dm);
+      if (cx) acc(M[0], fm[0], 1, sp);
+      if (cy) acc(M[1], fm[1], 1, sp);
+      if (cz) acc(M[2], fm[2], 1, sp);
+      if (cx * cy) acc(M[3], fm[3], cx * cy, sp);
+      if (cx * cz) acc(M[4], fm[4], cx * cz, sp);
+      if (cy * cz) acc(M[5], fm[5], cy * cz, sp);
     }
   }
 }
@@ -350,146 +353,202 @@ __device__ __forceinline__ void pull_cell(const S* __restrict__ src, const StepP
 // the bracket of Eq. 5 is b + a for i and b - a for opp(i), and every even
 // function of c (the KBC shear part, the second moments) is shared.
 
+// c_i . u, i < opp(i): the first non-zero component is +1
+template <int Q, typename T>
+__device__ __forceinline__ T vdot(int i, const T (&u)[3]) {
+  const int cx = Lattice<Q>::c(i, 0), cy = Lattice<Q>::c(i, 1), cz = Lattice<Q>::D == 3 ? Lattice<Q>::c(i, 2) : 0;
+  T s = cx ? u[0] : (cy ? u[1] : u[2]);
+  if (cx && cy) s = cy > 0 ? vadd(s, u[1]) : vsub(s, u[1]);
+  if ((cx || cy) && cz) s = cz > 0 ? vadd(s, u[2]) : vsub(s, u[2]);
+  return s;
+}
+
+template <int Q, typename T>
+__device__ __forceinline__ T vnorm2(const T (&u)[3]) {
+  const T s = vfma(u[0], u[0], vmul(u[1], u[1]));
+  return Lattice<Q>::D == 3 ? vfma(u[2], u[2], s) : s;
+}
+
 // Exact-difference body force: df_i += f_i^eq(rho, u + F/rho) - f_i^eq(rho, u).
-template <int Q>
-__device__ __forceinline__ void add_force(float (&df)[Q], float rho, const float (&u)[3], float usq,
-                                          const float (&F)[3]) {
-  const float ir = 1.0f / rho;
-  float v[3] = {u[0] + F[0] * ir, u[1] + F[1] * ir, u[2] + F[2] * ir};
-  if (Lattice<Q>::D == 2) v[2] = 0.f;
-  const float vsq = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-  const float dsq = -1.5f * (vsq - usq);
-  df[0] += weight<Q>(0) * rho * dsq;
+template <int Q, typename T>
+__device__ __forceinline__ void add_force(T (&df)[Q], T rho, T ir, const T (&u)[3], T usq, const float (&F)[3]) {
+  T v[3];
+#pragma unroll
+  for (int a = 0; a < Lattice<Q>::D; ++a) v[a] = vfma(vset<T>(F[a]), ir, u[a]);
+  const T dsq = vmul(vset<T>(-1.5f), vsub(vnorm2<Q>(v), usq));
+  df[0] = vfma(vmul(vset<T>(weight<Q>(0)), rho), dsq, df[0]);
 #pragma unroll
   for (int i = 1; i < Q; ++i) {
     if (opposite<Q>(i) > i) {
-      const float cu = cdot<Q>(i, u), cv = cdot<Q>(i, v);
-      const float e = 4.5f * (cv * cv - cu * cu) + dsq, o = 3.0f * (cv - cu);
-      const float wr = weight<Q>(i) * rho;
-      df[i] += wr * (e + o);
-      df[opposite<Q>(i)] += wr * (e - o);
+      const T cu = vdot<Q>(i, u), cv = vdot<Q>(i, v);
+      const T e = vfma(vset<T>(4.5f), vfma(cv, cv, vmul(vmul(cu, vset<T>(-1.0f)), cu)), dsq), o = vsub(cv, cu);
+      const T wr = vmul(vset<T>(weight<Q>(i)), rho);
+      df[i] = vfma(wr, vfma(vset<T>(3.0f), o, e), df[i]);
+      df[opposite<Q>(i)] = vfma(wr, vfma(vset<T>(-3.0f), o, e), df[opposite<Q>(i)]);
     }
   }
 }
 
-// KBC shear population ds_i from hd = D_aa / 2 (a = x, y, z) and
-// qo = Pi_ab / 4 (ab = xy, xz, yz); zero on the rest and corner directions.
-template <int Q>
-__device__ __forceinline__ float kbc_ds(int i, const float (&hd)[3], const float (&qo)[3]) {
-  const int cx = Lattice<Q>::c(i, 0), cy = Lattice<Q>::c(i, 1), cz = Lattice<Q>::c(i, 2);
-  if (nnz<Q>(i) == 1) return cx ? hd[0] : (cy ? hd[1] : hd[2]);
-  if (nnz<Q>(i) == 2) {
-    if (cx && cy) return (float)(cx * cy) * qo[0];
-    if (cx && cz) return (float)(cx * cz) * qo[1];
-    return (float)(cy * cz) * qo[2];
+// BGK (Eq. 3) on one cell (T = float) or two (T = F2), in place on deviations:
+// df_i += omega (df_i^eq - df_i), then the body force.
+template <int Q, typename T>
+__device__ __forceinline__ void collide_bgk(T (&df)[Q], const StepParams& p) {
+  T drho = df[0], j[3];
+#pragma unroll
+  for (int i = 1; i < Q; ++i) drho = vadd(drho, df[i]);
+#pragma unroll
+  for (int a = 0; a < Lattice<Q>::D; ++a) {
+    bool first = true;
+#pragma unroll
+    for (int i = 1; i < Q; ++i) {
+      const int c = Lattice<Q>::c(i, a);
+      if (c == 0) continue;
+      j[a] = first ? df[i] : (c > 0 ? vadd(j[a], df[i]) : vsub(j[a], df[i]));
+      first = false;
+    }
   }
-  return 0.f;
+  const T rho = vadd(vset<T>(1.0f), drho);
+  const T ir = vrcp(rho);
+  T u[3];
+#pragma unroll
+  for (int a = 0; a < Lattice<Q>::D; ++a) u[a] = vmul(j[a], ir);
+  const T usq = vnorm2<Q>(u);
+  const T b0 = vmul(vset<T>(-1.5f), usq);  // b of the rest direction (c = 0)
+  // df + omega (w x - df) as df - omega (df - w x), the same value
+  const T nom = vset<T>(-p.omega);
+  df[0] = vfma(nom, vfma(vset<T>(-weight<Q>(0)), vfma(rho, b0, drho), df[0]), df[0]);
+  const T r3 = vmul(rho, vset<T>(3.0f)), n3 = vmul(rho, vset<T>(-3.0f));
+#pragma unroll
+  for (int i = 1; i < Q; ++i) {
+    if (opposite<Q>(i) > i) {
+      const int k = opposite<Q>(i);
+      const T cu = vdot<Q>(i, u);
+      const T bb = vfma(rho, vfma(vmul(vset<T>(4.5f), cu), cu, b0), drho);
+      const T nw = vset<T>(-weight<Q>(i));
+      df[i] = vfma(nom, vfma(nw, vfma(r3, cu, bb), df[i]), df[i]);
+      df[k] = vfma(nom, vfma(nw, vfma(n3, cu, bb), df[k]), df[k]);
+    }
+  }
+  if (p.has_force) add_force<Q>(df, rho, ir, u, usq, p.F);
+}
+
+// KBC shear population ds_i, i < opp(i), from hd = D_aa / 2 (a = x, y, z) and
+// qo = Pi_ab / 4 (ab = xy, xz, yz) and their negatives nqo; directions with
+// one or two non-zero components (it is zero on the others).
+template <int Q, typename T>
+__device__ __forceinline__ T kbc_ds(int i, const T (&hd)[3], const T (&qo)[3], const T (&nqo)[3]) {
+  const int cx = Lattice<Q>::c(i, 0), cy = Lattice<Q>::c(i, 1), cz = Lattice<Q>::D == 3 ? Lattice<Q>::c(i, 2) : 0;
+  if (nnz<Q>(i) == 1) return cx ? hd[0] : (cy ? hd[1] : hd[2]);
+  const int k = cx && cy ? 0 : (cx && cz ? 1 : 2), c = cx && cy ? cx * cy : (cx && cz ? cx * cz : cy * cz);
+  return c > 0 ? qo[k] : nqo[k];
+}
+
+// KBC (Karlin, Bosch, Chikatamarla 2014) on one cell (T = float) or two
+// (T = F2): f^neq = ds + dh, beta = omega / 2,
+//   gamma = 1/beta - (2 - 1/beta) <ds|dh> / <dh|dh>,  <a|b> = sum a_i b_i / f_i^eq,
+//   f_i <- f_i - beta (2 ds_i + gamma dh_i)
+// where ds carries the deviatoric second moments of f^neq on the natural
+// moment basis: ds_i = D_aa / 2 for c_i = +-e_a, ds_i = c_ia c_ib Pi_ab / 4
+// for c_i with two non-zero components a, b, and 0 otherwise
+// (D_aa = Pi_aa - tr(Pi) / d).
+// The second moments of f^neq come from those of the deviations (moments_kbc)
+// and the closed form of the equilibrium's: on these lattices
+// sum_i c_ia c_ib f_i^eq = rho (d_ab / 3 + u_a u_b), so
+//   P_ab = M_ab - rho u_a u_b - d_ab drho / 3.
+// One pass then turns df into f^neq and forms <ds|dh> and <dh|dh>, with
+// dh = f^neq - ds; with them the update reads
+//   df_i <- df_i^eq + (1 - beta gamma) f^neq_i - beta (2 - gamma) ds_i.
+template <int Q, typename T>
+__device__ __forceinline__ void collide_kbc(T (&df)[Q], const StepParams& p) {
+  constexpr int D = Lattice<Q>::D;
+  const T mone = vset<T>(-1.0f);
+  T drho, j[3], M[6];
+  moments_kbc<Q>(df, drho, j, M);
+  const T rho = vadd(vset<T>(1.0f), drho), ir = vrcp(rho);
+  T u[3];
+#pragma unroll
+  for (int a = 0; a < D; ++a) u[a] = vmul(j[a], ir);
+  const T usq = vnorm2<Q>(u);
+  const T b0 = vmul(vset<T>(-1.5f), usq);  // b of the rest direction (c = 0)
+  const T nrho = vmul(rho, mone);
+  T nru[3], P[3], S;
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    nru[a] = vmul(nrho, u[a]);
+    P[a] = vfma(drho, vset<T>(-1.0f / 3.0f), vfma(nru[a], u[a], M[a]));
+    S = a == 0 ? P[0] : vadd(S, P[a]);
+  }
+  T hd[3], qo[3], nqo[3];
+#pragma unroll
+  for (int a = 0; a < D; ++a) hd[a] = vmul(vset<T>(0.5f), vfma(S, vset<T>(-1.0f / D), P[a]));
+#pragma unroll
+  for (int k = 0; k < (D == 3 ? 3 : 1); ++k) {
+    const int a = k == 2 ? 1 : 0, b = k == 0 ? 1 : 2;
+    qo[k] = vmul(vset<T>(0.25f), vfma(nru[a], u[b], M[3 + k]));
+    nqo[k] = vmul(qo[k], mone);
+  }
+  // <a|b> = sum a_i b_i / f_i^eq with f_i^eq = w_i rho (1 + b +- a); the
+  // common 1/rho cancels in gamma, and one reciprocal serves a pair:
+  // 1 / (X +- a) = (X -+ a) / (X^2 - a^2).  The rest direction has ds = 0.
+  const T e0 = vmul(vset<T>(weight<Q>(0)), vfma(rho, b0, drho));
+  df[0] = vsub(df[0], e0);
+  T hh = vmul(vmul(df[0], df[0]),
+              vdiv_fast(vset<T>(1.0f / weight<Q>(0)), vadd(vset<T>(1.0f), b0)));
+  T sh = vset<T>(0.0f);
+#pragma unroll
+  for (int i = 1; i < Q; ++i) {
+    if (opposite<Q>(i) > i) {
+      const int k = opposite<Q>(i);
+      const T cu = vdot<Q>(i, u), nw = vset<T>(-weight<Q>(i));
+      const T bq = vfma(vmul(vset<T>(4.5f), cu), cu, b0), a3 = vmul(vset<T>(3.0f), cu);
+      const T bb = vfma(rho, bq, drho);
+      const T fi = vfma(nw, vfma(rho, a3, bb), df[i]), fk = vfma(nw, vfma(nrho, a3, bb), df[k]);
+      df[i] = fi;
+      df[k] = fk;
+      const T X = vadd(vset<T>(1.0f), bq);
+      const T rc = vdiv_fast(vset<T>(1.0f / weight<Q>(i)), vfma(X, X, vmul(vmul(a3, mone), a3)));
+      const T ri = vmul(vsub(X, a3), rc), rk = vmul(vadd(X, a3), rc);
+      T hi = fi, hk = fk;
+      if (nnz<Q>(i) < 3) {
+        const T s = kbc_ds<Q>(i, hd, qo, nqo);
+        hi = vsub(fi, s);
+        hk = vsub(fk, s);
+        sh = vfma(s, vfma(hi, ri, vmul(hk, rk)), sh);
+      }
+      hh = vfma(vmul(hi, hi), ri, vfma(vmul(hk, hk), rk, hh));
+    }
+  }
+  const float beta = 0.5f * p.omega, ib = 1.0f / beta;
+  const T g = vsub(vset<T>(ib), vdiv(vmul(vset<T>(2.0f - ib), sh), hh));
+  const T gamma = vless(hh, vmul(vset<T>(1e-20f), rho), vset<T>(2.0f), g);
+  const T a1 = vfma(vset<T>(-beta), gamma, vset<T>(1.0f));
+  const T na2 = vmul(vset<T>(-beta), vsub(vset<T>(2.0f), gamma));
+  df[0] = vfma(a1, df[0], e0);
+  const T r3 = vmul(rho, vset<T>(3.0f)), n3 = vmul(rho, vset<T>(-3.0f));
+#pragma unroll
+  for (int i = 1; i < Q; ++i) {
+    if (opposite<Q>(i) > i) {
+      const int k = opposite<Q>(i);
+      const T cu = vdot<Q>(i, u), w = vset<T>(weight<Q>(i));
+      const T bb = vfma(rho, vfma(vmul(vset<T>(4.5f), cu), cu, b0), drho);
+      T si = vmul(a1, df[i]), sk = vmul(a1, df[k]);
+      if (nnz<Q>(i) < 3) {
+        const T nsd = vmul(na2, kbc_ds<Q>(i, hd, qo, nqo));
+        si = vfma(a1, df[i], nsd);
+        sk = vfma(a1, df[k], nsd);
+      }
+      df[i] = vfma(w, vfma(r3, cu, bb), si);
+      df[k] = vfma(w, vfma(n3, cu, bb), sk);
+    }
+  }
+  if (p.has_force) add_force<Q>(df, rho, ir, u, usq, p.F);
 }
 
 // Collision C of Eq. 1 on one fluid-like cell, in place on deviations.
-//   BGK (Eq. 3): df_i += omega (df_i^eq - df_i)
-//   KBC (Karlin, Bosch, Chikatamarla 2014): f^neq = ds + dh, beta = omega / 2,
-//     gamma = 1/beta - (2 - 1/beta) <ds|dh> / <dh|dh>,  <a|b> = sum a_i b_i / f_i^eq,
-//     f_i <- f_i - beta (2 ds_i + gamma dh_i)
-//   where ds carries the deviatoric second moments of f^neq on the natural
-//   moment basis: ds_i = D_aa / 2 for c_i = +-e_a, ds_i = c_ia c_ib Pi_ab / 4
-//   for c_i with two non-zero components a, b, and 0 otherwise
-//   (D_aa = Pi_aa - tr(Pi) / d).
-template <int Q, int COLL>
-__device__ __forceinline__ void collide(float (&df)[Q], const StepParams& p) {
-  if (COLL == COLL_NONE) return;
-  float drho, j[3], M[6];
-  if (COLL == COLL_KBC)
-    moments_kbc<Q>(df, drho, j, M);
-  else
-    moments<Q>(df, drho, j);
-  const float rho = 1.0f + drho;
-  const float ir = 1.0f / rho;
-  float u[3] = {j[0] * ir, j[1] * ir, j[2] * ir};
-  if (Lattice<Q>::D == 2) u[2] = 0.f;
-  const float usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-  float force_u[3];
-  if (p.has_force) {
-    force_u[0] = u[0];
-    force_u[1] = u[1];
-    force_u[2] = u[2];
-  }
-  const float b0 = -1.5f * usq;  // b of the rest direction (c = 0)
-  if (COLL == COLL_BGK) {
-    df[0] = fmaf(p.omega, weight<Q>(0) * (drho + rho * b0) - df[0], df[0]);
-#pragma unroll
-    for (int i = 1; i < Q; ++i) {
-      if (opposite<Q>(i) > i) {
-        const int j = opposite<Q>(i);
-        const float cu = cdot<Q>(i, u);
-        const float bb = drho + rho * fmaf(4.5f * cu, cu, b0), ra = rho * 3.0f * cu;
-        const float w = weight<Q>(i);
-        df[i] = fmaf(p.omega, w * (bb + ra) - df[i], df[i]);
-        df[j] = fmaf(p.omega, w * (bb - ra) - df[j], df[j]);
-      }
-    }
-  } else {
-    // KBC.  The second moments of f^neq come from those of the deviations
-    // (moments_kbc) and the closed form of the equilibrium's: on these
-    // lattices sum_i c_ia c_ib f_i^eq = rho (d_ab / 3 + u_a u_b), so
-    //   P_ab = M_ab - rho u_a u_b - d_ab drho / 3.
-    // One pass then turns df into f^neq and forms <ds|dh> and <dh|dh>, with
-    // dh = f^neq - ds; with them the update reads
-    //   df_i <- df_i^eq + (1 - beta gamma) f^neq_i - beta (2 - gamma) ds_i.
-    constexpr float third = 1.0f / 3.0f;
-    const float dd = drho * third;
-    const float P0 = M[0] - rho * u[0] * u[0] - dd, P1 = M[1] - rho * u[1] * u[1] - dd;
-    const float P2 = Lattice<Q>::D == 3 ? M[2] - rho * u[2] * u[2] - dd : 0.f;
-    constexpr float inv_d = 1.0f / Lattice<Q>::D;
-    const float tr = (P0 + P1 + P2) * inv_d;
-    // ds_i: D_aa / 2 on the axis directions, c_a c_b Pi_ab / 4 on the two-component ones
-    const float hd[3] = {0.5f * (P0 - tr), 0.5f * (P1 - tr), 0.5f * (P2 - tr)};
-    const float qo[3] = {0.25f * (M[3] - rho * u[0] * u[1]), 0.25f * (M[4] - rho * u[0] * u[2]),
-                         0.25f * (M[5] - rho * u[1] * u[2])};
-    // <a|b> = sum a_i b_i / f_i^eq with f_i^eq = w_i rho (1 + b +- a); the
-    // common 1/rho cancels in gamma, and one reciprocal serves a pair:
-    // 1 / (X +- a) = (X -+ a) / (X^2 - a^2).  The rest direction has ds = 0.
-    df[0] -= weight<Q>(0) * (drho + rho * b0);
-    float hh = df[0] * df[0] * __fdividef(1.0f / weight<Q>(0), 1.0f + b0), sh = 0.f;
-#pragma unroll
-    for (int i = 1; i < Q; ++i) {
-      if (opposite<Q>(i) > i) {
-        const int j = opposite<Q>(i);
-        const float cu = cdot<Q>(i, u);
-        const float w = weight<Q>(i);
-        const float bq = fmaf(4.5f * cu, cu, b0), a3 = 3.0f * cu;
-        const float bb = drho + rho * bq, ra = rho * a3;
-        const float fi = df[i] - w * (bb + ra), fj = df[j] - w * (bb - ra);
-        df[i] = fi;
-        df[j] = fj;
-        const float X = 1.0f + bq;
-        const float rc = __fdividef(1.0f / w, fmaf(X, X, -a3 * a3));
-        const float ri = (X - a3) * rc, rj = (X + a3) * rc;
-        const float s_ = kbc_ds<Q>(i, hd, qo);
-        const float hi = fi - s_, hj = fj - s_;
-        if (nnz<Q>(i) < 3) sh = fmaf(s_, fmaf(hi, ri, hj * rj), sh);
-        hh = fmaf(hi * hi, ri, fmaf(hj * hj, rj, hh));
-      }
-    }
-    const float beta = 0.5f * p.omega;
-    const float ib = 1.0f / beta;
-    const float gamma = (hh < 1e-20f * rho) ? 2.0f : ib - (2.0f - ib) * sh / hh;
-    const float a1 = 1.0f - beta * gamma, a2 = beta * (2.0f - gamma);
-    df[0] = fmaf(a1, df[0], weight<Q>(0) * (drho + rho * b0));
-#pragma unroll
-    for (int i = 1; i < Q; ++i) {
-      if (opposite<Q>(i) > i) {
-        const int j = opposite<Q>(i);
-        const float cu = cdot<Q>(i, u);
-        const float w = weight<Q>(i);
-        const float bb = drho + rho * fmaf(4.5f * cu, cu, b0), ra = rho * 3.0f * cu;
-        const float sd = a2 * kbc_ds<Q>(i, hd, qo);
-        df[i] = fmaf(w, bb + ra, fmaf(a1, df[i], -sd));
-        df[j] = fmaf(w, bb - ra, fmaf(a1, df[j], -sd));
-      }
-    }
-  }
-  if (p.has_force) add_force<Q>(df, rho, force_u, usq, p.F);
+template <int Q, int COLL, typename T>
+__device__ __forceinline__ void collide(T (&df)[Q], const StepParams& p) {
+  if constexpr (COLL == COLL_BGK) collide_bgk<Q>(df, p);
+  if constexpr (COLL == COLL_KBC) collide_kbc<Q>(df, p);
 }
 
 }  // namespace xlb
