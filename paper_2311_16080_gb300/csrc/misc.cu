@@ -29,13 +29,14 @@ __device__ __forceinline__ void cell_xyz(long long cell, int nx, int ny, bool sm
 
 // flags = type | FLAG_SLOW where a fluid-like cell has a WALL / LID / EQ cell
 // in its Q-stencil, or is an INLET / OUTLET / FWALL cell.  Codes >= 7 set
-// err[0]; an INLET, OUTLET or FWALL cell anywhere sets err[2].
+// err[0]; an INLET, OUTLET or FWALL cell anywhere sets bit 0 of err[2], a LID
+// or EQ cell bit 1.
 template <int Q>
 __global__ void k_mask_prepare(const uint8_t* __restrict__ mask, uint8_t* __restrict__ flags, int nx, int ny,
                                int nz, int* err) {
   // blocks stride over the rows (y, z), threads over x: no division per cell
   const long long rows = (long long)ny * nz;
-  bool io = false;
+  int seen = 0;
   for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
     const int y = (int)(row % ny), z = (int)(row / ny);
     const int ym = y == 0 ? ny - 1 : y - 1, yp = y == ny - 1 ? 0 : y + 1;
@@ -57,7 +58,7 @@ __global__ void k_mask_prepare(const uint8_t* __restrict__ mask, uint8_t* __rest
         continue;
       }
       int slow = (t == INLET || t == OUTLET || t == FWALL);
-      io |= slow != 0;
+      seen |= slow | (t == LID || t == EQ ? 2 : 0);
       if (fluid_like(t) && !slow) {
         const int xs[3] = {x == 0 ? nx - 1 : x - 1, x, x == nx - 1 ? 0 : x + 1};
 #pragma unroll
@@ -69,7 +70,7 @@ __global__ void k_mask_prepare(const uint8_t* __restrict__ mask, uint8_t* __rest
       flags[cell] = (uint8_t)(t | (slow ? FLAG_SLOW : 0));
     }
   }
-  if (io) atomicOr(err + 2, 1);
+  if (seen) atomicOr(err + 2, seen);
 }
 
 int launch_mask_prepare(int Q, const uint8_t* mask, uint8_t* flags, int nx, int ny, int nz, int* err,
