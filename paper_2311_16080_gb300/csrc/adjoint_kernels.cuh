@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(ROW_BLOCK) k_adjoint_init_grad(const float* __
 template <int Q, typename S>
 int launch_adj_typed(AdjOp op, const AdjointArgs& a) {
   const StepParams& p = a.p;
-  const long long nblk = row_blocks(p);
+  const long long nblk = cell_blocks(p);
   if (nblk <= 0) return 0;
   if (nblk > 0x7fffffffLL) return -1;
   const dim3 grid((unsigned)nblk), block(ROW_BLOCK);

@@ -55,6 +55,7 @@ struct xlb_ctx {
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int face[6] = {0, 0, 0, 0, 0, 0};  // described boundary faces (StepParams::face)
   bool x_linked = false;             // the x-faces' sources are served by ghost links
+  bool x_pull = false;               // ... which are the only ones: one cell per thread serves them itself
   bool x_inlet = false;              // the x = 0 plane is INLET, served by the bulk pass
   bool x_outlet = false;             // the x = nx - 1 plane is OUTLET, served by the bulk pass
   float* link_q = nullptr;  // Bouzidi wall distance per link (LINK_BZ entries), or null
@@ -179,6 +180,14 @@ static StepParams make_params(const xlb_ctx* c) {
   p.nz = (int)c->nz;
   p.plane = c->plane;
   p.omega = (float)c->omega;
+  // Rows that leave more than a tenth of their blocks' lanes idle: the cells
+  // as they lie in memory instead (97 x 83 x 61 FP32 periodic 10.4 us an
+  // update, 161 x 130 x 127 BF16 56 us; the 1761 x 330 cylinder, which wastes
+  // 2%, would lose 2% to the coordinates' divisions).
+  if ((c->nx + 127) / 128 * 128 * 10 > 11 * c->nx && c->nx >= 2) {
+    p.mag_x = magic_of((int)c->nx);
+    p.mag_y = magic_of((int)c->ny);
+  }
   p.has_mask = c->has_mask ? 1 : 0;
   p.flags = c->flags;
   p.has_force = c->has_force ? 1 : 0;
@@ -362,6 +371,8 @@ static int launch_step(xlb_ctx* c, const void* src, void* dst) {
   a.dst = dst;
   a.vec_width = bulk_variant(c) == XLB_KERNEL_VEC2 ? 2 : 4;
   a.p.has_mask = 0;  // bulk pass: every cell pulled as if periodic
+  const bool x_pull = c->x_pull && !vec;
+  if (x_pull) a.p.x_linked = 0;
   cudaEvent_t* pe = prof_begin(c, 0);
   const bool side = c->has_mask && c->n_fix > 0 && c->fix_side && c->aux;
   int r = XLB_OK;
@@ -386,9 +397,24 @@ static int launch_step(xlb_ctx* c, const void* src, void* dst) {
     cudaError_t e = cudaStreamWaitEvent(c->stream, c->ev_join, 0);
     if (!r && e != cudaSuccess) r = cuda_fail(c, e, "cudaStreamWaitEvent(join)");
   }
-  if (!r) r = boundary_pass(c, src, dst, side);
+  if (!r && !x_pull) r = boundary_pass(c, src, dst, side);
   prof_end(c, pe);
   return r;
+}
+
+// The ghost values of the links alone, once per call where the updates need
+// none (x_pull with one cell per thread): the wall force and the vector
+// kernels read them.
+static int write_links(xlb_ctx* c, void* dst) {
+  LaunchArgs a = base_args(c);
+  a.src = dst;
+  a.dst = dst;
+  a.links = c->links;
+  a.link_cells = c->link_cells;
+  a.link_q = c->link_q;
+  a.n_links = c->n_links;
+  a.fix_mode = FIX_STORED;
+  return dispatch(c, OP_BOUNDARY, a);
 }
 
 // Device error word (bounded waits that expired) -> XLB_ERR_TIMEOUT.
@@ -768,6 +794,7 @@ int xlb_set_mask(xlb_ctx* c, const uint8_t* mask) {
   int2* nlcells = nullptr;
   int* nfix = nullptr;
   long long nl = 0, nfx = 0;
+  bool new_x_pull = false;  // every link's source is on an x-face plane
   {
     const long long nb = bnd_list_blocks(c->N);
     int* counts = nullptr;
@@ -804,7 +831,17 @@ int xlb_set_mask(xlb_ctx* c, const uint8_t* mask) {
     if (e == cudaSuccess && nl > 0 &&
         launch_link_cells(c->Q, nlinks, nl, nf, (int)c->nx, (int)c->ny, (int)c->nz, nlcells, c->stream) != 0)
       e = cudaErrorInvalidValue;
+    int off_x = 1;
+    if (e == cudaSuccess && new_x_linked && nl > 0 && nfx == 0 && !new_x_inlet && !new_x_outlet) {
+      e = cudaMemsetAsync(c->err_word + 3, 0, sizeof(int), c->stream);
+      if (e == cudaSuccess &&
+          launch_links_off_x(nlcells, nl, (int)c->nx, new_face[0] != 0, new_face[1] != 0, c->err_word + 3, c->stream) != 0)
+        e = cudaErrorInvalidValue;
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(&off_x, c->err_word + 3, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    new_x_pull = e == cudaSuccess && off_x == 0;
     if (counts) cudaFree(counts);
     if (offs) cudaFree(offs);
     if (e != cudaSuccess) {
@@ -854,6 +891,7 @@ int xlb_set_mask(xlb_ctx* c, const uint8_t* mask) {
   c->has_lid_eq = new_le;
   for (int f = 0; f < 6; ++f) c->face[f] = new_face[f];
   c->x_linked = new_x_linked;
+  c->x_pull = new_x_pull;
   c->x_inlet = new_x_inlet;
   c->x_outlet = new_x_outlet;
   c->has_mask = true;
@@ -1230,6 +1268,7 @@ int xlb_step(xlb_ctx* c, int64_t n) {
     r = record_checkpoint(c);
     if (r) return r;
   }
+  if (c->x_pull && !use_vec(c) && c->kind_h && n > 0) return write_links(c, c->buf[c->cur]);
   return XLB_OK;
 }
 

@@ -2,9 +2,11 @@
 // instantiates them for one lattice and one storage type through
 // launch_typed; dispatch.cu routes (Q, storage) to those entry points.
 //
-// Thread mapping: one thread per cell; a block covers ROW_BLOCK consecutive x
-// of one (y, z) row and the grid is flattened over (x-blocks, rows), so every
-// warp touches 32 consecutive populations of each plane (coalesced).
+// Thread mapping: one thread per cell.  Where rows fill whole blocks a block
+// covers ROW_BLOCK consecutive x of one (y, z) row, which spares the cell its
+// coordinates' divisions; otherwise blocks run over the cells as they lie in
+// memory (x fastest, rows not padded), so that no lane idles at a row's end
+// and every warp still reads and writes consecutive populations.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -22,7 +24,30 @@ struct CellIdx {
   int self;
 };
 
-__device__ __forceinline__ bool cell_of_block(const StepParams& p, CellIdx& c) {
+// a / n and its remainder, m = magic_of(n)
+__device__ __forceinline__ int divide(int a, int n, uint32_t m, int& rem) {
+  if (m == 0u) {  // n = 1
+    rem = 0;
+    return a;
+  }
+  int q = (int)__umulhi((unsigned)a, m);
+  rem = a - q * n;
+  if (rem < 0) {
+    --q;
+    rem += n;
+  }
+  return q;
+}
+
+__device__ __forceinline__ bool cell_of_flat(const StepParams& p, CellIdx& c) {
+  c.self = (int)(blockIdx.x * (unsigned)ROW_BLOCK + threadIdx.x);
+  if ((unsigned)c.self >= (unsigned)(p.nx * p.ny * p.nz)) return false;
+  const int row = divide(c.self, p.nx, p.mag_x, c.x);
+  c.z = divide(row, p.ny, p.mag_y, c.y);
+  return true;
+}
+
+__device__ __forceinline__ bool cell_of_rows(const StepParams& p, CellIdx& c) {
   const unsigned nxb = (unsigned)(p.nx + ROW_BLOCK - 1) / ROW_BLOCK;
   const unsigned row = blockIdx.x / nxb;
   const unsigned xb = blockIdx.x - row * nxb;
@@ -34,10 +59,17 @@ __device__ __forceinline__ bool cell_of_block(const StepParams& p, CellIdx& c) {
   return true;
 }
 
-// Cell of a bulk-kernel thread: on a (x-blocks, ny, nz) grid when p.grid3,
-// else on the grid flattened over rows (cell_of_block).
+__device__ __forceinline__ bool cell_of_block(const StepParams& p, CellIdx& c) {
+  return p.mag_x ? cell_of_flat(p, c) : cell_of_rows(p, c);
+}
+
+// Cell of a bulk-kernel thread: flat over the cells (FLAT), on a (x-blocks, ny,
+// nz) grid when p.grid3, else on the grid flattened over rows.  FLAT is a
+// template argument: as a branch it cost the 256^3 FP32 cavity 1%.
+template <bool FLAT>
 __device__ __forceinline__ bool cell_of_grid(const StepParams& p, CellIdx& c) {
-  if (!p.grid3) return cell_of_block(p, c);
+  if (FLAT) return cell_of_flat(p, c);
+  if (!p.grid3) return cell_of_rows(p, c);
   c.x = (int)(blockIdx.x * ROW_BLOCK + threadIdx.x);
   if (c.x >= p.nx) return false;
   c.y = (int)blockIdx.y;
@@ -132,8 +164,65 @@ __device__ __forceinline__ int source_rule(uint32_t fc, int i, bool& skipped) {
   return t;
 }
 
+// The value a LID or EQ source w gives direction i of a cell, as its ghost
+// value would read: FP32 unrounded, 16-bit rounded into the storage type.
+// h_opp: the cell's own opposite population.
+template <typename S>
+__device__ __forceinline__ float ghost_value(const StepParams& p, int i, int w, int t, float h_opp) {
+  float v = t == EQ ? p.eq_df[i] : __fadd_rn(h_opp, p.lid_term[i]);
+  if constexpr (sizeof(S) == 2) {
+    S s;
+    const long long slot = (long long)i * p.plane + w;
+    st_ghost<S>(&s, (uint32_t)slot, v);
+    v = Store<S>::ld_plain(&s);
+  }
+  return v;
+}
+
+// Directions whose source lies on an x-face plane and is no skipped cell.
+template <int Q>
+__device__ __forceinline__ uint32_t x_rule_dirs(uint32_t fc) {
+  uint32_t m = (fc_type(fc, 0, 0) ? dir_bits<Q>(0, 1) : 0u) | (fc_type(fc, 0, 2) ? dir_bits<Q>(0, -1) : 0u);
+  if (fc & FC_RN) {
+#pragma unroll
+    for (int i = 1; i < Q; ++i) {
+      if (Lattice<Q>::c(i, 0) == 0) continue;
+      bool skipped;
+      source_rule<Q, false>(fc, i, skipped);
+      if (skipped) m &= ~(1u << i);
+    }
+  }
+  return m;
+}
+
+// Pull with the rules of the x-face planes (16-bit storage without FWALL
+// faces), the address chosen before the load so that a warp that meets an
+// x-face still issues one round of loads.
+template <int Q, typename S>
+__device__ __forceinline__ void pull_x_faces(const S* __restrict__ src, const StepParams& p, const Nbr& nb, int self,
+                                             uint32_t fc, uint32_t xr, float (&df)[Q]) {
+  const S* base = src;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    const S* a = base + src_index<Q>(nb, i);
+    if (Lattice<Q>::c(i, 0) != 0 && (xr >> i & 1)) a = src + (long long)opposite<Q>(i) * p.plane + self;
+    df[i] = Store<S>::ld(a);
+    base += p.plane;
+  }
+  if (p.face[0] <= WALL && p.face[1] <= WALL) return;
+  if (xr) {
+#pragma unroll
+    for (int i = 1; i < Q; ++i) {
+      if (Lattice<Q>::c(i, 0) == 0 || !(xr >> i & 1)) continue;
+      bool skipped;
+      const int t = source_rule<Q, false>(fc, i, skipped);
+      if (t == LID || t == EQ) df[i] = ghost_value<S>(p, i, src_index<Q>(nb, i), t, df[i]);
+    }
+  }
+}
+
 // Rules by coordinates for the sources on x-face planes in ordinary rows
-// (after a plain pull of the cell): WALL: h_opp(i)(x);  LID: h_opp(i)(x) +
+// (after a plain pull of the cell; lattices with an FWALL face): WALL: h_opp(i)(x);  LID: h_opp(i)(x) +
 // 2 w_i rho_w (c_i . u_w) / cs^2;  EQ: f_i^eq(rho_w, u_w).
 template <int Q, typename S, bool FW>
 __device__ __forceinline__ void x_face_rules(const S* __restrict__ src, const StepParams& p, int self, uint32_t fc,
@@ -239,11 +328,11 @@ struct GhostFaces {
 // GhostFaces describes; cells on FWALL face planes reverse instead of
 // colliding (FW).  Other boundary cells get values nobody reads until
 // k_boundary rewrites them; inlet / outlet cells are recomputed there too.
-template <int Q, typename S, int COLL, bool FW, bool IO = false>
+template <int Q, typename S, int COLL, bool FW, bool IO, bool FLAT>
 __global__ void __launch_bounds__(ROW_BLOCK, MinBlocks<Q, S, COLL>::value)
     k_stream_collide(const S* __restrict__ src, S* __restrict__ dst, const StepParams p) {
   CellIdx c;
-  if (!cell_of_grid(p, c)) return;
+  if (!cell_of_grid<FLAT>(p, c)) return;
   float df[Q];
   uint32_t fc = 0u;
   bool fwall = false;
@@ -258,8 +347,16 @@ __global__ void __launch_bounds__(ROW_BLOCK, MinBlocks<Q, S, COLL>::value)
     Nbr nb;
     make_nbr(nb, c.x, c.y, c.z, p.nx, p.ny, p.nz);
     if (outl) nb.xo[2] = c.x;
-    pull_plain<Q, S>(src, p, nb, df);
-    if (fc & FC_XN) x_face_rules<Q, S, FW>(src, p, c.self, fc, df);
+    if constexpr (FW) {
+      pull_plain<Q, S>(src, p, nb, df);
+      if (fc & FC_XN) x_face_rules<Q, S, FW>(src, p, c.self, fc, df);
+    } else {
+      const uint32_t xr = (fc & FC_XN) ? x_rule_dirs<Q>(fc) : 0u;
+      if (__any_sync(__activemask(), xr))
+        pull_x_faces<Q, S>(src, p, nb, c.self, fc, xr, df);
+      else
+        pull_plain<Q, S>(src, p, nb, df);
+    }
     fwall = (fc & FC_FWALL) != 0u;
   } else {
     Nbr nb;
@@ -284,7 +381,7 @@ __global__ void __launch_bounds__(ROW_BLOCK, MinBlocks<Q, S, COLL>::value)
 template <int Q, typename S, bool FW>
 __global__ void __launch_bounds__(ROW_BLOCK) k_face_ghosts(S* f, const StepParams p) {
   CellIdx c;
-  if (!cell_of_grid(p, c)) return;
+  if (!cell_of_block(p, c)) return;
   const uint32_t fc = face_code<FW>(p, c.x, c.y, c.z);
   if (!(fc & FC_RN) || (fc & FC_SKIP)) return;
   float hs[Q];
@@ -489,15 +586,15 @@ __global__ void __launch_bounds__(ROW_BLOCK) k_fix_recompute(const S* __restrict
 
 // ---------------------------------------------------------------------------
 // Vectorised bulk kernel.  Each thread owns V consecutive cells of one row
-// (x0 = V * slot); a warp covers 32 V consecutive cells and never straddles a
-// row.  Every direction is one aligned V-wide load of the source row at x0;
+// (x0 = V * slot); slots run on over the rows.  Every direction is one aligned V-wide load of the source row at x0;
 // the pull's x shift by c_x = +-1 takes the missing end element from the
 // neighbouring lane with a warp shuffle, and only the lane at the warp's (or
 // row's) edge loads it from memory, with the periodic wrap.  Faces as for
 // the one-cell kernel with 16-bit storage: the rows of y / z faces are
-// skipped (whole warps) and receive ghost values from the rows next to
-// them; sources on x-face planes are ghost links (16-bit storage) or take
-// the rule in the lanes at the ends of a row.  Stores are V-wide.  Needs
+// skipped and receive ghost values from the rows next to them; sources on
+// x-face planes are ghost links (a choice of address in the edge loads of the
+// row ends slowed every warp: 313 us against 234 us on the 256^3 FP16 periodic
+// box).  Stores are V-wide.  Needs
 // nx % V == 0; no FWALL faces.
 
 template <int Q, typename S, int COLL, int V>
@@ -507,26 +604,28 @@ struct VecMinBlocks {
 
 template <int Q, typename S, int COLL, int V>
 __global__ void __launch_bounds__(128, VecMinBlocks<Q, S, COLL, V>::value)
-    k_sc_vec(const S* __restrict__ src, S* __restrict__ dst, const StepParams p) {
+    k_sc_vec(const S* __restrict__ src, S* __restrict__ dst, const StepParams p, uint32_t slot_mag, uint32_t row_mag) {
   const int nx = p.nx, ny = p.ny, nz = p.nz;
-  const int spr = (nx / V + 31) / 32 * 32;  // slots per row, whole warps
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int row = (int)(t / spr);
-  if (row >= ny * nz) return;  // whole warps only
-  const int slot = (int)(t - (long long)row * spr);
+  // slots of V cells run on over the rows; the lanes beyond the last one
+  // repeat it and store nothing
+  const int spr = nx / V, total = spr * (ny * nz);
+  const int t = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  int slot, y;
+  const int row = divide(t < total ? t : total - 1, spr, slot_mag, slot);
+  const int z = divide(row, ny, row_mag, y);
   const int lane = threadIdx.x & 31;
-  const bool active = slot * V < nx;
-  const int x0 = active ? slot * V : nx - V;
-  const int y = row % ny, z = row / ny;
-  // face types of the row's coordinates (uniform over the warp); a row on a
-  // WALL / LID / EQ face plane holds ghost values only
+  const int x0 = slot * V;
+  bool active = t < total;
+  // face types of the row's coordinates; a row on a WALL / LID / EQ face
+  // plane holds ghost values only
   int ty[3] = {0, 0, 0}, tz[3] = {0, 0, 0};
   if (p.has_faces) {
     axis_face_types(y, ny, p.face[2], p.face[3], ty);
     axis_face_types(z, nz, p.face[4], p.face[5], tz);
-    if (face_combine<false>(0, ty[1], tz[1]) != 0) return;  // the whole warp
+    if (face_combine<false>(0, ty[1], tz[1]) != 0) active = false;
   }
-  const bool last = !active || x0 + V >= nx;  // no active right neighbour lane
+  if (!__any_sync(0xffffffffu, active)) return;  // (a skipped row's lanes still take part in the shuffles)
+  const bool last = slot == spr - 1;           // no right neighbour lane of this row
   const int xm = x0 == 0 ? nx - 1 : x0 - 1;    // element left of the vector
   // element right of the vector; an OUTLET plane at x = nx - 1 served here
   // copies the pull of x - 1 in the directions c_x = -1, whose sources lie in
@@ -554,7 +653,7 @@ __global__ void __launch_bounds__(128, VecMinBlocks<Q, S, COLL, V>::value)
       for (int k = 0; k < V; ++k) v[i][k] = w[k];
     } else if (cx == 1) {  // pull from x - 1
       const float up = __shfl_up_sync(0xffffffffu, w[V - 1], 1);
-      v[i][0] = lane > 0 ? up : Store<S>::ld(r + xm);
+      v[i][0] = (lane > 0 && slot > 0) ? up : Store<S>::ld(r + xm);
 #pragma unroll
       for (int k = 1; k < V; ++k) v[i][k] = w[k - 1];
     } else {  // pull from x + 1
@@ -575,36 +674,40 @@ __global__ void __launch_bounds__(128, VecMinBlocks<Q, S, COLL, V>::value)
 #pragma unroll
     for (int i = 0; i < Q; ++i) v[i][0] = d[i];
   }
-  // sources on x-face planes (only the lanes at the ends of a row have them;
-  // none when ghost links serve them)
-  if (p.has_faces && !p.x_linked && (x0 <= 1 || x0 + V >= nx - 1)) {
+  CellRound<S> rnd[V];
+  // 4 cells: two at a time in packed arithmetic (half the FP32 instructions at
+  // half their rate, so what it frees is issue slots: 256^3 FP16 periodic
+  // 233.6 -> 225.0 us); with 2 cells the register pairs cost more than that
+  // (cavity 269.6 -> 274.8 us)
+  if constexpr (V == 4) {
+#pragma unroll
+    for (int k = 0; k < V; k += 2) {
+      // two cells at once, in packed arithmetic
+      F2 f[Q];
+#pragma unroll
+      for (int i = 0; i < Q; ++i) f[i] = pack2(v[i][k], v[i][k + 1]);
+      collide<Q, COLL>(f, p);
+#pragma unroll
+      for (int i = 0; i < Q; ++i) unpack2(f[i], v[i][k], v[i][k + 1]);
+    }
 #pragma unroll
     for (int k = 0; k < V; ++k) {
-      int tx[3];
-      axis_face_types(x0 + k, nx, p.face[0], p.face[1], tx);
-      if ((tx[0] | tx[2]) == 0 || tx[1] != 0) continue;  // no x-face source, or an x-face cell itself
-      uint32_t fc = (ty[0] | ty[1] | ty[2] | tz[0] | tz[1] | tz[2]) != 0 ? FC_RN : 0u;
-#pragma unroll
-      for (int a = 0; a < 3; ++a)
-        fc |= (uint32_t)tx[a] << (3 * a) | (uint32_t)ty[a] << (3 * (3 + a)) | (uint32_t)tz[a] << (3 * (6 + a));
       float d[Q];
 #pragma unroll
       for (int i = 0; i < Q; ++i) d[i] = v[i][k];
-      x_face_rules<Q, S, false>(src, p, self0 + k, fc, d);
+      rnd[k].begin((uint32_t)(self0 + k), d);
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+      float d[Q];
+#pragma unroll
+      for (int i = 0; i < Q; ++i) d[i] = v[i][k];
+      collide<Q, COLL>(d, p);
+      rnd[k].begin((uint32_t)(self0 + k), d);
 #pragma unroll
       for (int i = 0; i < Q; ++i) v[i][k] = d[i];
     }
-  }
-  CellRound<S> rnd[V];
-#pragma unroll
-  for (int k = 0; k < V; ++k) {
-    float d[Q];
-#pragma unroll
-    for (int i = 0; i < Q; ++i) d[i] = v[i][k];
-    collide<Q, COLL>(d, p);
-    rnd[k].begin((uint32_t)(self0 + k), d);
-#pragma unroll
-    for (int i = 0; i < Q; ++i) v[i][k] = d[i];
   }
   if (!active) return;
   // ghost values for the skipped face rows next to this row (from registers,
@@ -877,9 +980,8 @@ __global__ void __launch_bounds__(256) k_wall_force(const S* __restrict__ f, con
 template <int Q, typename S, int COLL>
 int launch_typed(Op op, const LaunchArgs& a) {
   const StepParams& p = a.p;
-  const long long rows = (long long)p.ny * p.nz;
   const long long nxb = (p.nx + ROW_BLOCK - 1) / ROW_BLOCK;
-  const long long nblk = rows * nxb;
+  const long long nblk = cell_blocks(p);
   if (nblk <= 0) return 0;
   if (nblk > 0x7fffffffLL) return -1;
   const dim3 grid((unsigned)nblk), block(ROW_BLOCK);
@@ -890,7 +992,7 @@ int launch_typed(Op op, const LaunchArgs& a) {
       // bulk kernels run on an (x-blocks, ny, nz) grid where it fits
       StepParams q = p;
       dim3 g3 = grid;
-      if (p.ny <= 65535 && p.nz <= 65535) {
+      if (!p.mag_x && p.ny <= 65535 && p.nz <= 65535) {
         q.grid3 = 1;
         g3 = dim3((unsigned)nxb, (unsigned)p.ny, (unsigned)p.nz);
       }
@@ -899,17 +1001,19 @@ int launch_typed(Op op, const LaunchArgs& a) {
       if (op == OP_FACE_GHOSTS) {
         if (!p.has_faces || !GhostFaces<S>::value) return 0;
         if (fw)
-          k_face_ghosts<Q, S, true><<<g3, block, 0, st>>>((S*)a.dst, q);
+          k_face_ghosts<Q, S, true><<<grid, block, 0, st>>>((S*)a.dst, p);
         else
-          k_face_ghosts<Q, S, false><<<g3, block, 0, st>>>((S*)a.dst, q);
+          k_face_ghosts<Q, S, false><<<grid, block, 0, st>>>((S*)a.dst, p);
         return 0;
       }
-      if (fw)
-        k_stream_collide<Q, S, COLL, true><<<g3, block, 0, st>>>((const S*)a.src, (S*)a.dst, q);
-      else if (p.x_inlet || p.x_outlet)
-        k_stream_collide<Q, S, COLL, false, true><<<g3, block, 0, st>>>((const S*)a.src, (S*)a.dst, q);
-      else
-        k_stream_collide<Q, S, COLL, false><<<g3, block, 0, st>>>((const S*)a.src, (S*)a.dst, q);
+      const bool io = p.x_inlet || p.x_outlet;
+      auto kern = q.mag_x ? (fw ? k_stream_collide<Q, S, COLL, true, false, true>
+                                : io ? k_stream_collide<Q, S, COLL, false, true, true>
+                                     : k_stream_collide<Q, S, COLL, false, false, true>)
+                          : (fw ? k_stream_collide<Q, S, COLL, true, false, false>
+                                : io ? k_stream_collide<Q, S, COLL, false, true, false>
+                                     : k_stream_collide<Q, S, COLL, false, false, false>);
+      kern<<<g3, block, 0, st>>>((const S*)a.src, (S*)a.dst, q);
       return 0;
     }
     case OP_STEP_VEC: {
@@ -919,13 +1023,13 @@ int launch_typed(Op op, const LaunchArgs& a) {
       if constexpr (sizeof(S) == 2 && Q != 27 && COLL == COLL_BGK) {
         const int V = a.vec_width == 2 ? 2 : 4;
         if (p.nx % V != 0) return -7;
-        const long long spr = (p.nx / V + 31) / 32 * 32;
-        const long long blocks = (spr * p.ny * p.nz + 127) / 128;
-        if (blocks > 0x7fffffffLL) return -1;
+        const int spr = p.nx / V;
+        const long long blocks = ((long long)spr * p.ny * p.nz + 127) / 128;
+        const uint32_t sm = magic_of(spr), rm = magic_of(p.ny);
         if (V == 2)
-          k_sc_vec<Q, S, COLL, 2><<<(unsigned)blocks, 128, 0, st>>>((const S*)a.src, (S*)a.dst, p);
+          k_sc_vec<Q, S, COLL, 2><<<(unsigned)blocks, 128, 0, st>>>((const S*)a.src, (S*)a.dst, p, sm, rm);
         else
-          k_sc_vec<Q, S, COLL, 4><<<(unsigned)blocks, 128, 0, st>>>((const S*)a.src, (S*)a.dst, p);
+          k_sc_vec<Q, S, COLL, 4><<<(unsigned)blocks, 128, 0, st>>>((const S*)a.src, (S*)a.dst, p, sm, rm);
         return 0;
       }
       return -7;

@@ -59,8 +59,10 @@ int launch_d2q9(Op op, const LaunchArgs& a);
 int launch_d3q19(Op op, const LaunchArgs& a);
 int launch_d3q27(Op op, const LaunchArgs& a);
 
-// Number of blocks the row-mapped kernels launch for a lattice (partials).
+// Rows of block partials a lattice's scratch holds: one per 128 cells of a row.
 long long row_blocks(const StepParams& p);
+// Blocks the kernels mapped on cells launch (cell_of_block).
+long long cell_blocks(const StepParams& p);
 
 // Mask preparation: validates codes (< 7), writes flag bytes; err_word[0] is
 // set to 1 on an invalid code, bit 0 of err_word[2] where an INLET, OUTLET or
@@ -95,8 +97,11 @@ int launch_pred_count(int Q, const int* face, bool x_in, bool x_out, const uint8
                       int* counts, void* stream);
 int launch_pred_write(int Q, const int* face, bool x_in, bool x_out, const uint8_t* flags, int nx, int ny, int nz,
                       const long long* offs, int2* links, int* cells, void* stream);
+// *flag is set to 1 if some link's source (cells: launch_link_cells) lies off
+// the face planes among x = 0 (face0) and x = nx - 1 (face1).
 // Per link {cell x, dir i | ...}: the source cell x - c_i (periodic) and the
 // cell x + c_i when it is FLUID, else -1 (the boundary pass's Bouzidi partner).
+int launch_links_off_x(const int2* cells, long long n, int nx, bool face0, bool face1, int* flag, void* stream);
 int launch_link_cells(int Q, const int2* links, long long n, const uint8_t* flags, int nx, int ny, int nz,
                       int2* cells, void* stream);
 

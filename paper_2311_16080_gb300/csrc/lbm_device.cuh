@@ -115,10 +115,41 @@ __device__ __forceinline__ float cdot(int i, const float (&u)[3]) {
 //   EQ: f_i^eq(rho_w, u_w) (no load);  FWALL: the plain pull.
 // WALL / LID / EQ sources elsewhere hold ghost values (k_boundary).
 
-// Face type of the source coordinate index k (0: v - 1, 1: v, 2: v + 1) on
-// one axis: lo / hi are the face types of coordinate 0 and n - 1.
-__device__ __forceinline__ int face_code(int v, int n) {
-  return (v == 0 ? 1 : 0) | (v == n - 1 ? 2 : 0);
+// Bit i of the result: c_i has component v on the axis (i >= 1).
+template <int Q>
+__host__ __device__ constexpr uint32_t dir_bits(int axis, int v) {
+  uint32_t m = 0;
+  for (int i = 1; i < Q; ++i)
+    if (Lattice<Q>::c(i, axis) == v) m |= 1u << i;
+  return m;
+}
+
+// Directions of one cell whose source lies on a boundary face, one bit each:
+// they load the cell's own opposite population (own); of those, lid adds the
+// moving wall's term and eq takes the equilibrium value.  WALL wins where planes meet,
+// then FWALL (a plain pull).
+struct FaceDirs {
+  uint32_t own, lid, eq;
+};
+
+// The directions `at` gives for each face: the source lies on that plane.
+__device__ __forceinline__ FaceDirs face_dirs(const StepParams& p, const uint32_t (&at)[6]) {
+  uint32_t wall = 0u, fw = 0u, lid = 0u, eq = 0u;
+#pragma unroll
+  for (int f = 0; f < 6; ++f) {
+    // the types are the same for the whole launch
+    const int t = p.face[f];
+    if (t == WALL) wall |= at[f];
+    if (t == FWALL) fw |= at[f];
+    if (t == LID) lid |= at[f];
+    if (t == EQ) eq |= at[f];
+  }
+  fw |= wall;
+  FaceDirs d;
+  d.lid = lid & ~fw;
+  d.eq = eq & ~fw;
+  d.own = wall | d.lid | d.eq;
+  return d;
 }
 
 // Rule a source takes, from the three axes' face types of its coordinates:
@@ -154,31 +185,36 @@ __device__ __forceinline__ void reverse_populations(float (&df)[Q]) {
 template <int Q, typename S, bool FW = true>
 __device__ __forceinline__ bool pull_periodic(const S* __restrict__ src, const StepParams& p, const Nbr& nb,
                                               int self, int x, int y, int z, float (&df)[Q], bool outlet = false) {
-  int fcx[3] = {0, 0, 0}, fcy[3] = {0, 0, 0}, fcz[3] = {0, 0, 0};
+  // per face, the directions whose source is on it: a source coordinate v - c
+  // equal to the face's, c = +-1
+  uint32_t at[6] = {0u, 0u, 0u, 0u, 0u, 0u};
   bool near = false;
   if (p.has_faces) {
-    const int xs[3] = {nb.xo[0], x, nb.xo[2]};
-    if (y > 1 && y < p.ny - 2 && (p.nz == 1 || (z > 1 && z < p.nz - 2))) {
-      // a row two or more planes from the y / z face planes (uniform over a
-      // warp) can only meet x-faces
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const int cx = face_code(xs[k], p.nx);
-        fcx[k] = (cx & 1 ? p.face[0] : 0) | (cx & 2 ? p.face[1] : 0);
-        near |= (k != 1 || FW) && fcx[k];
-      }
-    } else {
-      const int ys[3] = {wrap_m(y, p.ny), y, wrap_p(y, p.ny)};
-      const int zs[3] = {p.nz > 1 ? wrap_m(z, p.nz) : 0, z, p.nz > 1 ? wrap_p(z, p.nz) : 0};
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const int cx = face_code(xs[k], p.nx), cy = face_code(ys[k], p.ny), cz = face_code(zs[k], p.nz);
-        fcx[k] = (cx & 1 ? p.face[0] : 0) | (cx & 2 ? p.face[1] : 0);
-        fcy[k] = (cy & 1 ? p.face[2] : 0) | (cy & 2 ? p.face[3] : 0);
-        fcz[k] = p.nz > 1 ? ((cz & 1 ? p.face[4] : 0) | (cz & 2 ? p.face[5] : 0)) : 0;
-        near |= (k != 1 || FW) && (fcx[k] | fcy[k] | fcz[k]);
+    const int lx = p.nx - 1, ly = p.ny - 1, lz = p.nz - 1;
+    const int xp = nb.xo[2];  // the coordinate x + 1, or x itself (outlet)
+    if (p.face[0] | p.face[1]) {
+      at[0] = (nb.xo[0] == 0 ? dir_bits<Q>(0, 1) : 0u) | (xp == 0 ? dir_bits<Q>(0, -1) : 0u);
+      at[1] = (nb.xo[0] == lx ? dir_bits<Q>(0, 1) : 0u) | (xp == lx ? dir_bits<Q>(0, -1) : 0u);
+    }
+    // a row two or more planes from the y / z face planes (uniform over a
+    // warp that covers one row) can only meet x-faces
+    if (!(y > 1 && y < p.ny - 2 && (p.nz == 1 || (z > 1 && z < p.nz - 2)))) {
+      const int ym = wrap_m(y, p.ny), yp = wrap_p(y, p.ny);
+      at[2] = (ym == 0 ? dir_bits<Q>(1, 1) : 0u) | (yp == 0 ? dir_bits<Q>(1, -1) : 0u);
+      at[3] = (ym == ly ? dir_bits<Q>(1, 1) : 0u) | (yp == ly ? dir_bits<Q>(1, -1) : 0u);
+      if (Lattice<Q>::D == 3 && p.nz > 1) {
+        const int zm = wrap_m(z, p.nz), zp = wrap_p(z, p.nz);
+        at[4] = (zm == 0 ? dir_bits<Q>(2, 1) : 0u) | (zp == 0 ? dir_bits<Q>(2, -1) : 0u);
+        at[5] = (zm == lz ? dir_bits<Q>(2, 1) : 0u) | (zp == lz ? dir_bits<Q>(2, -1) : 0u);
       }
     }
+#pragma unroll
+    for (int f = 0; f < 6; ++f)
+      if (!p.face[f]) at[f] = 0u;
+    near = (at[0] | at[1] | at[2] | at[3] | at[4] | at[5]) != 0u;
+    if (FW)
+      near |= (x == 0 && p.face[0]) || (x == lx && p.face[1]) || (y == 0 && p.face[2]) || (y == ly && p.face[3]) ||
+              (p.nz > 1 && ((z == 0 && p.face[4]) || (z == lz && p.face[5])));
   }
   const S* base = src;
   // warp-uniform choice: a warp with no lane next to a face loads plainly;
@@ -192,28 +228,35 @@ __device__ __forceinline__ bool pull_periodic(const S* __restrict__ src, const S
     }
     return false;
   }
+  // cells on a face plane: their sources with c = 0 are on it too
+  if (p.face[0] && x == 0) at[0] |= dir_bits<Q>(0, 0);
+  if (p.face[1] && x == p.nx - 1) at[1] |= dir_bits<Q>(0, 0);
+  if (p.face[2] && y == 0) at[2] |= dir_bits<Q>(1, 0);
+  if (p.face[3] && y == p.ny - 1) at[3] |= dir_bits<Q>(1, 0);
+  if (p.face[4] && p.nz > 1 && z == 0) at[4] |= dir_bits<Q>(2, 0);
+  if (p.face[5] && p.nz > 1 && z == p.nz - 1) at[5] |= dir_bits<Q>(2, 0);
+  const FaceDirs d = face_dirs(p, at);
   // all loads first (addresses chosen branch-free), adjustments after, so
   // the Q loads stay in flight together
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
-    const int t = i == 0 ? 0
-                         : face_combine<FW>(fcx[1 - Lattice<Q>::c(i, 0)], fcy[1 - Lattice<Q>::c(i, 1)],
-                                            fcz[1 - Lattice<Q>::c(i, 2)]);
     const int own = (Lattice<Q>::c(i, 0) == -1 && outlet) ? self - 1 : self;
-    const S* a = t ? src + (long long)opposite<Q>(i) * p.plane + own : base + src_index<Q>(nb, i);
+    const S* a = (d.own >> i & 1) ? src + (long long)opposite<Q>(i) * p.plane + own : base + src_index<Q>(nb, i);
     df[i] = Store<S>::ld(a);
     base += p.plane;
   }
+  if (d.lid | d.eq) {
 #pragma unroll
-  for (int i = 1; i < Q; ++i) {
-    const int t = face_combine<FW>(fcx[1 - Lattice<Q>::c(i, 0)], fcy[1 - Lattice<Q>::c(i, 1)],
-                                   fcz[1 - Lattice<Q>::c(i, 2)]);
-    if (t == EQ) df[i] = p.eq_df[i];
-    if (t == LID) df[i] += p.lid_term[i];
+    for (int i = 1; i < Q; ++i) {
+      if (d.eq >> i & 1) df[i] = p.eq_df[i];
+      if (d.lid >> i & 1) df[i] = __fadd_rn(df[i], p.lid_term[i]);
+    }
   }
   // where a WALL face meets an FWALL plane the cell is WALL and its slots are
   // never read, so reversing it as well is harmless
-  return FW && (fcx[1] == FWALL || fcy[1] == FWALL || fcz[1] == FWALL);
+  return FW && ((x == 0 && p.face[0] == FWALL) || (x == p.nx - 1 && p.face[1] == FWALL) ||
+                (y == 0 && p.face[2] == FWALL) || (y == p.ny - 1 && p.face[3] == FWALL) ||
+                (p.nz > 1 && ((z == 0 && p.face[4] == FWALL) || (z == p.nz - 1 && p.face[5] == FWALL))));
 }
 
 // Velocity boundaries at INLET cells, with inward normal n = sign e_axis

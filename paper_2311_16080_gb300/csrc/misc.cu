@@ -12,6 +12,10 @@ long long row_blocks(const StepParams& p) {
   return nxb * (long long)p.ny * p.nz;
 }
 
+long long cell_blocks(const StepParams& p) {
+  return p.mag_x ? ((long long)p.nx * p.ny * p.nz + 127) / 128 : row_blocks(p);
+}
+
 // Coordinates of a cell index; 32-bit divisions where the lattice allows.
 __device__ __forceinline__ void cell_xyz(long long cell, int nx, int ny, bool small, int& x, int& y, int& z) {
   if (small) {
@@ -306,6 +310,22 @@ __global__ void k_link_cells(const int2* __restrict__ links, long long n, const 
     const int b = wrap(x + cx, nx) + nx * (wrap(y + cy, ny) + ny * wrap(z + cz, nz));
     cells[e] = make_int2(w, (flags[b] & FLAG_TYPE) == FLUID ? b : -1);
   }
+}
+
+__global__ void k_links_off_x(const int2* __restrict__ cells, long long n, int nx, bool face0, bool face1, int* flag) {
+  bool off = false;
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
+    const int x = cells[e].x % nx;
+    off |= !((face0 && x == 0) || (face1 && x == nx - 1));
+  }
+  if (__syncthreads_or(off) && threadIdx.x == 0) atomicExch(flag, 1);
+}
+
+int launch_links_off_x(const int2* cells, long long n, int nx, bool face0, bool face1, int* flag, void* stream) {
+  const long long b = (n + 255) / 256;
+  k_links_off_x<<<(unsigned)(b < 152 * 8 ? b : 152 * 8), 256, 0, (cudaStream_t)stream>>>(cells, n, nx, face0, face1,
+                                                                                       flag);
+  return 0;
 }
 
 int launch_link_cells(int Q, const int2* links, long long n, const uint8_t* flags, int nx, int ny, int nz,

@@ -66,7 +66,15 @@ struct StepParams {
   // bulk kernels: 1 when launched on a (x-blocks, ny, nz) grid, 0 when the
   // grid is flattened over rows (ny or nz above the grid limit)
   int grid3;
+  // kernels mapped on cells: magic_of(nx), magic_of(ny) when they run on a
+  // grid flat over the cells (rows that do not fill their blocks), else 0
+  uint32_t mag_x, mag_y;
 };
+
+// Division of a cell or row index (below 2^31) by an extent n >= 2 as a
+// multiplication: the quotient's estimate is exact or one too large.  0 stands
+// for n = 1.
+inline uint32_t magic_of(int n) { return (uint32_t)(((1ULL << 32) + (unsigned)n - 1) / (unsigned)n); }
 
 // Ghost link entries are int2 {cell, dir | type << 8 | flags << 16}; LINK_BZ
 // marks a WALL link with a Bouzidi wall distance (in a parallel float array).
