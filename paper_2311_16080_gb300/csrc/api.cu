@@ -24,6 +24,7 @@
 #include "lattice.cuh"
 #include "launch.h"
 #include "resident2d.h"
+#include "tile2d.h"
 
 using namespace xlb;
 
@@ -95,10 +96,16 @@ struct xlb_ctx {
   // kernel variant of the bulk pass (XLB_KERNEL_*)
   int variant = 0;
   ResidentShape res = {-1, 0, 0, false};  // launch shape of the resident kernel (ctas < 0: not asked yet)
+  // the tiled D2Q9 kernel: its plan, and the cells with Bouzidi links (Tile2dArgs)
+  Tile2dPlan tile = {0, 0, 0, 0, -1, 0.f};  // halo < 0: not asked yet
+  int* bz = nullptr;
+  float* bz_q = nullptr;
+  int64_t n_bz = 0;  // cells with Bouzidi links
   // graph replay of the update (xlb_set_step_graph): g updates per graph, one
   // executable graph per starting buffer, each valid for one parameter epoch
   int64_t graph_g = 0;
   cudaGraphExec_t gexec[2] = {nullptr, nullptr};
+  int gto[2] = {0, 0};  // the buffer each leaves the state in
   uint64_t gexec_epoch[2] = {0, 0};
   uint64_t epoch = 1;  // bumped by every change of the update's parameters
   // profiling
@@ -664,6 +671,8 @@ void xlb_destroy(xlb_ctx* c) {
   if (c->inlet_field) cudaFree(c->inlet_field);
   if (c->fix) cudaFree(c->fix);
   if (c->init_fields) cudaFree(c->init_fields);
+  if (c->bz) cudaFree(c->bz);
+  if (c->bz_q) cudaFree(c->bz_q);
   if (c->fix_side) cudaFree(c->fix_side);
   if (c->aux) {
     cudaStreamSynchronize(c->aux);
@@ -1003,6 +1012,35 @@ int xlb_set_wall_distances(xlb_ctx* c, int64_t n, const int64_t* cell, const int
   if (r) return r;
   if (c->link_q) CK(cudaFree(c->link_q));
   c->link_q = nullptr;
+  if (c->bz) CK(cudaFree(c->bz));
+  if (c->bz_q) CK(cudaFree(c->bz_q));
+  c->bz = nullptr;
+  c->bz_q = nullptr;
+  c->n_bz = 0;
+  if (n > 0 && c->Q == 9) {
+    // the same by cell, for the tiled kernel
+    std::vector<uint8_t> fl((size_t)c->N);
+    CK(cudaMemcpy(fl.data(), c->flags, fl.size(), cudaMemcpyDeviceToHost));
+    std::vector<int> row((size_t)c->N, 0);
+    std::vector<float> rq;
+    for (int64_t k = 0; k < n; ++k) {
+      const int j = lattice_opposite(9, dir[k]);
+      int& r0 = row[(size_t)cell[k]];
+      if (!r0) {
+        rq.insert(rq.end(), 9, -1.0f);
+        r0 = (int)(rq.size() / 9);
+      }
+      const int64_t x = (cell[k] % c->nx + Lattice<9>::c(j, 0) + c->nx) % c->nx;
+      const int64_t y = (cell[k] / c->nx + Lattice<9>::c(j, 1) + c->ny) % c->ny;
+      const bool behind = (fl[(size_t)(x + c->nx * y)] & FLAG_TYPE) == XLB_CELL_FLUID;
+      rq[(size_t)(9 * (r0 - 1) + dir[k])] = q[k] < 0.5f && !behind ? 0.5f : q[k];
+    }
+    c->n_bz = (int64_t)rq.size() / 9;
+    CK(cudaMalloc(&c->bz, sizeof(int) * row.size()));
+    CK(cudaMalloc(&c->bz_q, sizeof(float) * rq.size()));
+    CK(cudaMemcpy(c->bz, row.data(), sizeof(int) * row.size(), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(c->bz_q, rq.data(), sizeof(float) * rq.size(), cudaMemcpyHostToDevice));
+  }
   if (n > 0) CK(cudaMalloc(&c->link_q, sizeof(float) * hq.size()));
   if (n > 0) CK(cudaMemcpy(c->link_q, hq.data(), sizeof(float) * hq.size(), cudaMemcpyHostToDevice));
   if (!hl.empty()) CK(cudaMemcpy(c->links, hl.data(), sizeof(int2) * hl.size(), cudaMemcpyHostToDevice));
@@ -1121,9 +1159,64 @@ static int record_checkpoint(xlb_ctx* c) {
   return XLB_OK;
 }
 
+// Whether the tiled D2Q9 kernel may take this ctx's updates: FLUID and WALL
+// cells, inflow and outflow planes together (the lattice then ends at them),
+// Bouzidi links.
+static bool tile_ok(xlb_ctx* c) {
+  if (c->Q != 9 || c->coll == XLB_COLL_NONE || c->has_lid_eq || c->n_fix > 0 || has_fwall_face(c)) return false;
+  if (c->x_inlet != c->x_outlet || (c->x_inlet && (c->inlet_axis != 0 || c->inlet_sign != 1))) return false;
+  if (c->link_q && !c->bz) return false;
+  if (c->tile.halo < 0) c->tile = tile2d_plan(c->storage, c->coll, (int)c->nx, (int)c->ny);
+  if (c->tile.halo < 2 || c->n_bz + 2 * (c->tile.by + 2 * c->tile.halo) > TILE_LIST) return false;
+  // one launch per update: 4.1 us, 1.6 us replayed from a graph, or the
+  // populations at 8 TB/s from L2; a boundary pass 3.6 us more
+  const double mem = 1.2 + 18.0 * c->esize * (double)c->N / 8e6;
+  double us = std::max(c->graph_g > 0 ? 1.6 : 4.1, mem);
+  if (c->n_links > 0) us += c->graph_g > 0 ? 3.6 : 5.0;
+  return c->tile.us < 0.9 * us;
+}
+
+// n updates of the post-collision state in buf[*cur], launched (or captured)
+// on the ctx stream; *cur becomes the buffer that holds the result.  The tiled
+// kernel needs no ghost values; those of the last state are written at the end.
+static int run_updates(xlb_ctx* c, int* cur, int64_t n) {
+  int r = XLB_OK;
+  if (n < 2 || c->prof || !tile_ok(c)) {
+    for (int64_t k = 0; k < n; ++k) {
+      r = launch_step(c, c->buf[*cur], c->buf[*cur ^ 1]);
+      if (r) return r;
+      *cur ^= 1;
+    }
+    return XLB_OK;
+  }
+  Tile2dArgs a;
+  memset(&a, 0, sizeof a);
+  a.p = make_params(c);
+  if (!c->has_mask) a.p.flags = nullptr;
+  a.storage = c->storage;
+  a.coll = c->coll;
+  a.bz = c->link_q ? c->bz : nullptr;
+  a.bz_q = c->bz_q;
+  a.plan = c->tile;
+  a.stream = c->stream;
+  for (int64_t left = n; left > 0;) {
+    const int64_t launches = (left + c->tile.halo - 1) / c->tile.halo;
+    a.steps = (int)((left + launches - 1) / launches);
+    a.src = c->buf[*cur];
+    a.dst = c->buf[*cur ^ 1];
+    const int e = launch_tile2d(a);
+    const cudaError_t ce = cudaGetLastError();
+    if (ce != cudaSuccess) return cuda_fail(c, ce, "tile kernel launch");
+    if (e) return fail(c, XLB_ERR_CUDA, "tile kernel launch rejected (code %d)", e);
+    *cur ^= 1;
+    left -= a.steps;
+  }
+  return boundary_pass(c, nullptr, c->buf[*cur]);
+}
+
 // Executable graph of graph_g updates starting from buffer `from`, captured
 // on the ctx stream with the current parameters (recaptured when the epoch
-// has moved on).  The graph holds exactly the launches launch_step makes.
+// has moved on).  The graph holds the launches run_updates makes.
 static int step_graph(xlb_ctx* c, int from, cudaGraphExec_t* out) {
   if (c->gexec[from] && c->gexec_epoch[from] == c->epoch) {
     *out = c->gexec[from];
@@ -1137,11 +1230,8 @@ static int step_graph(xlb_ctx* c, int from, cudaGraphExec_t* out) {
   CK(cudaStreamIsCapturing(c->stream, &cs));
   if (cs != cudaStreamCaptureStatusNone) return fail(c, XLB_ERR_STATE, "the ctx stream is already capturing");
   CK(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
-  int cur = from, r = XLB_OK;
-  for (int64_t k = 0; k < c->graph_g && r == XLB_OK; ++k) {
-    r = launch_step(c, c->buf[cur], c->buf[cur ^ 1]);
-    cur ^= 1;
-  }
+  int cur = from;
+  const int r = run_updates(c, &cur, c->graph_g);
   cudaGraph_t g = nullptr;
   const cudaError_t e = cudaStreamEndCapture(c->stream, &g);
   if (r != XLB_OK || e != cudaSuccess) {
@@ -1156,6 +1246,7 @@ static int step_graph(xlb_ctx* c, int from, cudaGraphExec_t* out) {
     return cuda_fail(c, ei, "cudaGraphInstantiate");
   }
   c->gexec_epoch[from] = c->epoch;
+  c->gto[from] = cur;
   *out = c->gexec[from];
   return XLB_OK;
 }
@@ -1196,6 +1287,7 @@ static int step_resident(xlb_ctx* c, int64_t room, int64_t* done) {
   const int64_t cells = (c->ny + c->res.ctas - 1) / c->res.ctas * c->nx;
   const bool graph = c->graph_g > 0 && !c->tape_open && room >= c->graph_g;
   if (!c->res.one && (graph || (cells > 4096 && c->n_links == 0))) return XLB_OK;
+  if (!c->res.one && tile_ok(c) && c->tile.us < 2.0 + cells / 2500.0) return XLB_OK;  // run_updates takes it
   ResidentArgs a;
   memset(&a, 0, sizeof a);
   a.src = c->buf[c->cur];
@@ -1251,20 +1343,24 @@ int xlb_step(xlb_ctx* c, int64_t n) {
       r = step_graph(c, c->cur, &ge);
       if (r) return r;
       CK(cudaGraphLaunch(ge, c->stream));
-      if (c->graph_g & 1) c->cur ^= 1;
+      c->cur = c->gto[c->cur];
       c->t += c->graph_g;
       k += c->graph_g - 1;
       continue;
     }
+    int64_t m = 1;
     if (!c->kind_h) {
       r = launch_collide_local(c, c->buf[c->cur]);
       c->kind_h = 1;
     } else {
-      r = launch_step(c, c->buf[c->cur], c->buf[c->cur ^ 1]);
-      c->cur ^= 1;
+      // up to the next checkpoint of an open tape
+      m = n - k;
+      if (c->tape_open) m = std::min(m, c->tape_k - c->t % c->tape_k);
+      r = run_updates(c, &c->cur, m);
     }
     if (r) return r;
-    c->t += 1;
+    c->t += m;
+    k += m - 1;
     r = record_checkpoint(c);
     if (r) return r;
   }

@@ -514,10 +514,11 @@ __device__ __forceinline__ void link_ghost(S* __restrict__ dst, const StepParams
     //   q <  1/2: 2q hi + (1 - 2q) h_opp(i)(x + c_i)  (hi if x + c_i is not FLUID)
     //   q >= 1/2: hi / (2q) + (1 - 1/(2q)) h_i(x)
     if (q < 0.5f) {
-      v = g.y >= 0 ? 2.0f * q * h + (1.0f - 2.0f * q) * hb : h;
+      const float q2 = 2.0f * q;
+      v = g.y >= 0 ? __fmaf_rn(q2, h, __fmul_rn(__fsub_rn(1.0f, q2), hb)) : h;
     } else {
       const float inv = 0.5f / q;
-      v = inv * h + (1.0f - inv) * hb;
+      v = __fmaf_rn(inv, h, __fmul_rn(__fsub_rn(1.0f, inv), hb));
     }
   }
   v = t == EQ ? eqv : (t == LID ? v + add : v);

@@ -3,27 +3,14 @@
 // between the first read and the last write nothing goes through L2 or HBM
 // and a step costs a cluster barrier instead of a launch.
 //
-// In place, one buffer (the swap of two directions per update that Bailey et
-// al. 2009 call the AA pattern).  Slot A[x][i] holds h_i(x) before an odd
-// update.  With L_j(x) = A[x][j] where x + c_j is a WALL cell and
-// A[x + c_j][opp(j)] elsewhere:
-//   odd update:  f_opp(j)(x) is in L_j(x) (streamed, or bounced back from the
-//                wall); after the collision h_j(x) goes to L_j(x);
-//   even update: f_i(x) is then in A[x][opp(i)] and h_i(x) goes to A[x][i].
-// Every slot is read and written by one thread per update, so one barrier
-// per update is enough, and the even ones touch nothing but the own cell.
-// The last update writes h straight to global memory.
-//
-// A cell is 9 consecutive slots: with FP32 a stride of 9 words, which reaches
-// every bank once per warp, and the direction is an immediate offset, so a
-// neighbour costs one addition whatever the domain's size.  16-bit slots
-// take a stride of 10 (5 words, again every bank once), the tenth being the
-// cell's meta word.
+// The slots and the in-place scheme: slots2d.cuh.  The last update writes h
+// straight to global memory.
 #include <cuda_runtime.h>
 
 #include "../../include/xlb.h"
 #include "lbm_device.cuh"
 #include "resident2d.h"
+#include "slots2d.cuh"
 
 namespace xlb {
 namespace {
@@ -33,12 +20,6 @@ constexpr int M_SOLID = 1 << 8;                       // the cell itself is a WA
 constexpr int M_XL = 1 << 9, M_XR = 1 << 10;          // x = 0 / x = nx - 1
 constexpr int M_YB = 1 << 11, M_YT = 1 << 12;         // first / last row of the block's part
 constexpr int M_WALLS = 0xff;
-
-template <typename S>
-struct Slots {
-  static constexpr int STRIDE = sizeof(S) == 4 ? 9 : 10;          // slots per cell
-  static constexpr int CELL = STRIDE * (int)sizeof(S);            // bytes per cell
-};
 
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
@@ -62,45 +43,6 @@ __device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
-}
-
-// slot access by 32-bit shared address; REMOTE: the address may lie in
-// another block of the cluster
-template <typename S, bool REMOTE>
-__device__ __forceinline__ float slot_ld(uint32_t a) {
-  if constexpr (sizeof(S) == 4) {
-    float v;
-    if (REMOTE)
-      asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
-    else
-      asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
-    return v;
-  } else {
-    unsigned short u;
-    if (REMOTE)
-      asm volatile("ld.shared::cluster.u16 %0, [%1];" : "=h"(u) : "r"(a) : "memory");
-    else
-      asm volatile("ld.shared.u16 %0, [%1];" : "=h"(u) : "r"(a) : "memory");
-    S s;
-    memcpy(&s, &u, 2);
-    return Store<S>::ld_plain(&s);
-  }
-}
-
-template <typename S, bool REMOTE>
-__device__ __forceinline__ void slot_st(uint32_t a, const CellRound<S>& rnd, int i, float v) {
-  if constexpr (sizeof(S) == 4) {
-    if (REMOTE)
-      asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
-    else
-      asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
-  } else {
-    const unsigned short u = rnd.bits(i, v);
-    if (REMOTE)
-      asm volatile("st.shared::cluster.u16 [%0], %1;" ::"r"(a), "h"(u) : "memory");
-    else
-      asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"(u) : "memory");
-  }
 }
 
 // Addresses L_j(x), j = 1..8, of one cell's odd update, from the addresses of

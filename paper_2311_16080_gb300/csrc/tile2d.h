@@ -1,0 +1,39 @@
+// Host interface of the tiled D2Q9 kernel (tile2d.cu): several updates per
+// launch on lattices too large for one cluster.
+#pragma once
+#include <stdint.h>
+
+#include "xlb_types.h"
+
+namespace xlb {
+
+// Tiles of bx x by cells (the last ones may be smaller), tx of them per row of
+// tiles, each with a ring of `halo` cells; halo updates per launch.
+// halo = 0: no plan.
+struct Tile2dPlan {
+  int bx, by, tx, ty, halo;
+  float us;  // the model's time per update
+};
+
+Tile2dPlan tile2d_plan(int storage, int coll, int nx, int ny);
+
+// Cells of one region with rules of their own (INLET, beside an OUTLET,
+// Bouzidi links) that a block has room for.
+constexpr int TILE_LIST = 1536;
+
+struct Tile2dArgs {
+  StepParams p;          // flags null: every cell FLUID
+  int storage, coll;
+  const void* src;       // post-collision populations
+  void* dst;             // the same `steps` updates later (another buffer)
+  const int* bz;         // per cell 0 or 1 + its row in bz_q, or null
+  const float* bz_q;     // 9 per row: wall distance of the link in each direction, or -1; 1/2 (halfway) for
+                         // a distance below 1/2 where the cell behind is not FLUID
+  Tile2dPlan plan;
+  int steps;             // 1 .. halo
+  void* stream;
+};
+
+int launch_tile2d(const Tile2dArgs& a);
+
+}  // namespace xlb

@@ -1,5 +1,6 @@
 """The resident D2Q9 kernel (a domain in the shared memory of one cluster, many
-updates in one launch) against the update-by-update kernels, bit for bit:
+updates in one launch) and the tiled one (larger lattices, several updates per
+launch) against the update-by-update kernels, bit for bit:
 profiling a context makes it launch every update by itself.  Sizes at the
 edges of its shapes: fewer rows than blocks, one and two cells per thread and
 more, rows that do not divide among the blocks, odd and even update counts,
@@ -84,3 +85,40 @@ def test_resident_segments_of_a_tape():
         g.append(out)
         s.close()
     assert np.array_equal(g[0], g[1])
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("nx,ny,collision,walls", [
+    (160, 150, "bgk", False), (301, 203, "bgk", True), (257, 499, "kbc", True), (1200, 40, "bgk", True)])
+def test_tiles_equal_update_by_update(nx, ny, collision, walls, storage):
+    c = _case(nx, ny, collision, walls)
+    a, b = c.gpu_sim(storage), c.gpu_sim(storage)
+    X.xlb_profile_enable(b.ctx, True)
+    fl = O.fluid_like(c.mask)
+    for n in (1, 2, 17):
+        a.step(n)
+        b.step(n)
+        assert np.array_equal(a.populations()[0][:, fl], b.populations()[0][:, fl]), n
+    if walls:
+        assert np.array_equal(a.wall_force(), b.wall_force())
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("graph", [0, 9])
+@pytest.mark.parametrize("n_d,inlet,bouzidi", [(10, "zou_he", True), (20, "regularized", True), (14, "zou_he", False)])
+def test_tiles_with_inflow_outflow_and_curved_walls(n_d, inlet, bouzidi, graph, storage):
+    from test_gpu_cylinder import Cyl
+    c = Cyl(n_d=n_d, u_mean=0.04, inlet=inlet, bouzidi=bouzidi)
+    a, b = c.gpu(storage), c.gpu(storage)
+    a.set_step_graph(graph)
+    X.xlb_profile_enable(b.ctx, True)
+    fl = O.fluid_like(c.mask)
+    for n in (2, 3, 40):
+        a.step(n)
+        b.step(n)
+        assert np.array_equal(a.populations()[0][:, fl], b.populations()[0][:, fl]), n
+        assert np.array_equal(a.wall_force(), b.wall_force())
+    a.close()
+    b.close()
