@@ -101,11 +101,11 @@ __device__ __forceinline__ int dst_index(const Nbr& nb, int i) {
 
 // hbar(x) = (S_bc^T abar)(x) for a fluid-like cell x.
 template <int Q>
-__device__ __forceinline__ void gather_adjoint(const float* __restrict__ ain, const StepParams& p, const Nbr& nb,
+__device__ __forceinline__ void gather_adjoint(const float* ain, const StepParams& p, const Nbr& nb,
                                                int self, int slow, float (&hb)[Q]) {
   if (!slow) {
 #pragma unroll
-    for (int i = 0; i < Q; ++i) hb[i] = __ldg(ain + (long long)i * p.plane + dst_index<Q>(nb, i));
+    for (int i = 0; i < Q; ++i) hb[i] = ain[(long long)i * p.plane + dst_index<Q>(nb, i)];
     return;
   }
 #pragma unroll
@@ -113,9 +113,9 @@ __device__ __forceinline__ void gather_adjoint(const float* __restrict__ ain, co
     const int d = dst_index<Q>(nb, i);
     const int t = p.flags[d] & FLAG_TYPE;
     if (fluid_like(t))
-      hb[i] = __ldg(ain + (long long)i * p.plane + d);
+      hb[i] = ain[(long long)i * p.plane + d];
     else if (t == WALL || t == LID)
-      hb[i] = __ldg(ain + (long long)opposite<Q>(i) * p.plane + self);
+      hb[i] = ain[(long long)opposite<Q>(i) * p.plane + self];
     else
       hb[i] = 0.f;
   }
@@ -147,11 +147,12 @@ __device__ __forceinline__ void init_state(const float* rho0, const float* u0, l
 }
 
 template <int Q, typename S, int COLL>
-__global__ void __launch_bounds__(ROW_BLOCK) k_adjoint_step(const S* __restrict__ hprev,
-                                                            const float* __restrict__ ain,
-                                                            float* __restrict__ aout, const StepParams p) {
+__global__ void __launch_bounds__(ROW_BLOCK) k_adjoint_step(const S* hprev, const float* ain, float* aout,
+                                                            const StepParams p) {
   CellIdx c;
   if (!cell_of_block(p, c)) return;
+  grid_wait();
+  grid_release();
   const int fl = p.has_mask ? p.flags[c.self] : 0;
   if (!fluid_like(fl & FLAG_TYPE)) {
     zero_out<Q, S>(aout, p, c.self);
@@ -298,13 +299,9 @@ int launch_adj_typed(AdjOp op, const AdjointArgs& a) {
       return 0;
     }
     case ADJ_STEP:
-      if (a.coll == COLL_NONE)
-        k_adjoint_step<Q, S, COLL_NONE><<<grid, block, 0, st>>>((const S*)a.state, a.abar_in, a.abar_out, p);
-      else if (a.coll == COLL_BGK)
-        k_adjoint_step<Q, S, COLL_BGK><<<grid, block, 0, st>>>((const S*)a.state, a.abar_in, a.abar_out, p);
-      else
-        return -2;
-      return 0;
+      if (a.coll != COLL_NONE && a.coll != COLL_BGK) return -2;
+      return launch_overlapped(a.coll == COLL_NONE ? k_adjoint_step<Q, S, COLL_NONE> : k_adjoint_step<Q, S, COLL_BGK>,
+                               grid, block, 0, st, (const S*)a.state, a.abar_in, a.abar_out, p) == cudaSuccess ? 0 : -3;
     case ADJ_STEP0:
       if (a.coll == COLL_NONE)
         k_adjoint_step0<Q, S, COLL_NONE><<<grid, block, 0, st>>>(a.fields_in, a.fields_in2, a.ucs, a.abar_in,

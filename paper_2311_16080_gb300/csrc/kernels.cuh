@@ -14,6 +14,7 @@
 
 #include "launch.h"
 #include "lbm_device.cuh"
+#include "overlap.cuh"
 
 namespace xlb {
 
@@ -199,7 +200,7 @@ __device__ __forceinline__ uint32_t x_rule_dirs(uint32_t fc) {
 // faces), the address chosen before the load so that a warp that meets an
 // x-face still issues one round of loads.
 template <int Q, typename S>
-__device__ __forceinline__ void pull_x_faces(const S* __restrict__ src, const StepParams& p, const Nbr& nb, int self,
+__device__ __forceinline__ void pull_x_faces(const S* src, const StepParams& p, const Nbr& nb, int self,
                                              uint32_t fc, uint32_t xr, float (&df)[Q]) {
   const S* base = src;
 #pragma unroll
@@ -225,7 +226,7 @@ __device__ __forceinline__ void pull_x_faces(const S* __restrict__ src, const St
 // (after a plain pull of the cell; lattices with an FWALL face): WALL: h_opp(i)(x);  LID: h_opp(i)(x) +
 // 2 w_i rho_w (c_i . u_w) / cs^2;  EQ: f_i^eq(rho_w, u_w).
 template <int Q, typename S, bool FW>
-__device__ __forceinline__ void x_face_rules(const S* __restrict__ src, const StepParams& p, int self, uint32_t fc,
+__device__ __forceinline__ void x_face_rules(const S* src, const StepParams& p, int self, uint32_t fc,
                                              float (&df)[Q]) {
   if (!(fc & FC_RN)) {
     // an ordinary row: the source's type is the x-face's alone, one per side
@@ -262,7 +263,7 @@ __device__ __forceinline__ void x_face_rules(const S* __restrict__ src, const St
 // df: the cell's post-collision values, rnd: how they are rounded into
 // storage.  (w, i) determines x, so no two cells write the same slot.
 template <int Q, typename S, bool FW>
-__device__ __forceinline__ void push_ghosts(S* __restrict__ dst, const StepParams& p, int x, int y, int z,
+__device__ __forceinline__ void push_ghosts(S* dst, const StepParams& p, int x, int y, int z,
                                             uint32_t fc, const float (&df)[Q], const CellRound<S>& rnd) {
   Nbr nb;
   make_nbr(nb, x, y, z, p.nx, p.ny, p.nz);
@@ -283,7 +284,7 @@ __device__ __forceinline__ void push_ghosts(S* __restrict__ dst, const StepParam
 // the planes with one pointer (a 64-bit add per plane; a product i * plane
 // per direction costs more instructions).
 template <int Q, typename S>
-__device__ __forceinline__ void pull_plain(const S* __restrict__ src, const StepParams& p, const Nbr& nb,
+__device__ __forceinline__ void pull_plain(const S* src, const StepParams& p, const Nbr& nb,
                                            float (&df)[Q]) {
   const S* base = src;
 #pragma unroll
@@ -294,7 +295,7 @@ __device__ __forceinline__ void pull_plain(const S* __restrict__ src, const Step
 }
 
 template <int Q, typename S>
-__device__ __forceinline__ void store_cell(S* __restrict__ dst, const StepParams& p, int self, const CellRound<S>& rnd,
+__device__ __forceinline__ void store_cell(S* dst, const StepParams& p, int self, const CellRound<S>& rnd,
                                            const float (&df)[Q]) {
   S* out = dst + self;
 #pragma unroll
@@ -330,9 +331,11 @@ struct GhostFaces {
 // k_boundary rewrites them; inlet / outlet cells are recomputed there too.
 template <int Q, typename S, int COLL, bool FW, bool IO, bool FLAT>
 __global__ void __launch_bounds__(ROW_BLOCK, MinBlocks<Q, S, COLL>::value)
-    k_stream_collide(const S* __restrict__ src, S* __restrict__ dst, const StepParams p) {
+    k_stream_collide(const S* src, S* dst, const StepParams p) {
   CellIdx c;
   if (!cell_of_grid<FLAT>(p, c)) return;
+  grid_wait();
+  grid_release();
   float df[Q];
   uint32_t fc = 0u;
   bool fwall = false;
@@ -398,7 +401,7 @@ __global__ void __launch_bounds__(ROW_BLOCK) k_face_ghosts(S* f, const StepParam
 //   EQ: f_i^eq(rho_w, u_w).
 // (w, i) determines x, so no two links write the same slot.
 template <int Q, typename S>
-__device__ __forceinline__ void write_ghost(S* __restrict__ dst, const StepParams& p, int x, int y, int z, int i,
+__device__ __forceinline__ void write_ghost(S* dst, const StepParams& p, int x, int y, int z, int i,
                                             int t, float h_opp) {
   int dx = 0, dy = 0, dz = 0;
   float add = 0.f, eqv = 0.f;
@@ -439,7 +442,7 @@ constexpr int LINKS_PER_THREAD = 4;
 
 // One fix-up cell kf of the boundary pass, by `mode` (see k_boundary).
 template <int Q, typename S, int COLL>
-__device__ __forceinline__ void fix_cell(const S* __restrict__ src, S* __restrict__ dst, const StepParams& p,
+__device__ __forceinline__ void fix_cell(const S* src, S* dst, const StepParams& p,
                                          const int* __restrict__ fix, int n_fix, int mode, S* __restrict__ side,
                                          int kf) {
   const int self = __ldg(fix + kf);
@@ -497,7 +500,7 @@ __device__ __forceinline__ void fix_cell(const S* __restrict__ src, S* __restric
 // the Bouzidi partner value; both are FLUID cells of dst, which the boundary
 // pass never writes.
 template <int Q, typename S>
-__device__ __forceinline__ void link_ghost(S* __restrict__ dst, const StepParams& p, int2 l, int2 g, float q,
+__device__ __forceinline__ void link_ghost(S* dst, const StepParams& p, int2 l, int2 g, float q,
                                            float h, float hb) {
   const int i = l.y & 0xff, t = (l.y >> 8) & 0xff;
   float add = 0.f, eqv = 0.f;
@@ -527,7 +530,7 @@ __device__ __forceinline__ void link_ghost(S* __restrict__ dst, const StepParams
 }
 
 template <int Q, typename S, int COLL>
-__global__ void __launch_bounds__(ROW_BLOCK) k_boundary(const S* __restrict__ src, S* __restrict__ dst,
+__global__ void __launch_bounds__(ROW_BLOCK) k_boundary(const S* src, S* dst,
                                                         const StepParams p, const int2* __restrict__ links,
                                                         const int2* __restrict__ link_cells,
                                                         const float* __restrict__ link_q, int n_links,
@@ -536,6 +539,8 @@ __global__ void __launch_bounds__(ROW_BLOCK) k_boundary(const S* __restrict__ sr
   // link threads: LINKS_PER_THREAD links each, strided by the link-thread
   // count so that a warp's loads and stores stay on consecutive entries; all
   // of a link's reads depend only on its table entries (two rounds of loads)
+  grid_wait();
+  grid_release();
   const int n_lt = (n_links + LINKS_PER_THREAD - 1) / LINKS_PER_THREAD;
   const int k = blockIdx.x * ROW_BLOCK + threadIdx.x;
   if (k < n_lt) {
@@ -605,7 +610,9 @@ struct VecMinBlocks {
 
 template <int Q, typename S, int COLL, int V>
 __global__ void __launch_bounds__(128, VecMinBlocks<Q, S, COLL, V>::value)
-    k_sc_vec(const S* __restrict__ src, S* __restrict__ dst, const StepParams p, uint32_t slot_mag, uint32_t row_mag) {
+    k_sc_vec(const S* src, S* dst, const StepParams p, uint32_t slot_mag, uint32_t row_mag) {
+  grid_wait();
+  grid_release();
   const int nx = p.nx, ny = p.ny, nz = p.nz;
   // slots of V cells run on over the rows; the lanes beyond the last one
   // repeat it and store nothing
@@ -1014,8 +1021,7 @@ int launch_typed(Op op, const LaunchArgs& a) {
                           : (fw ? k_stream_collide<Q, S, COLL, true, false, false>
                                 : io ? k_stream_collide<Q, S, COLL, false, true, false>
                                      : k_stream_collide<Q, S, COLL, false, false, false>);
-      kern<<<g3, block, 0, st>>>((const S*)a.src, (S*)a.dst, q);
-      return 0;
+      return launch_overlapped(kern, g3, block, 0, st, (const S*)a.src, (S*)a.dst, q) == cudaSuccess ? 0 : -3;
     }
     case OP_STEP_VEC: {
       // 16-bit storage, BGK, D2Q9 / D3Q19 only (FP32 is faster with one cell
@@ -1027,11 +1033,9 @@ int launch_typed(Op op, const LaunchArgs& a) {
         const int spr = p.nx / V;
         const long long blocks = ((long long)spr * p.ny * p.nz + 127) / 128;
         const uint32_t sm = magic_of(spr), rm = magic_of(p.ny);
-        if (V == 2)
-          k_sc_vec<Q, S, COLL, 2><<<(unsigned)blocks, 128, 0, st>>>((const S*)a.src, (S*)a.dst, p, sm, rm);
-        else
-          k_sc_vec<Q, S, COLL, 4><<<(unsigned)blocks, 128, 0, st>>>((const S*)a.src, (S*)a.dst, p, sm, rm);
-        return 0;
+        auto kern = V == 2 ? k_sc_vec<Q, S, COLL, 2> : k_sc_vec<Q, S, COLL, 4>;
+        return launch_overlapped(kern, dim3((unsigned)blocks), dim3(128), 0, st, (const S*)a.src, (S*)a.dst, p, sm,
+                                 rm) == cudaSuccess ? 0 : -3;
       }
       return -7;
     }
@@ -1046,10 +1050,9 @@ int launch_typed(Op op, const LaunchArgs& a) {
             (const S*)a.src, p, a.fix, (int)a.n_fix, (S*)a.side);
         return 0;
       }
-      k_boundary<Q, S, COLL><<<g, ROW_BLOCK, 0, st>>>((const S*)a.src, (S*)a.dst, p, a.links, a.link_cells,
-                                                     a.link_q, (int)a.n_links, a.fix, (int)a.n_fix, a.fix_mode,
-                                                     (S*)a.side);
-      return 0;
+      return launch_overlapped(k_boundary<Q, S, COLL>, dim3(g), block, 0, st, (const S*)a.src, (S*)a.dst, p, a.links,
+                               a.link_cells, a.link_q, (int)a.n_links, a.fix, (int)a.n_fix, a.fix_mode,
+                               (S*)a.side) == cudaSuccess ? 0 : -3;
     }
     case OP_COLLIDE_LOCAL:
       k_collide_local<Q, S, COLL><<<grid, block, 0, st>>>((S*)a.dst, p);

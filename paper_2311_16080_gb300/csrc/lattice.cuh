@@ -108,11 +108,13 @@ static_assert(opposite_holds<9>() && opposite_holds<19>() && opposite_holds<27>(
 template <typename S>
 struct Store;
 
+// ld: a plain load.  The read-only path (__ldg) is not for these kernels: they
+// start before the kernel that writes their input has ended (grid_wait).
 // ld_l2 / st_l2: coherent at L2 (bypass L1), for data written earlier in the
 // same kernel by other threads of the block.
 template <>
 struct Store<float> {
-  __device__ __forceinline__ static float ld(const float* p) { return __ldg(p); }
+  __device__ __forceinline__ static float ld(const float* p) { return *p; }
   __device__ __forceinline__ static float ld_l2(const float* p) { return __ldcg(p); }
   __device__ __forceinline__ static void st_l2(float* p, float v) { __stcg(p, v); }
   __device__ __forceinline__ static float ld_plain(const float* p) { return *p; }
@@ -122,7 +124,7 @@ struct Store<float> {
 
 template <>
 struct Store<__half> {
-  __device__ __forceinline__ static float ld(const __half* p) { return __half2float(__ldg(p)); }
+  __device__ __forceinline__ static float ld(const __half* p) { return __half2float(*p); }
   __device__ __forceinline__ static float ld_l2(const __half* p) { return __half2float(__ldcg(p)); }
   __device__ __forceinline__ static void st_l2(__half* p, float v) { __stcg(p, __float2half_rn(v)); }
   __device__ __forceinline__ static float ld_plain(const __half* p) { return __half2float(*p); }
@@ -133,7 +135,7 @@ struct Store<__half> {
 
 template <>
 struct Store<__nv_bfloat16> {
-  __device__ __forceinline__ static float ld(const __nv_bfloat16* p) { return __bfloat162float(__ldg(p)); }
+  __device__ __forceinline__ static float ld(const __nv_bfloat16* p) { return __bfloat162float(*p); }
   __device__ __forceinline__ static float ld_l2(const __nv_bfloat16* p) { return __bfloat162float(__ldcg(p)); }
   __device__ __forceinline__ static void st_l2(__nv_bfloat16* p, float v) { __stcg(p, __float2bfloat16_rn(v)); }
   __device__ __forceinline__ static float ld_plain(const __nv_bfloat16* p) { return __bfloat162float(*p); }
@@ -263,7 +265,7 @@ struct VecIO;
 template <>
 struct VecIO<float, 4> {
   __device__ __forceinline__ static void ld(const float* p, float (&v)[4]) {
-    const float4 w = __ldg(reinterpret_cast<const float4*>(p));
+    const float4 w = *reinterpret_cast<const float4*>(p);
     v[0] = w.x; v[1] = w.y; v[2] = w.z; v[3] = w.w;
   }
   __device__ __forceinline__ static void st(float* p, const float (&v)[4]) {
@@ -274,7 +276,7 @@ struct VecIO<float, 4> {
 template <>
 struct VecIO<float, 2> {
   __device__ __forceinline__ static void ld(const float* p, float (&v)[2]) {
-    const float2 w = __ldg(reinterpret_cast<const float2*>(p));
+    const float2 w = *reinterpret_cast<const float2*>(p);
     v[0] = w.x; v[1] = w.y;
   }
   __device__ __forceinline__ static void st(float* p, const float (&v)[2]) {
@@ -305,17 +307,17 @@ struct VecIO16 {
   using O = Half2Ops<H>;
   __device__ __forceinline__ static void ld_words(const H* p, uint32_t (&w)[W]) {
     if constexpr (W == 4) {
-      const uint4 q = __ldg(reinterpret_cast<const uint4*>(p));
+      const uint4 q = *reinterpret_cast<const uint4*>(p);
       w[0] = q.x;
       w[1] = q.y;
       w[2] = q.z;
       w[3] = q.w;
     } else if constexpr (W == 2) {
-      const uint2 q = __ldg(reinterpret_cast<const uint2*>(p));
+      const uint2 q = *reinterpret_cast<const uint2*>(p);
       w[0] = q.x;
       w[1] = q.y;
     } else {
-      w[0] = __ldg(reinterpret_cast<const unsigned int*>(p));
+      w[0] = *reinterpret_cast<const unsigned int*>(p);
     }
   }
   __device__ __forceinline__ static void st_words(H* p, const uint32_t (&w)[W]) {

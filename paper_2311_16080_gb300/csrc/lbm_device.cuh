@@ -183,7 +183,7 @@ __device__ __forceinline__ void reverse_populations(float (&df)[Q]) {
 // x - 1 in the directions c_x = -1, nb.xo[2] then being x itself) the face
 // rules of those directions take the populations of x - 1.
 template <int Q, typename S, bool FW = true>
-__device__ __forceinline__ bool pull_periodic(const S* __restrict__ src, const StepParams& p, const Nbr& nb,
+__device__ __forceinline__ bool pull_periodic(const S* src, const StepParams& p, const Nbr& nb,
                                               int self, int x, int y, int z, float (&df)[Q], bool outlet = false) {
   // per face, the directions whose source is on it: a source coordinate v - c
   // equal to the face's, c = +-1
@@ -374,7 +374,7 @@ __device__ __forceinline__ void inlet_rule(const StepParams& p, int self, float 
 // Zou-He and OUTLET cells copy their c_x = -1 populations from the pull at
 // x - 1 (zero-gradient outflow).
 template <int Q, typename S>
-__device__ __forceinline__ void pull_cell(const S* __restrict__ src, const StepParams& p, int x, int y, int z,
+__device__ __forceinline__ void pull_cell(const S* src, const StepParams& p, int x, int y, int z,
                                           int type, const Nbr& nb, float (&df)[Q]) {
   const int self = x + p.nx * (y + p.ny * z);
   pull_periodic<Q, S>(src, p, nb, self, x, y, z, df);

@@ -20,6 +20,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/xlb.h"
+#include "overlap.cuh"
 #include "slots2d.cuh"
 #include "tile2d.h"
 
@@ -139,7 +140,7 @@ __device__ __forceinline__ void special_push(const StepParams& p, const TileCtx&
 // instructions per cell and update); the load and store of the tile and the
 // launch, some 4.5 us, are shared by the updates of a launch.
 template <typename S, int COLL>
-__global__ void __launch_bounds__(TILE_THREADS, 1) k_tile2d(const S* __restrict__ A, S* __restrict__ B,
+__global__ void __launch_bounds__(TILE_THREADS, 1) k_tile2d(const S* A, S* B,
                                                             const StepParams p, const int* __restrict__ bz,
                                                             const float* __restrict__ bz_q, const Tile2dPlan plan,
                                                             int steps) {
@@ -167,6 +168,8 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile2d(const S* __restrict_
   __shared__ int n_list;
   if (threadIdx.x == 0) n_list = 0;
   __syncthreads();
+  grid_wait();
+  grid_release();
   auto lattice_cell = [&](int c) {
     const int ly = c / rw, lx = c - ly * rw;
     int gx = rx0 + lx, gy = ry0 + ly;
@@ -307,9 +310,9 @@ int launch_tile_typed(const Tile2dArgs& a) {
   const long long smem = tile_smem<S>(a.plan.bx, a.plan.by, a.plan.halo);
   if (smem > TILE_SMEM) return -1;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM) != cudaSuccess) return -3;
-  kern<<<(unsigned)(a.plan.tx * a.plan.ty), TILE_THREADS, (size_t)smem, (cudaStream_t)a.stream>>>(
-      (const S*)a.src, (S*)a.dst, a.p, a.bz, a.bz_q, a.plan, a.steps);
-  return 0;
+  return launch_overlapped(kern, dim3((unsigned)(a.plan.tx * a.plan.ty)), dim3(TILE_THREADS), (size_t)smem,
+                           (cudaStream_t)a.stream, (const S*)a.src, (S*)a.dst, a.p, a.bz, a.bz_q, a.plan,
+                           a.steps) == cudaSuccess ? 0 : -3;
 }
 
 template <typename S>
