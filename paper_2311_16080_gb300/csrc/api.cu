@@ -1022,20 +1022,31 @@ int xlb_set_wall_distances(xlb_ctx* c, int64_t n, const int64_t* cell, const int
     std::vector<uint8_t> fl((size_t)c->N);
     CK(cudaMemcpy(fl.data(), c->flags, fl.size(), cudaMemcpyDeviceToHost));
     std::vector<int> row((size_t)c->N, 0);
-    std::vector<float> rq;
+    std::vector<float> rq;  // Tile2dArgs::bz_q
+    std::vector<uint32_t> bits;
     for (int64_t k = 0; k < n; ++k) {
       const int j = lattice_opposite(9, dir[k]);
       int& r0 = row[(size_t)cell[k]];
       if (!r0) {
-        rq.insert(rq.end(), 9, -1.0f);
-        r0 = (int)(rq.size() / 9);
+        rq.insert(rq.end(), 18, 0.0f);
+        bits.insert(bits.end(), 2, 0u);
+        r0 = (int)(rq.size() / 18);
       }
       const int64_t x = (cell[k] % c->nx + Lattice<9>::c(j, 0) + c->nx) % c->nx;
       const int64_t y = (cell[k] / c->nx + Lattice<9>::c(j, 1) + c->ny) % c->ny;
       const bool behind = (fl[(size_t)(x + c->nx * y)] & FLAG_TYPE) == XLB_CELL_FLUID;
-      rq[(size_t)(9 * (r0 - 1) + dir[k])] = q[k] < 0.5f && !behind ? 0.5f : q[k];
+      const float qk = q[k] < 0.5f && !behind ? 0.5f : q[k];
+      const float w = qk < 0.5f ? 2.0f * qk : 0.5f / qk;
+      float* pair = rq.data() + 18 * (size_t)(r0 - 1) + 2 * dir[k];
+      pair[0] = w;
+      pair[1] = 1.0f - w;
+      uint32_t* b = bits.data() + 2 * (size_t)(r0 - 1);
+      b[0] &= ~(1u << dir[k]);
+      b[1] &= ~(1u << dir[k]);
+      b[qk < 0.5f ? 0 : 1] |= 1u << dir[k];
     }
-    c->n_bz = (int64_t)rq.size() / 9;
+    for (size_t r0 = 0; r0 < bits.size() / 2; ++r0) memcpy(rq.data() + 18 * r0, bits.data() + 2 * r0, 8);
+    c->n_bz = (int64_t)rq.size() / 18;
     CK(cudaMalloc(&c->bz, sizeof(int) * row.size()));
     CK(cudaMalloc(&c->bz_q, sizeof(float) * rq.size()));
     CK(cudaMemcpy(c->bz, row.data(), sizeof(int) * row.size(), cudaMemcpyHostToDevice));
@@ -1159,6 +1170,15 @@ static int record_checkpoint(xlb_ctx* c) {
   return XLB_OK;
 }
 
+// Time of one D2Q9 update launched by itself, as measured on lattices of 128^2
+// to 601 x 599 cells: 2.1 us, 1.55 us replayed from a graph, or the cells' time;
+// a boundary pass 2.4 us more, 3.3 us in 16-bit storage.
+static double single_update_us(const xlb_ctx* c) {
+  const double rate = c->coll == XLB_COLL_KBC ? 69e3 : c->storage == XLB_STORE_BF16 ? 60e3 : 108e3;  // cells per us
+  const double us = std::max(c->graph_g > 0 ? 1.55 : 2.1, 1.1 + (double)c->N / rate);
+  return us + (c->n_links > 0 ? (c->esize == 2 ? 3.3 : 2.4) : 0.0);
+}
+
 // Whether the tiled D2Q9 kernel may take this ctx's updates: FLUID and WALL
 // cells, inflow and outflow planes together (the lattice then ends at them),
 // Bouzidi links.
@@ -1168,12 +1188,7 @@ static bool tile_ok(xlb_ctx* c) {
   if (c->link_q && !c->bz) return false;
   if (c->tile.halo < 0) c->tile = tile2d_plan(c->storage, c->coll, (int)c->nx, (int)c->ny);
   if (c->tile.halo < 2 || c->n_bz + 2 * (c->tile.by + 2 * c->tile.halo) > TILE_LIST) return false;
-  // one launch per update: 4.1 us, 1.6 us replayed from a graph, or the
-  // populations at 8 TB/s from L2; a boundary pass 3.6 us more
-  const double mem = 1.2 + 18.0 * c->esize * (double)c->N / 8e6;
-  double us = std::max(c->graph_g > 0 ? 1.6 : 4.1, mem);
-  if (c->n_links > 0) us += c->graph_g > 0 ? 3.6 : 5.0;
-  return c->tile.us < 0.9 * us;
+  return c->tile.us < 0.95 * single_update_us(c);
 }
 
 // n updates of the post-collision state in buf[*cur], launched (or captured)
@@ -1280,14 +1295,13 @@ static int step_resident(xlb_ctx* c, int64_t room, int64_t* done) {
     return XLB_OK;
   if (c->res.ctas < 0) c->res = resident2d_shape(c->storage, c->coll, (int)c->nx, (int)c->ny, true);
   if (c->res.ctas == 0) return XLB_OK;
-  // An update costs 0.7 to 1.6 us here while a thread holds at most two
-  // cells (128^2 on 16 blocks), 3.7 us at 4096 cells a block, 5.7 us at the
-  // most; launched one by one 4.1 us, 10 us with a boundary pass, and 1.6 to
-  // 3 us replayed from a graph.
-  const int64_t cells = (c->ny + c->res.ctas - 1) / c->res.ctas * c->nx;
-  const bool graph = c->graph_g > 0 && !c->tape_open && room >= c->graph_g;
-  if (!c->res.one && (graph || (cells > 4096 && c->n_links == 0))) return XLB_OK;
-  if (!c->res.one && tile_ok(c) && c->tile.us < 2.0 + cells / 2500.0) return XLB_OK;  // run_updates takes it
+  // While a thread holds at most two cells an update costs 0.75 us and 0.85 us
+  // more for each 1024 cells a block (128^2 on 16 blocks: 1.6 us; KBC twice
+  // that); with more the tiles are faster (256 x 128: 3.5 us against 2.0).
+  if (!c->res.one) return XLB_OK;
+  const double cells = (double)((c->ny + c->res.ctas - 1) / c->res.ctas * c->nx);
+  const double us = 0.75 + 0.85 * cells / 1024.0 * (c->coll == XLB_COLL_KBC ? 2.0 : 1.0);
+  if (us > single_update_us(c) || (tile_ok(c) && us > c->tile.us)) return XLB_OK;
   ResidentArgs a;
   memset(&a, 0, sizeof a);
   a.src = c->buf[c->cur];

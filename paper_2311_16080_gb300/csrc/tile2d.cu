@@ -19,6 +19,8 @@
 //   stash, and the outlet column is updated after a barrier of its own.
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "../../include/xlb.h"
 #include "overlap.cuh"
 #include "slots2d.cuh"
@@ -28,7 +30,7 @@ namespace xlb {
 namespace {
 
 constexpr int TILE_THREADS = 768;
-constexpr long long TILE_SMEM = 222 * 1024;  // dynamic; the list is static
+constexpr long long TILE_SMEM = 220 * 1024;  // dynamic; the list is static
 
 // meta word of a cell: bits 0-7: x + c_j is a WALL cell or outside the region
 // (j = 1..8)
@@ -39,7 +41,7 @@ constexpr int M_INNER = 1 << 13;   // of the tile, not of the ring
 constexpr int M_WALLS = 0xff;
 // cells with rules of their own: not in the main loop, where a few lanes would
 // hold up every warp they sit in (the 1761 x 330 cylinder: 13 us an update),
-// but packed in a list that whole warps work off
+// but packed in a list that a few warps work off beside it
 constexpr int M_LISTED = M_INLET | M_BEFORE | M_BZ;
 
 // A value as a ghost slot (k of the lattice) would store it.
@@ -53,7 +55,6 @@ __device__ __forceinline__ float ghost_round(uint32_t slot, float v) {
 struct TileCtx {
   uint32_t base;       // slots
   int rw;              // region's row length
-  const float* bz_q;
 };
 
 template <typename S>
@@ -72,25 +73,22 @@ __device__ __forceinline__ void tile_slots(const TileCtx& t, int c, int m, uint3
 }
 
 // Rules of one cell that is INLET, OUTLET, beside an OUTLET or has Bouzidi
-// links, on its pulled populations; `self` its cell in the lattice.
+// links (rows of the table at q), on its pulled populations; `self` its cell in
+// the lattice.
 template <typename S>
-__device__ __forceinline__ void special_pull(const StepParams& p, const TileCtx& t, int m, int row, int self,
-                                             const int* __restrict__ bz, float* stash, float (&f)[9]) {
+__device__ __forceinline__ void special_pull(const StepParams& p, int m, int row, int self,
+                                             const float2* __restrict__ q, float* stash, float (&f)[9]) {
   if (m & M_BZ) {
-    const float* q = t.bz_q + 9 * (__ldg(bz + self) - 1);
+    const uint32_t low = __float_as_uint(__ldg(q).x);  // links with q < 1/2
     float g[9];
-#pragma unroll
-    for (int i = 0; i < 9; ++i) g[i] = f[i];
+    g[0] = f[0];
 #pragma unroll
     for (int i = 1; i < 9; ++i) {
       const int j = opposite<9>(i);
-      const float qi = __ldg(q + i);
-      if (qi >= 0.f && qi < 0.5f) {  // (the table holds 1/2 where x + c_j is not FLUID)
-        const float q2 = 2.0f * qi;
-        const float v = __fmaf_rn(q2, f[j], __fmul_rn(__fsub_rn(1.0f, q2), f[i]));
-        const int w = self + Lattice<9>::c(i, 0) + p.nx * Lattice<9>::c(i, 1);
-        g[j] = ghost_round<S>((uint32_t)((long long)j * p.plane + w), v);
-      }
+      const float2 w = __ldg(q + i);
+      const int wall = self + Lattice<9>::c(i, 0) + p.nx * Lattice<9>::c(i, 1);
+      const float v = ghost_round<S>((uint32_t)((long long)j * p.plane + wall), __fmaf_rn(w.x, f[j], __fmul_rn(w.y, f[i])));
+      g[j] = (low >> i & 1) ? v : f[j];
     }
 #pragma unroll
     for (int i = 0; i < 9; ++i) f[i] = g[i];
@@ -108,23 +106,21 @@ __device__ __forceinline__ void special_pull(const StepParams& p, const TileCtx&
   if (m & M_INLET) inlet_rule<9>(p, self, f);
 }
 
-// What a cell with Bouzidi links leaves in its slots: q >= 1/2 links take the
-// mixed value in place of h_i.
+// What a cell with Bouzidi links leaves in its slots (at a): links with
+// q >= 1/2 take the mixed value in place of h_i.
 template <typename S>
-__device__ __forceinline__ void special_push(const StepParams& p, const TileCtx& t, int self,
-                                             const int* __restrict__ bz, uint32_t a, float (&h)[9]) {
+__device__ __forceinline__ void special_push(const StepParams& p, int self, const float2* __restrict__ q, uint32_t a,
+                                             float (&h)[9]) {
   constexpr int SB = (int)sizeof(S);
-  const float* q = t.bz_q + 9 * (__ldg(bz + self) - 1);
+  const uint32_t high = __float_as_uint(__ldg(q).y);  // links with q >= 1/2
 #pragma unroll
   for (int i = 1; i < 9; ++i) {
     const int j = opposite<9>(i);
-    const float qi = __ldg(q + i);
-    if (qi >= 0.5f) {
-      const float inv = 0.5f / qi;
-      const float v = __fmaf_rn(inv, h[i], __fmul_rn(__fsub_rn(1.0f, inv), h[j]));
-      const int w = self + Lattice<9>::c(i, 0) + p.nx * Lattice<9>::c(i, 1);
-      S s;
-      st_ghost<S>(&s, (uint32_t)((long long)j * p.plane + w), v);
+    const float2 w = __ldg(q + i);
+    const int wall = self + Lattice<9>::c(i, 0) + p.nx * Lattice<9>::c(i, 1);
+    S s;
+    st_ghost<S>(&s, (uint32_t)((long long)j * p.plane + wall), __fmaf_rn(w.x, h[i], __fmul_rn(w.y, h[j])));
+    if (high >> i & 1) {
       if constexpr (sizeof(S) == 4) {
         asm volatile("st.shared.f32 [%0], %1;" ::"r"(a + i * SB), "f"(s) : "memory");
       } else {
@@ -142,7 +138,7 @@ __device__ __forceinline__ void special_push(const StepParams& p, const TileCtx&
 template <typename S, int COLL>
 __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile2d(const S* A, S* B,
                                                             const StepParams p, const int* __restrict__ bz,
-                                                            const float* __restrict__ bz_q, const Tile2dPlan plan,
+                                                            const float2* __restrict__ bz_q, const Tile2dPlan plan,
                                                             int steps) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int CB = Slots<S>::CELL, SB = (int)sizeof(S);
@@ -160,11 +156,10 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile2d(const S* A, S* B,
   TileCtx t;
   t.base = (uint32_t)__cvta_generic_to_shared(smem);
   t.rw = rw;
-  t.bz_q = bz_q;
   unsigned short* meta = reinterpret_cast<unsigned short*>(smem + (sizeof(S) == 4 ? (size_t)cap * CB : 9 * SB));
   float* stash = reinterpret_cast<float*>(
       smem + ((size_t)cap * (sizeof(S) == 4 ? CB + 2 : CB) + 15) / 16 * 16);
-  __shared__ unsigned short list[TILE_LIST];
+  __shared__ uint32_t list[TILE_LIST];  // cell | row of bz_q << 16
   __shared__ int n_list;
   if (threadIdx.x == 0) n_list = 0;
   __syncthreads();
@@ -177,43 +172,105 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile2d(const S* A, S* B,
     gy = gy < 0 ? gy + ny : (gy >= ny ? gy - ny : gy);
     return gx + nx * gy;
   };
-  for (int c = threadIdx.x; c < cells; c += TILE_THREADS) {
-    const int ly = c / rw, lx = c - ly * rw;
-    const int self = lattice_cell(c), gy = self / nx, gx = self - gy * nx;
-    int m = 0;
-    const int f = p.flags ? p.flags[self] : 0, type = f & FLAG_TYPE;
-    if (lx >= ix0 - rx0 && lx < ix1 - rx0 && ly >= h && ly < iy1 - ry0) m |= M_INNER;
-    if (type == WALL) m |= M_SOLID;
-    if (type == INLET) m |= M_INLET;
-    if (type == OUTLET) m |= M_OUTLET;
-    if (p.x_outlet && gx == nx - 2 && (p.flags[self + 1] & FLAG_TYPE) == OUTLET) m |= M_BEFORE;
-    if (bz && bz[self]) m |= M_BZ;
-    const int xs[3] = {gx == 0 ? nx - 1 : gx - 1, gx, gx == nx - 1 ? 0 : gx + 1};
-    const int ys[3] = {gy == 0 ? ny - 1 : gy - 1, gy, gy == ny - 1 ? 0 : gy + 1};
+  // the populations, with every round's loads in flight
+  const int dly = TILE_THREADS / rw, dlx = TILE_THREADS - dly * rw;  // a round further
+  auto wrapped = [&](int lx, int ly) {
+    int gx = rx0 + lx, gy = ry0 + ly;
+    gx = gx < 0 ? gx + nx : (gx >= nx ? gx - nx : gx);
+    gy = gy < 0 ? gy + ny : (gy >= ny ? gy - ny : gy);
+    return gx + nx * gy;
+  };
+  {
+    int ly = (int)threadIdx.x / rw, lx = (int)threadIdx.x - ly * rw;
+    auto next = [&]() {
+      lx += dlx;
+      ly += dly;
+      if (lx >= rw) {
+        lx -= rw;
+        ++ly;
+      }
+    };
+    if constexpr (sizeof(S) == 4) {
+      for (int c = threadIdx.x; c < cells; c += TILE_THREADS, next()) {
+        const S* g = A + wrapped(lx, ly);
+        const uint32_t a = t.base + (uint32_t)c * CB;
 #pragma unroll
-    for (int j = 1; j < 9; ++j) {
-      const int cx = Lattice<9>::c(j, 0), cy = Lattice<9>::c(j, 1);
-      bool bounce = lx + cx < 0 || lx + cx >= rw || ly + cy < 0 || ly + cy >= rh;
-      if (!bounce && (f & FLAG_SLOW)) bounce = (p.flags[xs[1 + cx] + nx * ys[1 + cy]] & FLAG_TYPE) == WALL;
-      if (bounce) m |= 1 << (j - 1);
-    }
-    meta[c * MS] = (unsigned short)m;
-    float v[9];
-    S* cell = reinterpret_cast<S*>(smem + (size_t)c * CB);
+        for (int i = 0; i < 9; ++i)
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(a + i * SB), "l"(g + (long long)i * p.plane)
+                       : "memory");
+      }
+      asm volatile("cp.async.wait_all;" ::: "memory");
+    } else {
+      for (int c = threadIdx.x; c < cells; c += 3 * TILE_THREADS) {
+        S v[3][9];
 #pragma unroll
-    for (int i = 0; i < 9; ++i) {
-      const S s = A[(long long)i * p.plane + self];
-      cell[i] = s;
-      v[i] = Store<S>::ld_plain(&s);
-    }
-    if (m & M_BZ) special_push<S>(p, t, self, bz, t.base + (uint32_t)c * CB, v);
-    if ((m & M_LISTED) && !(m & M_SOLID)) {
-      const int k = atomicAdd(&n_list, 1);
-      if (k < TILE_LIST) list[k] = (unsigned short)c;  // (the host takes no lattice with more)
+        for (int k = 0; k < 3; ++k, next()) {
+          if (c + k * TILE_THREADS >= cells) continue;
+          const S* g = A + wrapped(lx, ly);
+#pragma unroll
+          for (int i = 0; i < 9; ++i) v[k][i] = g[(long long)i * p.plane];
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          if (c + k * TILE_THREADS >= cells) continue;
+          S* cell = reinterpret_cast<S*>(smem + (size_t)(c + k * TILE_THREADS) * CB);
+#pragma unroll
+          for (int i = 0; i < 9; ++i) cell[i] = v[k][i];
+        }
+      }
     }
   }
-  const bool outlet = p.x_outlet && rx1 == nx;
+  // the meta words; a thread handles the cells it loaded
+  {
+    int ly = (int)threadIdx.x / rw, lx = (int)threadIdx.x - ly * rw;
+    for (int c = threadIdx.x; c < cells; c += TILE_THREADS) {
+      int m = 0, row = 0;
+      if (lx >= ix0 - rx0 && lx < ix1 - rx0 && ly >= h && ly < iy1 - ry0) m |= M_INNER;
+#pragma unroll
+      for (int j = 1; j < 9; ++j) {
+        const int x = lx + Lattice<9>::c(j, 0), y = ly + Lattice<9>::c(j, 1);
+        if (x < 0 || x >= rw || y < 0 || y >= rh) m |= 1 << (j - 1);
+      }
+      if (p.flags) {
+        const int self = wrapped(lx, ly);
+        const int f = p.flags[self], type = f & FLAG_TYPE;
+        if (type == WALL) m |= M_SOLID;
+        if (type == INLET) m |= M_INLET;
+        if (type == OUTLET) m |= M_OUTLET;
+        if (f & FLAG_SLOW) {
+          const int gy = self / nx, gx = self - gy * nx;
+          const int xs[3] = {gx == 0 ? nx - 1 : gx - 1, gx, gx == nx - 1 ? 0 : gx + 1};
+          const int ys[3] = {gy == 0 ? ny - 1 : gy - 1, gy, gy == ny - 1 ? 0 : gy + 1};
+#pragma unroll
+          for (int j = 1; j < 9; ++j)
+            if ((p.flags[xs[1 + Lattice<9>::c(j, 0)] + nx * ys[1 + Lattice<9>::c(j, 1)]] & FLAG_TYPE) == WALL)
+              m |= 1 << (j - 1);
+        }
+        if (p.x_outlet && lx == rw - 2 && rx1 == nx && (p.flags[self + 1] & FLAG_TYPE) == OUTLET) m |= M_BEFORE;
+        if (bz && (row = bz[self])) {
+          m |= M_BZ;
+          float v[9];
+          const S* cell = reinterpret_cast<const S*>(smem + (size_t)c * CB);
+#pragma unroll
+          for (int i = 0; i < 9; ++i) v[i] = Store<S>::ld_plain(cell + i);
+          special_push<S>(p, self, bz_q + 9 * (row - 1), t.base + (uint32_t)c * CB, v);
+        }
+      }
+      meta[c * MS] = (unsigned short)m;
+      if ((m & M_LISTED) && !(m & M_SOLID)) {
+        const int k = atomicAdd(&n_list, 1);
+        if (k < TILE_LIST) list[k] = (uint32_t)c | (uint32_t)row << 16;  // (the host takes no lattice with more)
+      }
+      lx += dlx;
+      ly += dly;
+      if (lx >= rw) {
+        lx -= rw;
+        ++ly;
+      }
+    }
+  }
   __syncthreads();
+  const bool outlet = p.x_outlet && rx1 == nx;
   const int listed = min(n_list, TILE_LIST);
   // the slots of cell c's update
   auto slots = [&](int c, int m, bool odd, uint32_t (&L)[9]) {
@@ -235,14 +292,15 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile2d(const S* A, S* B,
     }
   };
   // one update of a cell with rules of its own
-  auto special = [&](int c, bool odd, bool last) {
+  auto special = [&](int c, int row, bool odd, bool last) {
     const int m = meta[c * MS], self = lattice_cell(c);
     uint32_t L[9];
     slots(c, m, odd, L);
     float f[9];
 #pragma unroll
     for (int j = 0; j < 9; ++j) f[opposite<9>(j)] = slot_ld<S, false>(L[j]);
-    special_pull<S>(p, t, m, c / rw, self, bz, stash, f);
+    const float2* q = bz_q + 9 * (row - 1);
+    special_pull<S>(p, m, c / rw, self, q, stash, f);
     collide<9, COLL>(f, p);
     CellRound<S> r;
     r.begin((uint32_t)self, f);
@@ -250,16 +308,36 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile2d(const S* A, S* B,
     if ((m & M_BZ) && !last) {
 #pragma unroll
       for (int i = 0; i < 9; ++i) f[i] = r.rounded(i, f[i]);
-      special_push<S>(p, t, self, bz, t.base + (uint32_t)c * CB, f);
+      special_push<S>(p, self, q, t.base + (uint32_t)c * CB, f);
     }
   };
+  // The listed cells and the outlet column belong to the last warps, which take
+  // no part in the main loop: one such cell costs a warp some 2 us of latency.
+  int own = (listed + 31) / 32;
+  if (outlet && own < 1) own = 1;
+  if (own > 8) own = 8;
+  const int n_main = TILE_THREADS - 32 * own;
   for (int k = 0; k < steps; ++k) {
     const bool odd = !(k & 1), last = k == steps - 1;
-    // the list, from the last warps on: the main loop's last round leaves them idle
-    for (int s = TILE_THREADS - 1 - (int)threadIdx.x; s < listed; s += TILE_THREADS) special(list[s], odd, last);
-    for (int c0 = threadIdx.x; c0 < cells; c0 += 2 * TILE_THREADS) {
-      const int c1 = c0 + TILE_THREADS;
-      int m0 = meta[c0 * MS], m1 = c1 < cells ? meta[c1 * MS] : M_SOLID;
+    // the rows whose neighbours are still right
+    const int c_lo = (k + 1) * rw, c_hi = cells - (k + 1) * rw;
+    if ((int)threadIdx.x >= n_main) {
+      // the listed cells, then the outlet column, once the stash is whole
+      for (int s = (int)threadIdx.x - n_main; s < listed; s += TILE_THREADS - n_main) {
+        const int c = (int)(list[s] & 0xffffu);
+        if (c >= c_lo && c < c_hi) special(c, (int)(list[s] >> 16), odd, last);
+      }
+      if (outlet) {
+        asm volatile("bar.sync 1, %0;" ::"r"(TILE_THREADS - n_main) : "memory");
+        for (int r = k + 1 + (int)threadIdx.x - n_main; r < rh - (k + 1); r += TILE_THREADS - n_main) {
+          const int c = r * rw + rw - 1;
+          if ((meta[c * MS] & (M_OUTLET | M_SOLID)) == M_OUTLET) special(c, 0, odd, last);
+        }
+      }
+    } else
+    for (int c0 = c_lo + threadIdx.x; c0 < c_hi; c0 += 2 * n_main) {
+      const int c1 = c0 + n_main;
+      int m0 = meta[c0 * MS], m1 = c1 < c_hi ? meta[c1 * MS] : M_SOLID;
       if (m0 & (M_LISTED | M_OUTLET)) m0 |= M_SOLID;  // not here
       if (m1 & (M_LISTED | M_OUTLET)) m1 |= M_SOLID;
       if (m0 & m1 & M_SOLID) continue;
@@ -276,7 +354,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile2d(const S* A, S* B,
 #pragma unroll
       for (int i = 0; i < 9; ++i) unpack2(f[i], a[i], b[i]);
       int s0 = 0, s1 = 0;
-      if (sizeof(S) == 2 || last) {
+      if (std::is_same<S, __nv_bfloat16>::value || last) {  // (the rounding key, the cell to store)
         s0 = lattice_cell(e0);
         s1 = lattice_cell(e1);
       }
@@ -287,14 +365,6 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile2d(const S* A, S* B,
       store(L1, m1, s1, r1, b, last);
     }
     __syncthreads();
-    if (outlet) {
-      // the outlet column, once the stash is whole
-      for (int r = threadIdx.x; r < rh; r += TILE_THREADS) {
-        const int c = r * rw + rw - 1;
-        if ((meta[c * MS] & (M_OUTLET | M_SOLID)) == M_OUTLET) special(c, odd, last);
-      }
-      __syncthreads();
-    }
   }
 }
 
@@ -311,7 +381,7 @@ int launch_tile_typed(const Tile2dArgs& a) {
   if (smem > TILE_SMEM) return -1;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM) != cudaSuccess) return -3;
   return launch_overlapped(kern, dim3((unsigned)(a.plan.tx * a.plan.ty)), dim3(TILE_THREADS), (size_t)smem,
-                           (cudaStream_t)a.stream, (const S*)a.src, (S*)a.dst, a.p, a.bz, a.bz_q, a.plan,
+                           (cudaStream_t)a.stream, (const S*)a.src, (S*)a.dst, a.p, a.bz, (const float2*)a.bz_q, a.plan,
                            a.steps) == cudaSuccess ? 0 : -3;
 }
 
@@ -325,12 +395,13 @@ int tile_by_coll(const Tile2dArgs& a) {
 }  // namespace
 
 // Tiles that a model of the kernel expects to take the least time per update:
-// waves of blocks over the SMs, 4.5 us a launch for load and store, and a
-// region's update at 1350 cells per us and SM (KBC 500).  Measured (FP32 BGK
-// with walls) 300 x 200: 2.5 us, launched one by one 8.2, graph 4.7; 601 x 599:
-// 5.7, 10.7 and 7.3; the 1761 x 330 cylinder 8.8, graph 12.6.
+// waves of blocks over the SMs, 5 us a launch for load and store, and per update
+// 0.8 us and a time for each round of two cells per thread.  Measured per update
+// (FP32 BGK with walls) 300 x 200: 2.3 us, launched one by one 4.9, graph 4.1;
+// 601 x 599: 4.7, 7.6 and 7.0; the 1761 x 330 cylinder 7.5, graph 11.5.
 Tile2dPlan tile2d_plan(int storage, int coll, int nx, int ny) {
   Tile2dPlan best = {0, 0, 0, 0, 0, 0.f};
+  const float over = 5.0f, per = coll == COLL_KBC ? 2.9f : storage == XLB_STORE_BF16 ? 1.8f : 0.85f;
   for (int tx = 1; tx <= nx && tx <= 152; ++tx) {
     const int bx = (nx + tx - 1) / tx;
     if ((nx + bx - 1) / bx != tx) continue;
@@ -343,7 +414,10 @@ Tile2dPlan tile2d_plan(int storage, int coll, int nx, int ny) {
         const long long smem = storage == XLB_STORE_F32 ? tile_smem<float>(bx, by, h) : tile_smem<__half>(bx, by, h);
         if (smem > TILE_SMEM) break;
         const int waves = (tx * ty + 151) / 152;
-        const float us = waves * (4.5f + h * (0.4f + cells / (coll == COLL_KBC ? 500.0f : 1350.0f))) / h;
+        // (a row of the ring less per update on either side)
+        const long long busy = (long long)(bx + 2 * h) * (by + h - 1);
+        const float rounds = (float)((busy + 2 * TILE_THREADS - 1) / (2 * TILE_THREADS));
+        const float us = waves * (over + h * (0.8f + rounds * per)) / h;
         if (best.halo == 0 || us < best.us) best = {bx, by, tx, ty, h, us};
       }
     }

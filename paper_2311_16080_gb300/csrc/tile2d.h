@@ -26,9 +26,12 @@ struct Tile2dArgs {
   int storage, coll;
   const void* src;       // post-collision populations
   void* dst;             // the same `steps` updates later (another buffer)
-  const int* bz;         // per cell 0 or 1 + its row in bz_q, or null
-  const float* bz_q;     // 9 per row: wall distance of the link in each direction, or -1; 1/2 (halfway) for
-                         // a distance below 1/2 where the cell behind is not FLUID
+  const int* bz;         // per cell 0 or 1 + its row in bz_q (rows < 65535), or null
+  // 9 pairs per row.  Pair i of a link in direction i with wall distance q:
+  // {2q, 1 - 2q} or {1/(2q), 1 - 1/(2q)} (q >= 1/2); {1, 0}, the halfway rule as
+  // q = 1/2, for a distance below 1/2 where the cell behind is not FLUID.  Pair
+  // 0: the bit sets of the links with q < 1/2 and of those with q >= 1/2.
+  const float* bz_q;
   Tile2dPlan plan;
   int steps;             // 1 .. halo
   void* stream;
