@@ -67,6 +67,7 @@ struct xlb_ctx {
   bool has_lid_eq = false;        // LID or EQ cells
   float* init_fields = nullptr;  // (1 + D) * N: rho0, u0 (component-major)
   bool has_init = false;
+  uint64_t init_epoch = 0;  // buf[cur] is f_0 of init_fields under this epoch's parameters (0: it is not)
   int kind_h = 0;
   int64_t t = 0;
   // boundary values and force
@@ -442,6 +443,7 @@ static int check_device_error(xlb_ctx* c) {
 // boundaries it was streamed with and the change acts from step t + 1 on.
 static int materialize_post_stream(xlb_ctx* c) {
   if (!c->kind_h) return XLB_OK;
+  c->init_epoch = 0;
   const int coll = c->coll;
   c->coll = XLB_COLL_NONE;
   const int r = launch_step(c, c->buf[c->cur], c->buf[c->cur ^ 1]);
@@ -457,6 +459,19 @@ static int launch_collide_local(xlb_ctx* c, void* buf) {
   a.dst = buf;
   int r = dispatch(c, OP_COLLIDE_LOCAL, a);
   if (!r) r = boundary_pass(c, nullptr, buf);  // ghosts of the first post-collision state
+  return r;
+}
+
+// The first update: from the initial fields where the state is still f_0 as
+// xlb_init left it, else a local collision of the stored state.
+static int launch_first(xlb_ctx* c, void* buf) {
+  if (c->init_epoch != c->epoch || c->coll == XLB_COLL_NONE) return launch_collide_local(c, buf);
+  LaunchArgs a = base_args(c);
+  a.dst = buf;
+  a.rho = c->init_fields;
+  a.u = c->init_fields + c->N;
+  int r = dispatch(c, OP_FIRST, a);
+  if (!r) r = boundary_pass(c, nullptr, buf);
   return r;
 }
 
@@ -1153,8 +1168,10 @@ int xlb_init(xlb_ctx* c, const float* rho, const float* u) {
   }
   if (!is_device_ptr(rho ? (const void*)rho : (const void*)u)) CK(cudaStreamSynchronize(c->stream));
   c->has_init = true;
+  c->init_epoch = 0;
   int r = launch_init(c, c->buf[c->cur]);
   if (r) return r;
+  c->init_epoch = c->epoch;
   c->kind_h = 0;
   c->t = 0;
   return XLB_OK;
@@ -1364,7 +1381,7 @@ int xlb_step(xlb_ctx* c, int64_t n) {
     }
     int64_t m = 1;
     if (!c->kind_h) {
-      r = launch_collide_local(c, c->buf[c->cur]);
+      r = launch_first(c, c->buf[c->cur]);
       c->kind_h = 1;
     } else {
       // up to the next checkpoint of an open tape
@@ -1576,6 +1593,7 @@ int xlb_state_get(xlb_ctx* c, void* buf, size_t bytes) {
 int xlb_state_set(xlb_ctx* c, const void* buf, size_t bytes) {
   if (!c || !buf) return XLB_ERR_ARG;
   if (c->tape_open) return fail(c, XLB_ERR_STATE, "a tape is open");
+  c->init_epoch = 0;
   if (bytes < 64 + state_bytes_raw(c)) return fail(c, XLB_ERR_ARG, "buffer too small");
   char hdr[64];
   CK(cudaMemcpy(hdr, buf, 64, cudaMemcpyDefault));
@@ -1595,6 +1613,7 @@ int xlb_state_set(xlb_ctx* c, const void* buf, size_t bytes) {
 
 int xlb_populations(xlb_ctx* c, void** ptr, int64_t* plane) {
   if (!c || !ptr || !plane) return XLB_ERR_ARG;
+  c->init_epoch = 0;  // the caller may write through the pointer
   *ptr = c->buf[c->cur];
   *plane = c->plane;
   return XLB_OK;

@@ -23,7 +23,8 @@ XLB_FWD_KBC(27)
 // Collision-dependent ops of a KBC ctx go to the KBC units; everything else to
 // the NONE / BGK units (which also hold the collision-independent kernels).
 static bool kbc_op(Op op, const LaunchArgs& a) {
-  return a.coll == 2 && (op == OP_STEP || op == OP_STEP_VEC || op == OP_BOUNDARY || op == OP_COLLIDE_LOCAL);
+  return a.coll == 2 && (op == OP_STEP || op == OP_STEP_VEC || op == OP_BOUNDARY || op == OP_COLLIDE_LOCAL ||
+                         op == OP_FIRST);
 }
 
 #define XLB_ADJ(Q) \

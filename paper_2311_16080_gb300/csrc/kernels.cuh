@@ -771,6 +771,45 @@ __global__ void __launch_bounds__(ROW_BLOCK) k_collide_local(S* f, const StepPar
   for (int i = 0; i < Q; ++i) rnd.st(f + (long long)i * p.plane + c.self, i, df[i]);
 }
 
+// f^eq(rho, u) - w of one cell from the initial fields (Eq. 5), as k_init
+// stores it before rounding.
+template <int Q>
+__device__ __forceinline__ void init_cell(const float* rho_in, const float* u_in, long long ucs, int self,
+                                          float (&df)[Q]) {
+  const float rho = rho_in ? rho_in[self] : 1.0f;
+  float u[3] = {0.f, 0.f, 0.f};
+  if (u_in) {
+    u[0] = u_in[self];
+    u[1] = u_in[ucs + self];
+    if (Lattice<Q>::D == 3) u[2] = u_in[2 * ucs + self];
+  }
+  const float usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+  const float drho = rho - 1.0f;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) df[i] = weight<Q>(i) * (drho + rho * eq_poly<Q>(i, u, usq));
+}
+
+// The first update after an initialisation, a local collision of f_0: f_0 is
+// formed again from the fields, which are (1 + D) values per cell against the
+// Q that k_init stored (256^3 D3Q19 FP32: 379 us by k_collide_local).  Cells
+// that hold no state keep what k_init gave them, FWALL cells (at rest) too.
+template <int Q, typename S, int COLL>
+__global__ void __launch_bounds__(ROW_BLOCK) k_first(S* f, const StepParams p, const float* rho_in, const float* u_in,
+                                                     long long ucs) {
+  CellIdx c;
+  if (!cell_of_block(p, c)) return;
+  if (p.has_mask && !fluid_like(p.flags[c.self] & FLAG_TYPE)) return;
+  float df[Q];
+  init_cell<Q>(rho_in, u_in, ucs, c.self, df);
+  CellRound<S> rnd;
+  rnd.begin((uint32_t)c.self, df);
+#pragma unroll
+  for (int i = 0; i < Q; ++i) df[i] = rnd.rounded(i, df[i]);
+  collide<Q, COLL>(df, p);
+  rnd.begin((uint32_t)c.self, df);
+  store_cell<Q, S>(f, p, c.self, rnd, df);
+}
+
 // f_0 = f^eq(rho, u) on fluid-like cells (Eq. 5); EQ cells take
 // f^eq(rho_w, u_w); solid cells the rest state.  rho / u may be null
 // (rho = 1, u = 0); u is component-major with stride ucs.
@@ -782,17 +821,7 @@ __global__ void __launch_bounds__(ROW_BLOCK) k_init(S* f, const StepParams p, co
   const int t = p.has_mask ? (p.flags[c.self] & FLAG_TYPE) : FLUID;
   float df[Q];
   if (fluid_like(t)) {
-    const float rho = rho_in ? rho_in[c.self] : 1.0f;
-    float u[3] = {0.f, 0.f, 0.f};
-    if (u_in) {
-      u[0] = u_in[c.self];
-      u[1] = u_in[ucs + c.self];
-      if (Lattice<Q>::D == 3) u[2] = u_in[2 * ucs + c.self];
-    }
-    const float usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    const float drho = rho - 1.0f;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) df[i] = weight<Q>(i) * (drho + rho * eq_poly<Q>(i, u, usq));
+    init_cell<Q>(rho_in, u_in, ucs, c.self, df);
   } else if (t == EQ) {
 #pragma unroll
     for (int i = 0; i < Q; ++i) df[i] = p.eq_df[i];
@@ -821,25 +850,23 @@ __device__ __forceinline__ void post_stream(const S* f, const StepParams& p, con
   }
 }
 
-// Readouts of the post-stream state, one kernel for the three of them (so
-// that the boundary-aware pull is compiled once per lattice and storage):
-//  RD_MACRO:   observables (Eqs. 6-7): rho and the reported velocity
-//              u = (j + F/2) / rho on fluid-like cells; EQ cells report
-//              (rho_w, u_w); solid cells zeros.  u is component-major, stride ucs.
+// Sums over the post-stream state, one kernel for both of them (so that the
+// boundary-aware pull is compiled once per lattice and storage):
 //  RD_MOMENTS: FP64 block partial sums of (mass, j_x, j_y, j_z) over the
 //              fluid-like cells (populations w_i + df_i, bare momentum).
 //  RD_KE:      FP64 block partial sums of the kinetic energy (1/2) rho |u|^2
-//              of the observables RD_MACRO reports (rho, u formed in FP32, the
+//              of the observables k_macro reports (rho, u formed in FP32, the
 //              square and the sum in FP64): the loss of the gradient
 //              workloads (Section 6 takes gradients of rollout losses).
+// Observables (Eqs. 6-7): rho and the reported velocity u = (j + F/2) / rho on
+// fluid-like cells; EQ cells report (rho_w, u_w); solid cells zeros.
 // Grid-stride over the cells of the box [lo, lo + ext); one partial row
-// (4 doubles) per block for the sums.
-enum ReadoutMode { RD_MACRO = 0, RD_MOMENTS = 1, RD_KE = 2 };
+// (4 doubles) per block.
+enum ReadoutMode { RD_MOMENTS = 1, RD_KE = 2 };
 
 template <int Q, typename S>
 __global__ void __launch_bounds__(ROW_BLOCK) k_readout(const S* f, const StepParams p, int kind_h, int mode,
-                                                       int3 lo, int3 ext, float* rho_out, float* u_out,
-                                                       long long ucs, double* partial) {
+                                                       int3 lo, int3 ext, double* partial) {
   const long long nbox = (long long)ext.x * ext.y * ext.z;
   double acc[4] = {0.0, 0.0, 0.0, 0.0};
   for (long long k = blockIdx.x * (long long)ROW_BLOCK + threadIdx.x; k < nbox;
@@ -889,19 +916,9 @@ __global__ void __launch_bounds__(ROW_BLOCK) k_readout(const S* f, const StepPar
       u[1] = p.eq_u[1];
       u[2] = Lattice<Q>::D == 3 ? p.eq_u[2] : 0.f;
     }
-    if (mode == RD_KE) {
-      const double u0 = u[0], u1 = u[1], u2 = u[2];
-      acc[0] += 0.5 * (double)rho * (u0 * u0 + u1 * u1 + u2 * u2);
-    } else if (mode == RD_MACRO) {
-      if (rho_out) rho_out[c.self] = rho;
-      if (u_out) {
-        u_out[c.self] = u[0];
-        u_out[ucs + c.self] = u[1];
-        if (Lattice<Q>::D == 3) u_out[2 * ucs + c.self] = u[2];
-      }
-    }
+    const double u0 = u[0], u1 = u[1], u2 = u[2];
+    acc[0] += 0.5 * (double)rho * (u0 * u0 + u1 * u1 + u2 * u2);
   }
-  if (mode == RD_MACRO) return;
   __shared__ double red[ROW_BLOCK / 32][4];
 #pragma unroll
   for (int m = 0; m < 4; ++m)
@@ -917,6 +934,51 @@ __global__ void __launch_bounds__(ROW_BLOCK) k_readout(const S* f, const StepPar
       for (int q = 0; q < ROW_BLOCK / 32; ++q) s += red[q][m];
       partial[4 * (long long)blockIdx.x + m] = s;
     }
+}
+
+// The observables of the whole lattice, one cell per thread of the bulk
+// passes' mapping; only cells beside a boundary take the pull with its rules
+// (k_readout's grid-stride loop and its rule-aware pull for every cell took 491
+// us for a 256^3 D3Q19 FP32 cavity; its bytes take 228).
+template <int Q, typename S>
+__global__ void __launch_bounds__(ROW_BLOCK) k_macro(const S* f, const StepParams p, int kind_h, float* rho_out,
+                                                     float* u_out, long long ucs) {
+  CellIdx c;
+  if (!cell_of_block(p, c)) return;
+  const int fl = p.has_mask ? p.flags[c.self] : 0, t = fl & FLAG_TYPE;
+  float rho = 0.f, u[3] = {0.f, 0.f, 0.f};
+  if (fluid_like(t)) {
+    float df[Q];
+    if (kind_h && !(fl & FLAG_SLOW)) {
+      Nbr nb;
+      make_nbr(nb, c.x, c.y, c.z, p.nx, p.ny, p.nz);
+      pull_plain<Q, S>(f, p, nb, df);
+    } else {
+      post_stream<Q, S>(f, p, c, fl, kind_h, df);
+    }
+    float drho, j[3];
+    moments<Q>(df, drho, j);
+    if (p.has_force) {
+      j[0] += 0.5f * p.F[0];
+      j[1] += 0.5f * p.F[1];
+      j[2] += 0.5f * p.F[2];
+    }
+    rho = 1.0f + drho;
+    u[0] = j[0] / rho;
+    u[1] = j[1] / rho;
+    u[2] = Lattice<Q>::D == 3 ? j[2] / rho : 0.f;
+  } else if (t == EQ) {
+    rho = p.eq_rho;
+    u[0] = p.eq_u[0];
+    u[1] = p.eq_u[1];
+    u[2] = p.eq_u[2];
+  }
+  if (rho_out) rho_out[c.self] = rho;
+  if (u_out) {
+    u_out[c.self] = u[0];
+    u_out[ucs + c.self] = u[1];
+    if (Lattice<Q>::D == 3) u_out[2 * ucs + c.self] = u[2];
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1054,6 +1116,12 @@ int launch_typed(Op op, const LaunchArgs& a) {
                                a.link_cells, a.link_q, (int)a.n_links, a.fix, (int)a.n_fix, a.fix_mode,
                                (S*)a.side) == cudaSuccess ? 0 : -3;
     }
+    case OP_FIRST:
+      if constexpr (COLL != COLL_NONE) {
+        k_first<Q, S, COLL><<<grid, block, 0, st>>>((S*)a.dst, p, a.rho, a.u, a.ucs);
+        return 0;
+      }
+      return -4;
     case OP_COLLIDE_LOCAL:
       k_collide_local<Q, S, COLL><<<grid, block, 0, st>>>((S*)a.dst, p);
       return 0;
@@ -1066,21 +1134,22 @@ int launch_typed(Op op, const LaunchArgs& a) {
         k_init<Q, S><<<grid, block, 0, st>>>((S*)a.dst, p, a.rho, a.u, a.ucs);
         return 0;
       case OP_MACRO:
+        k_macro<Q, S><<<grid, block, 0, st>>>((const S*)a.src, p, a.kind_h, a.rho_out, a.u_out, a.ucs);
+        return 0;
       case OP_REDUCE_PARTIAL:
       case OP_KE_PARTIAL: {
-        // readouts over a box: the whole lattice, or the KE box; the sums take
+        // sums over a box: the whole lattice, or the KE box, by
         // min(ceil(box cells / ROW_BLOCK), partial_capacity) blocks, at least 1
         const bool box = op == OP_KE_PARTIAL;
         const int3 lo = box ? make_int3(a.box_lo[0], a.box_lo[1], a.box_lo[2]) : make_int3(0, 0, 0);
         const int3 ext = box ? make_int3(a.box_ext[0], a.box_ext[1], a.box_ext[2]) : make_int3(p.nx, p.ny, p.nz);
         const long long nbox = (long long)ext.x * ext.y * ext.z;
         long long b = (nbox + ROW_BLOCK - 1) / ROW_BLOCK;
-        if (op != OP_MACRO && b > a.partial_capacity) b = a.partial_capacity;
+        if (b > a.partial_capacity) b = a.partial_capacity;
         if (b > 0x7fffffffLL) b = 0x7fffffffLL;
         if (b < 1) b = 1;
-        const int mode = op == OP_MACRO ? RD_MACRO : (op == OP_REDUCE_PARTIAL ? RD_MOMENTS : RD_KE);
-        k_readout<Q, S><<<(unsigned)b, ROW_BLOCK, 0, st>>>((const S*)a.src, p, a.kind_h, mode, lo, ext, a.rho_out,
-                                                          a.u_out, a.ucs, a.partial);
+        k_readout<Q, S><<<(unsigned)b, ROW_BLOCK, 0, st>>>((const S*)a.src, p, a.kind_h, box ? RD_KE : RD_MOMENTS, lo,
+                                                          ext, a.partial);
         return 0;
       }
       case OP_WALL_FORCE: {

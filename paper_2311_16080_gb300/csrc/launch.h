@@ -20,6 +20,7 @@ enum Op {
                          // min(ceil(n_links / 256), partial_capacity) rows, at least 1
   OP_KE_PARTIAL = 10,    // block partial sums of the kinetic energy over a box:
                          // min(ceil(box cells / ROW_BLOCK), partial_capacity) rows, at least 1
+  OP_FIRST = 12,         // dst = C(f^eq(rho, u)) on the cells that hold state (the first update)
   OP_FACE_GHOSTS = 11    // ghost values of the boundary faces from the stored state in dst
 };
 
