@@ -91,6 +91,7 @@ struct xlb_ctx {
   char* tape_arena = nullptr;  // checkpoints, tape slots and adjoint buffers, kept for reuse
   size_t tape_arena_bytes = 0;
   int64_t seg_loaded = -1;
+  int64_t seg_next = -1;  // the forward pass has put the last segment's states before this time into the slots
   float* abar[2] = {nullptr, nullptr};
   int acur = 0;
   int64_t adj_t = -1;  // time index of the adjoint held in abar[acur]
@@ -1347,6 +1348,34 @@ static int step_resident(xlb_ctx* c, int64_t room, int64_t* done) {
   return boundary_pass(c, nullptr, c->buf[c->cur]);
 }
 
+// The last segment of an open tape: its states are the ones the adjoint walks
+// first, so its updates go straight to the tape slots instead of being
+// recomputed (time t = s k + j belongs in slot j).  Takes up to `room` updates
+// from time t on and leaves the state of the last one in buf[cur] too.
+static int step_last_segment(xlb_ctx* c, int64_t room, int64_t* done) {
+  *done = 0;
+  if (!c->tape_open || !c->kind_h) return XLB_OK;
+  const int64_t s = (c->tape_T - 1) / c->tape_k, t0 = s * c->tape_k;
+  if (c->t < t0 || c->t < 1) return XLB_OK;
+  if (c->t != std::max<int64_t>(t0, 1) && c->t != c->seg_next) return XLB_OK;  // (updates taken elsewhere: recomputed)
+  auto slot = [&](int64_t t) { return c->slots[(size_t)(t - t0)]; };
+  const size_t bytes = state_bytes_raw(c);
+  // the first state of the segment, or of this call
+  CK(cudaMemcpyAsync(slot(c->t), c->buf[c->cur], bytes, cudaMemcpyDeviceToDevice, c->stream));
+  const int64_t n = std::min(room, c->tape_T - c->t);
+  for (int64_t k = 0; k < n; ++k) {
+    const int64_t t = c->t + k;
+    const bool out = k + 1 == n;
+    const int r = launch_step(c, slot(t), out ? c->buf[c->cur ^ 1] : slot(t + 1));
+    if (r) return r;
+  }
+  c->cur ^= 1;
+  c->seg_next = c->t + n;
+  if (c->seg_next == c->tape_T) c->seg_loaded = s;
+  *done = n;
+  return XLB_OK;
+}
+
 int xlb_step(xlb_ctx* c, int64_t n) {
   if (!c) return XLB_ERR_ARG;
   if (n < 0) return fail(c, XLB_ERR_ARG, "n must be >= 0");
@@ -1358,8 +1387,10 @@ int xlb_step(xlb_ctx* c, int64_t n) {
     if (c->kind_h && !c->prof) {
       // up to the next checkpoint of an open tape
       int64_t room = n - k, m = 0;
+      r = step_last_segment(c, room, &m);
+      if (r) return r;
       if (c->tape_open) room = std::min(room, c->tape_k - c->t % c->tape_k);
-      r = step_resident(c, room, &m);
+      if (m == 0) r = step_resident(c, room, &m);
       if (r) return r;
       if (m > 0) {
         c->t += m;
@@ -1633,6 +1664,7 @@ int xlb_tape_end(xlb_ctx* c) {
   c->abar[0] = c->abar[1] = nullptr;
   c->tape_open = false;
   c->seg_loaded = -1;
+  c->seg_next = -1;
   c->adj_t = -1;
   return XLB_OK;
 }

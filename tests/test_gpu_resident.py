@@ -122,3 +122,33 @@ def test_tiles_with_inflow_outflow_and_curved_walls(n_d, inlet, bouzidi, graph, 
         assert np.array_equal(a.wall_force(), b.wall_force())
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("T,k,chunks", [(1, 1, (1,)), (2, 2, (2,)), (12, 4, (12,)), (13, 4, (5, 6, 2)), (9, 20, (4, 5)),
+                                        (11, 5, (10, 1)), (8, 1, (8,))])
+def test_last_tape_segment_needs_no_recomputation(T, k, chunks):
+    """The forward pass keeps the last segment's states in the tape slots: the
+    gradient equals the one of a forward pass that profiles (and so launches
+    every update by itself and keeps nothing), in any chunks, and the state
+    between the chunks is the live one."""
+    sh = (6, 7, 10)
+    r, u = I.random_flow(sh, 3, seed=81, rho_amp=0.01, u_amp=0.02)
+    m = I.lid_driven_cavity_mask(10, 7, 6)
+    c = Case(19, sh, 1.4, "bgk", mask=m, lid=(1.0, (0.03, 0.0, 0.0)), rho0=r, u0=u)
+    out = []
+    for mode in ("keep", "profile", "mixed"):
+        s = c.gpu_sim()
+        X.xlb_tape_begin(s.ctx, T, k)
+        for i, n in enumerate(chunks):
+            X.xlb_profile_enable(s.ctx, mode == "profile" or (mode == "mixed" and i % 2 == 1))
+            s.step(n)
+            mid = s.macroscopic()
+        X.xlb_adjoint_seed_macro(s.ctx, np.ones(sh, np.float32), None)
+        X.xlb_adjoint_step(s.ctx, T)
+        g = np.empty(sh, np.float32)
+        X.xlb_adjoint_init_grad(s.ctx, g, None)
+        out.append((g,) + mid)
+        s.close()
+    for other in out[1:]:
+        for x, y in zip(out[0], other):
+            assert np.array_equal(x, y)
