@@ -363,9 +363,11 @@ int xlb_tape_release(xlb_ctx* ctx);
  *     (16-bit storage, D2Q9 / D3Q19, BGK, nx % 4 == 0);
  *   XLB_KERNEL_VEC2:   the same with 2 cells per thread and 32-bit words
  *     (nx even);
- *   XLB_KERNEL_AUTO:   the default: with FP16 storage VEC on lattices without
- *     boundary planes and VEC2 with them, else DIRECT (the fastest measured
- *     on 256^3 D3Q19 lattices; BF16 and FP32 run DIRECT).
+ *   XLB_KERNEL_AUTO:   the default, the fastest measured: FP16 runs VEC on
+ *     lattices without boundary planes and VEC2 with them (D3Q19: VEC from 8 M
+ *     cells, DIRECT between 16,384 and 3 M cells where the x-faces are the
+ *     only links), BF16 DIRECT (VEC on D3Q19 lattices of 500,000 cells or more
+ *     without boundary planes), FP32 DIRECT.
  * A mask with an FWALL face plane always runs DIRECT. */
 enum { XLB_KERNEL_AUTO = 0, XLB_KERNEL_DIRECT = 1, XLB_KERNEL_VEC = 2, XLB_KERNEL_VEC2 = 3 };
 

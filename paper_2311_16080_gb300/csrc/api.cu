@@ -304,21 +304,33 @@ static bool has_fwall_face(const xlb_ctx* c) {
 }
 
 // The bulk variant an update launches: the requested one where it can run
-// this ctx, and for AUTO the fastest measured on the 256^3 D3Q19 lattices
-// (periodic box and cavity): with FP16 storage 4 cells per thread without
-// boundary faces (70.4 k MLUPS against 66.3 k for one cell per thread) and 2
-// cells per thread with them (59.0 k against 57.3 k); with BF16 storage
-// (whose stochastic rounding adds per-value work) and FP32 one cell per
-// thread.  Masks with FWALL faces always run one cell per thread.
+// this ctx, and for AUTO the fastest measured on D3Q19 lattices (us per update,
+// one / two / four cells per thread):
+//   FP16 without boundary planes   256^3 253 / 232 / 223, 64^3 5.4 / 5.0 / 4.9
+//   FP16 cavity                    256^3 289 / 263 / 259, 160^3 74 / 73 / 74,
+//                                  132 x 100 x 90 23 / 25 / 27, 64^3 8 / 12 / 13
+//   BF16 without boundary planes   256^3 297 / 312 / 292, 160^3 82 / 80 / 76,
+//                                  64^3 6.2 / 6.6 / 6.8
+//   BF16 cavity                    one cell throughout; FP32 too.
+// One cell per thread gains on the cavities because it serves the x-faces
+// itself (x_pull) and then needs no boundary pass; lattices of a few thousand
+// cells, where launches decide, keep two.  Masks with FWALL faces always run
+// one cell per thread.
 static int bulk_variant(const xlb_ctx* c) {
   if (c->variant == XLB_KERNEL_DIRECT || has_fwall_face(c)) return XLB_KERNEL_DIRECT;
   if (c->variant == XLB_KERNEL_VEC2) return vec_possible(c, 2) ? XLB_KERNEL_VEC2 : XLB_KERNEL_DIRECT;
   if (c->variant == XLB_KERNEL_VEC) return vec_possible(c, 4) ? XLB_KERNEL_VEC : XLB_KERNEL_DIRECT;
-  if (c->storage != XLB_STORE_F16) return XLB_KERNEL_DIRECT;
+  if (c->storage == XLB_STORE_F32) return XLB_KERNEL_DIRECT;
   bool faces = false;
   for (int f = 0; f < 6; ++f) faces |= c->face[f] != 0;
   if (c->has_mask && c->n_links > 0) faces = true;  // boundary planes served by ghost links
+  if (c->storage == XLB_STORE_BF16)
+    return !faces && c->Q == 19 && c->N >= 500000 && vec_possible(c, 4) ? XLB_KERNEL_VEC : XLB_KERNEL_DIRECT;
   if (!faces && vec_possible(c, 4)) return XLB_KERNEL_VEC;
+  if (faces && c->Q == 19) {
+    if (c->N >= 8000000 && vec_possible(c, 4)) return XLB_KERNEL_VEC;
+    if (c->x_pull && c->N >= 16384 && c->N < 3000000) return XLB_KERNEL_DIRECT;
+  }
   if (vec_possible(c, 2)) return XLB_KERNEL_VEC2;
   return XLB_KERNEL_DIRECT;
 }

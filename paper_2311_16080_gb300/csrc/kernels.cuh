@@ -127,6 +127,7 @@ __device__ __forceinline__ uint32_t face_code(const StepParams& p, int x, int y,
   // over a warp, which covers one row) can only meet x-faces: their types
   // follow from four compares per lane
   if (y > 1 && y < p.ny - 2 && (p.nz == 1 || (z > 1 && z < p.nz - 2))) {
+    if ((p.face[0] | p.face[1]) == 0 || (x > 1 && x < p.nx - 2)) return 0u;
     const int tm = (x == 1 ? p.face[0] : 0) | (x == 0 ? p.face[1] : 0);           // x - 1
     const int ts = (x == 0 ? p.face[0] : 0) | (x == p.nx - 1 ? p.face[1] : 0);    // x
     const int tp = (x == p.nx - 1 ? p.face[0] : 0) | (x == p.nx - 2 ? p.face[1] : 0);  // x + 1

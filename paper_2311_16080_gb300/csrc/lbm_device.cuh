@@ -185,42 +185,15 @@ __device__ __forceinline__ void reverse_populations(float (&df)[Q]) {
 template <int Q, typename S, bool FW = true>
 __device__ __forceinline__ bool pull_periodic(const S* src, const StepParams& p, const Nbr& nb,
                                               int self, int x, int y, int z, float (&df)[Q], bool outlet = false) {
-  // per face, the directions whose source is on it: a source coordinate v - c
-  // equal to the face's, c = +-1
-  uint32_t at[6] = {0u, 0u, 0u, 0u, 0u, 0u};
-  bool near = false;
-  if (p.has_faces) {
-    const int lx = p.nx - 1, ly = p.ny - 1, lz = p.nz - 1;
-    const int xp = nb.xo[2];  // the coordinate x + 1, or x itself (outlet)
-    if (p.face[0] | p.face[1]) {
-      at[0] = (nb.xo[0] == 0 ? dir_bits<Q>(0, 1) : 0u) | (xp == 0 ? dir_bits<Q>(0, -1) : 0u);
-      at[1] = (nb.xo[0] == lx ? dir_bits<Q>(0, 1) : 0u) | (xp == lx ? dir_bits<Q>(0, -1) : 0u);
-    }
-    // a row two or more planes from the y / z face planes (uniform over a
-    // warp that covers one row) can only meet x-faces
-    if (!(y > 1 && y < p.ny - 2 && (p.nz == 1 || (z > 1 && z < p.nz - 2)))) {
-      const int ym = wrap_m(y, p.ny), yp = wrap_p(y, p.ny);
-      at[2] = (ym == 0 ? dir_bits<Q>(1, 1) : 0u) | (yp == 0 ? dir_bits<Q>(1, -1) : 0u);
-      at[3] = (ym == ly ? dir_bits<Q>(1, 1) : 0u) | (yp == ly ? dir_bits<Q>(1, -1) : 0u);
-      if (Lattice<Q>::D == 3 && p.nz > 1) {
-        const int zm = wrap_m(z, p.nz), zp = wrap_p(z, p.nz);
-        at[4] = (zm == 0 ? dir_bits<Q>(2, 1) : 0u) | (zp == 0 ? dir_bits<Q>(2, -1) : 0u);
-        at[5] = (zm == lz ? dir_bits<Q>(2, 1) : 0u) | (zp == lz ? dir_bits<Q>(2, -1) : 0u);
-      }
-    }
-#pragma unroll
-    for (int f = 0; f < 6; ++f)
-      if (!p.face[f]) at[f] = 0u;
-    near = (at[0] | at[1] | at[2] | at[3] | at[4] | at[5]) != 0u;
-    if (FW)
-      near |= (x == 0 && p.face[0]) || (x == lx && p.face[1]) || (y == 0 && p.face[2]) || (y == ly && p.face[3]) ||
-              (p.nz > 1 && ((z == 0 && p.face[4]) || (z == lz && p.face[5])));
-  }
+  // next to a face plane, or on it (a superset: its directions follow below)
+  const bool near_x = (p.face[0] | p.face[1]) != 0 && (x <= 1 || x >= p.nx - 2);
+  const bool near_y = (p.face[2] | p.face[3]) != 0 && (y <= 1 || y >= p.ny - 2);
+  const bool near_z = (p.face[4] | p.face[5]) != 0 && (z <= 1 || z >= p.nz - 2);
   const S* base = src;
   // warp-uniform choice: a warp with no lane next to a face loads plainly;
   // otherwise every lane picks each address branch-free, so either way the
   // warp issues one round of Q independent loads
-  if (!__any_sync(__activemask(), near)) {
+  if (!__any_sync(__activemask(), near_x || near_y || near_z)) {
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
       df[i] = Store<S>::ld(base + src_index<Q>(nb, i));
@@ -228,13 +201,25 @@ __device__ __forceinline__ bool pull_periodic(const S* src, const StepParams& p,
     }
     return false;
   }
-  // cells on a face plane: their sources with c = 0 are on it too
-  if (p.face[0] && x == 0) at[0] |= dir_bits<Q>(0, 0);
-  if (p.face[1] && x == p.nx - 1) at[1] |= dir_bits<Q>(0, 0);
-  if (p.face[2] && y == 0) at[2] |= dir_bits<Q>(1, 0);
-  if (p.face[3] && y == p.ny - 1) at[3] |= dir_bits<Q>(1, 0);
-  if (p.face[4] && p.nz > 1 && z == 0) at[4] |= dir_bits<Q>(2, 0);
-  if (p.face[5] && p.nz > 1 && z == p.nz - 1) at[5] |= dir_bits<Q>(2, 0);
+  // per face, the directions whose source is on it: a source coordinate v - c
+  // equal to the face's
+  uint32_t at[6] = {0u, 0u, 0u, 0u, 0u, 0u};
+  const int lx = p.nx - 1, ly = p.ny - 1, lz = p.nz - 1;
+  if (near_x) {
+    const int xm = nb.xo[0], xp = nb.xo[2];  // xp: x + 1, or x itself (outlet)
+    at[0] = (xm == 0 ? dir_bits<Q>(0, 1) : 0u) | (x == 0 ? dir_bits<Q>(0, 0) : 0u) | (xp == 0 ? dir_bits<Q>(0, -1) : 0u);
+    at[1] = (xm == lx ? dir_bits<Q>(0, 1) : 0u) | (x == lx ? dir_bits<Q>(0, 0) : 0u) | (xp == lx ? dir_bits<Q>(0, -1) : 0u);
+  }
+  if (near_y) {
+    const int ym = wrap_m(y, p.ny), yp = wrap_p(y, p.ny);
+    at[2] = (ym == 0 ? dir_bits<Q>(1, 1) : 0u) | (y == 0 ? dir_bits<Q>(1, 0) : 0u) | (yp == 0 ? dir_bits<Q>(1, -1) : 0u);
+    at[3] = (ym == ly ? dir_bits<Q>(1, 1) : 0u) | (y == ly ? dir_bits<Q>(1, 0) : 0u) | (yp == ly ? dir_bits<Q>(1, -1) : 0u);
+  }
+  if (Lattice<Q>::D == 3 && p.nz > 1 && near_z) {
+    const int zm = wrap_m(z, p.nz), zp = wrap_p(z, p.nz);
+    at[4] = (zm == 0 ? dir_bits<Q>(2, 1) : 0u) | (z == 0 ? dir_bits<Q>(2, 0) : 0u) | (zp == 0 ? dir_bits<Q>(2, -1) : 0u);
+    at[5] = (zm == lz ? dir_bits<Q>(2, 1) : 0u) | (z == lz ? dir_bits<Q>(2, 0) : 0u) | (zp == lz ? dir_bits<Q>(2, -1) : 0u);
+  }
   const FaceDirs d = face_dirs(p, at);
   // all loads first (addresses chosen branch-free), adjustments after, so
   // the Q loads stay in flight together
