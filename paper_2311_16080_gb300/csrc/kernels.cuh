@@ -942,7 +942,7 @@ __global__ void __launch_bounds__(ROW_BLOCK) k_readout(const S* f, const StepPar
 // (k_readout's grid-stride loop and its rule-aware pull for every cell took 491
 // us for a 256^3 D3Q19 FP32 cavity; its bytes take 228).
 template <int Q, typename S>
-__global__ void __launch_bounds__(ROW_BLOCK) k_macro(const S* f, const StepParams p, int kind_h, float* rho_out,
+__global__ void __launch_bounds__(ROW_BLOCK, MinBlocks<Q, S, COLL_BGK>::value) k_macro(const S* f, const StepParams p, int kind_h, float* rho_out,
                                                      float* u_out, long long ucs) {
   CellIdx c;
   if (!cell_of_block(p, c)) return;

@@ -186,9 +186,12 @@ template <int Q, typename S, bool FW = true>
 __device__ __forceinline__ bool pull_periodic(const S* src, const StepParams& p, const Nbr& nb,
                                               int self, int x, int y, int z, float (&df)[Q], bool outlet = false) {
   // next to a face plane, or on it (a superset: its directions follow below)
-  const bool near_x = (p.face[0] | p.face[1]) != 0 && (x <= 1 || x >= p.nx - 2);
-  const bool near_y = (p.face[2] | p.face[3]) != 0 && (y <= 1 || y >= p.ny - 2);
-  const bool near_z = (p.face[4] | p.face[5]) != 0 && (z <= 1 || z >= p.nz - 2);
+  bool near_x = false, near_y = false, near_z = false;
+  if (p.has_faces) {
+    near_x = (p.face[0] | p.face[1]) != 0 && (x <= 1 || x >= p.nx - 2);
+    near_y = (p.face[2] | p.face[3]) != 0 && (y <= 1 || y >= p.ny - 2);
+    near_z = (p.face[4] | p.face[5]) != 0 && (z <= 1 || z >= p.nz - 2);
+  }
   const S* base = src;
   // warp-uniform choice: a warp with no lane next to a face loads plainly;
   // otherwise every lane picks each address branch-free, so either way the
