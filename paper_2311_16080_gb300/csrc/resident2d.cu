@@ -95,8 +95,14 @@ __device__ __forceinline__ void update_pair(const uint32_t (&L0)[9], const uint3
   // odd: slot L_j holds f_opp(j); even: slot i of the cell holds f_opp(i)
 #pragma unroll
   for (int j = 0; j < 9; ++j) {
-    a[opposite<9>(j)] = slot_ld<S, REMOTE>(ODD ? L0[j] : L0[0] + j * SB);
-    b[opposite<9>(j)] = slot_ld<S, REMOTE>(ODD ? L1[j] : L1[0] + j * SB);
+    // (a slot in the cell's own row is the block's own)
+    if (Lattice<9>::c(j, 1) != 0) {
+      a[opposite<9>(j)] = slot_ld<S, REMOTE>(ODD ? L0[j] : L0[0] + j * SB);
+      b[opposite<9>(j)] = slot_ld<S, REMOTE>(ODD ? L1[j] : L1[0] + j * SB);
+    } else {
+      a[opposite<9>(j)] = slot_ld<S, false>(ODD ? L0[j] : L0[0] + j * SB);
+      b[opposite<9>(j)] = slot_ld<S, false>(ODD ? L1[j] : L1[0] + j * SB);
+    }
   }
   F2 f[9];
 #pragma unroll
@@ -117,11 +123,21 @@ __device__ __forceinline__ void update_pair(const uint32_t (&L0)[9], const uint3
   }
   if (!(m0 & M_SOLID)) {
 #pragma unroll
-    for (int i = 0; i < 9; ++i) slot_st<S, REMOTE>(ODD ? L0[i] : L0[0] + i * SB, r0, i, a[i]);
+    for (int i = 0; i < 9; ++i) {
+      if (Lattice<9>::c(i, 1) != 0)
+        slot_st<S, REMOTE>(ODD ? L0[i] : L0[0] + i * SB, r0, i, a[i]);
+      else
+        slot_st<S, false>(ODD ? L0[i] : L0[0] + i * SB, r0, i, a[i]);
+    }
   }
   if (!(m1 & M_SOLID)) {
 #pragma unroll
-    for (int i = 0; i < 9; ++i) slot_st<S, REMOTE>(ODD ? L1[i] : L1[0] + i * SB, r1, i, b[i]);
+    for (int i = 0; i < 9; ++i) {
+      if (Lattice<9>::c(i, 1) != 0)
+        slot_st<S, REMOTE>(ODD ? L1[i] : L1[0] + i * SB, r1, i, b[i]);
+      else
+        slot_st<S, false>(ODD ? L1[i] : L1[0] + i * SB, r1, i, b[i]);
+    }
   }
 }
 
