@@ -1325,12 +1325,12 @@ static int step_resident(xlb_ctx* c, int64_t room, int64_t* done) {
     return XLB_OK;
   if (c->res.ctas < 0) c->res = resident2d_shape(c->storage, c->coll, (int)c->nx, (int)c->ny, true);
   if (c->res.ctas == 0) return XLB_OK;
-  // While a thread holds at most two cells an update costs 0.75 us and 0.85 us
-  // more for each 1024 cells a block (128^2 on 16 blocks: 1.6 us; KBC twice
-  // that); with more the tiles are faster (256 x 128: 3.5 us against 2.0).
+  // With one cell per thread an update costs 0.6 us and 0.9 us more for each
+  // 1024 cells a block (128^2 on 16 blocks: 1.5 us; KBC twice that); with more
+  // the tiles are faster (256 x 128: 3.5 us against 2.0).
   if (!c->res.one) return XLB_OK;
   const double cells = (double)((c->ny + c->res.ctas - 1) / c->res.ctas * c->nx);
-  const double us = 0.75 + 0.85 * cells / 1024.0 * (c->coll == XLB_COLL_KBC ? 2.0 : 1.0);
+  const double us = 0.6 + 0.9 * cells / 1024.0 * (c->coll == XLB_COLL_KBC ? 2.0 : 1.0);
   if (us > single_update_us(c) || (tile_ok(c) && us > c->tile.us)) return XLB_OK;
   ResidentArgs a;
   memset(&a, 0, sizeof a);

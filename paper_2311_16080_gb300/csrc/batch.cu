@@ -16,6 +16,8 @@
 #include <string.h>
 
 #include <algorithm>
+#include <functional>
+#include <map>
 #include <string>
 #include <vector>
 
@@ -309,8 +311,6 @@ struct xlb_batch {
   int* res_order = nullptr;   // the groups' domains one after the other, then those that do not fit
   int n_rest = 0;             // domains that do not fit: they take the queue
   bool queue_only = false;    // the tuner times the queue's launch shape
-  std::vector<cudaStream_t> aux;  // one per group but the first: branches of the captured graph
-  std::vector<cudaEvent_t> ev;
   bool graph_queue = false;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t graph_exec = nullptr;
@@ -339,10 +339,11 @@ static void by_storage(int storage, F&& f) {
   if (storage == XLB_STORE_BF16) f(__nv_bfloat16());
 }
 
-// Group the domains by the cluster size they need; `ord`: largest first.
+// Group the domains by the launch shape they need (blocks per cluster, one or
+// two blocks per SM); `ord`: largest first.
 static bool group_domains(xlb_batch* b, const std::vector<int>& ord) {
-  std::vector<std::vector<int>> by(17);
-  std::vector<Bucket> shape(17);
+  std::map<std::pair<int, int>, std::vector<int>, std::greater<std::pair<int, int>>> by;
+  std::map<std::pair<int, int>, ResidentShape> shape;
   std::vector<int> all, rest;
   for (int d : ord) {
     const ResidentShape s = resident2d_shape(b->storage, COLL_BGK, b->hdoms[d].nx, b->hdoms[d].ny, false);
@@ -350,41 +351,31 @@ static bool group_domains(xlb_batch* b, const std::vector<int>& ord) {
       rest.push_back(d);
       continue;
     }
-    by[s.ctas].push_back(d);
-    ResidentShape& m = shape[s.ctas].shape;
-    m.ctas = s.ctas;
-    m.threads = std::max(m.threads, s.threads);
+    const std::pair<int, int> key(s.ctas, !s.one && s.threads > 512);
+    by[key].push_back(d);
+    auto it = shape.find(key);
+    if (it == shape.end()) {
+      shape[key] = s;
+      continue;
+    }
+    ResidentShape& m = it->second;
+    // one cell per thread only where that serves every domain of the group
+    m.threads = m.one == s.one ? std::max(m.threads, s.threads) : (m.one ? s.threads : m.threads);
+    m.one = m.one && s.one;
     m.smem = std::max(m.smem, s.smem);
-    m.one = by[s.ctas].size() == 1 ? s.one : m.one && s.one;
-    if (!m.one) m.threads = std::min(m.threads, 384);
   }
-  for (int c = 16; c >= 1; --c) {
-    if (by[c].empty()) continue;
-    shape[c].first = (int)all.size();
-    shape[c].count = (int)by[c].size();
-    b->buckets.push_back(shape[c]);
-    all.insert(all.end(), by[c].begin(), by[c].end());
+  for (auto& g : by) {  // larger clusters first
+    Bucket k;
+    k.shape = shape[g.first];
+    k.first = (int)all.size();
+    k.count = (int)g.second.size();
+    b->buckets.push_back(k);
+    all.insert(all.end(), g.second.begin(), g.second.end());
   }
   b->n_rest = (int)rest.size();
   all.insert(all.end(), rest.begin(), rest.end());
-  if (cudaMalloc(&b->res_order, sizeof(int) * all.size()) != cudaSuccess ||
-      cudaMemcpy(b->res_order, all.data(), sizeof(int) * all.size(), cudaMemcpyHostToDevice) != cudaSuccess)
-    return false;
-  // larger clusters first: they need several free SMs of one cluster at once
-  int lo = 0, hi = 0;
-  if (cudaDeviceGetStreamPriorityRange(&lo, &hi) != cudaSuccess) return false;
-  const size_t branches = b->buckets.size() + (b->n_rest > 0);
-  for (size_t k = 0; k < branches; ++k) {
-    cudaStream_t s = nullptr;
-    if (cudaStreamCreateWithPriority(&s, cudaStreamNonBlocking, std::min(lo, hi + (int)k)) != cudaSuccess) return false;
-    b->aux.push_back(s);
-  }
-  for (size_t k = 0; k < branches + 1; ++k) {
-    cudaEvent_t e = nullptr;
-    if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return false;
-    b->ev.push_back(e);
-  }
-  return true;
+  return cudaMalloc(&b->res_order, sizeof(int) * all.size()) == cudaSuccess &&
+         cudaMemcpy(b->res_order, all.data(), sizeof(int) * all.size(), cudaMemcpyHostToDevice) == cudaSuccess;
 }
 
 static unsigned grid_of(long long n, int t) { return (unsigned)((n + t - 1) / t); }
@@ -401,8 +392,6 @@ void xlb_batch_destroy(xlb_batch* b) {
   if (b->doms) cudaFree(b->doms);
   if (b->order) cudaFree(b->order);
   if (b->res_order) cudaFree(b->res_order);
-  for (auto s : b->aux) cudaStreamDestroy(s);
-  for (auto e : b->ev) cudaEventDestroy(e);
   if (b->start) cudaFree(b->start);
   if (b->flags) cudaFree(b->flags);
   if (b->counter) cudaFree(b->counter);
@@ -602,23 +591,14 @@ int xlb_batch_step(xlb_batch* b, int64_t n) {
     if (b->graph) cudaGraphDestroy(b->graph);
     b->graph_exec = nullptr;
     b->graph = nullptr;
-    BCK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-    cudaEventRecord(b->ev[0], b->stream);
-    int rr = 0;
-    size_t used = 0;
-    auto branch = [&]() {
-      cudaStream_t s = b->aux[used];
-      cudaStreamWaitEvent(s, b->ev[0], 0);
-      return s;
-    };
-    auto join = [&](cudaStream_t s) {
-      cudaEventRecord(b->ev[1 + used], s);
-      cudaStreamWaitEvent(b->stream, b->ev[1 + used], 0);
-      ++used;
-    };
+    BCK(cudaGraphCreate(&b->graph, 0));
+    // no node of one group depends on another's; larger clusters first, since
+    // they need several free SMs at once
+    int lo = 0, hi = 0;
+    BCK(cudaDeviceGetStreamPriorityRange(&lo, &hi));
+    int prio = hi;
     if (!queue)
       for (const Bucket& k : b->buckets) {
-        cudaStream_t s = branch();
         ResidentArgs a;
         memset(&a, 0, sizeof a);
         a.src = b->buf[b->cur];
@@ -632,24 +612,37 @@ int xlb_batch_step(xlb_batch* b, int64_t n) {
         a.omega = (float)b->omega;
         a.steps = (int)n;
         a.shape = k.shape;
-        a.stream = s;
-        const int e = launch_resident2d(a);
-        if (e) rr = e;
-        join(s);
+        if (add_resident2d_node(a, b->graph, prio) != 0) {
+          cudaGetLastError();
+          return bfail(b, XLB_ERR_CUDA, "resident kernel rejected");
+        }
+        if (prio < lo) ++prio;
       }
     if (n_queue > 0) {
-      cudaStream_t s = branch();
-      cudaMemsetAsync(b->counter, 0, sizeof(int), s);
+      cudaGraphNode_t reset, node;
+      cudaMemsetParams mp = {};
+      mp.dst = b->counter;
+      mp.elementSize = sizeof(int);
+      mp.width = 1;
+      mp.height = 1;
+      BCK(cudaGraphAddMemsetNode(&reset, b->graph, nullptr, 0, &mp));
+      cudaError_t e = cudaSuccess;
       by_storage(b->storage, [&](auto tag) {
         using S = decltype(tag);
-        k_batch_persistent<S><<<grid, b->threads, 0, s>>>(b->doms, q_order, n_queue, (S*)b->buf[b->cur],
-                                                          (S*)b->buf[b->cur ^ 1], b->flags, (float)b->omega, (int)n,
-                                                          b->counter);
+        S* A = (S*)b->buf[b->cur];
+        S* B = (S*)b->buf[b->cur ^ 1];
+        float om = (float)b->omega;
+        int steps = (int)n, nq = n_queue;
+        void* args[] = {&b->doms, &q_order, &nq, &A, &B, &b->flags, &om, &steps, &b->counter};
+        cudaKernelNodeParams kp = {};
+        kp.func = (void*)k_batch_persistent<S>;
+        kp.gridDim = dim3((unsigned)grid);
+        kp.blockDim = dim3((unsigned)b->threads);
+        kp.kernelParams = args;
+        e = cudaGraphAddKernelNode(&node, b->graph, &reset, 1, &kp);
       });
-      join(s);
+      BCK(e);
     }
-    BCK(cudaStreamEndCapture(b->stream, &b->graph));
-    if (rr) return bfail(b, XLB_ERR_CUDA, "resident kernel launch rejected");
     BCK(cudaGraphInstantiate(&b->graph_exec, b->graph, 0));
     b->graph_steps = (int)n;
     b->graph_threads = b->threads;

@@ -66,6 +66,19 @@ __device__ __forceinline__ void odd_slots(uint32_t aM, uint32_t aU, uint32_t aD,
   }
 }
 
+// Cells per thread: one, whose slot addresses stay in registers for the whole
+// call, or as many as it takes, two at a time.
+enum ResidentMode { R_SINGLE, R_LOOP };
+
+// Whether a slot in direction j of an odd update may lie in another block: a
+// neighbouring row's, in the first and last rows (FAR).  (Upper and lower rows
+// apart cost more in diverging warps than they spared: channel 203 x 67 573 ->
+// 612 us.)
+template <bool FAR>
+__device__ constexpr bool is_far(int j) {
+  return FAR && Lattice<9>::c(j, 1) != 0;
+}
+
 // The block's part of the domain and what an update needs of it.
 struct Part {
   uint32_t base, topU, botD;  // slots; where the rows beyond the last / first one lie
@@ -83,11 +96,41 @@ __device__ __forceinline__ void cell_slots(const Part& d, int c, int m, uint32_t
   odd_slots<S>(aM, aU, aD, m, d.nx, L);
 }
 
+// One update of one cell with slots L (L[0]: its own).
+template <typename S, int COLL, bool ODD, bool FAR>
+__device__ __forceinline__ void update_one(const uint32_t (&L)[9], int c, const Part& d, const StepParams& p, bool last,
+                                           S* out) {
+  constexpr int SB = (int)sizeof(S);
+  float f[9];
+#pragma unroll
+  for (int j = 0; j < 9; ++j) {
+    if (is_far<FAR>(j))
+      f[opposite<9>(j)] = slot_ld<S, true>(ODD ? L[j] : L[0] + j * SB);
+    else
+      f[opposite<9>(j)] = slot_ld<S, false>(ODD ? L[j] : L[0] + j * SB);
+  }
+  collide<9, COLL>(f, p);
+  CellRound<S> r;
+  r.begin(d.key0 + c, f);
+  if (last) {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) r.st(out + (long long)i * d.plane + c, i, f[i]);
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < 9; ++i) {
+    if (is_far<FAR>(i))
+      slot_st<S, true>(ODD ? L[i] : L[0] + i * SB, r, i, f[i]);
+    else
+      slot_st<S, false>(ODD ? L[i] : L[0] + i * SB, r, i, f[i]);
+  }
+}
+
 // One update of two cells (c0 and c1, the collision in packed arithmetic);
 // m: their meta words, a cell that takes no part is marked M_SOLID and its
 // addresses are then the other's.  In the call's last update the result goes
 // to global memory (out: the part's first cell), else back to the slots.
-template <typename S, int COLL, bool ODD, bool REMOTE>
+template <typename S, int COLL, bool ODD, bool FAR>
 __device__ __forceinline__ void update_pair(const uint32_t (&L0)[9], const uint32_t (&L1)[9], int c0, int c1, int m0,
                                             int m1, const Part& d, const StepParams& p, bool last, S* out) {
   constexpr int SB = (int)sizeof(S);
@@ -95,10 +138,9 @@ __device__ __forceinline__ void update_pair(const uint32_t (&L0)[9], const uint3
   // odd: slot L_j holds f_opp(j); even: slot i of the cell holds f_opp(i)
 #pragma unroll
   for (int j = 0; j < 9; ++j) {
-    // (a slot in the cell's own row is the block's own)
-    if (Lattice<9>::c(j, 1) != 0) {
-      a[opposite<9>(j)] = slot_ld<S, REMOTE>(ODD ? L0[j] : L0[0] + j * SB);
-      b[opposite<9>(j)] = slot_ld<S, REMOTE>(ODD ? L1[j] : L1[0] + j * SB);
+    if (is_far<FAR>(j)) {
+      a[opposite<9>(j)] = slot_ld<S, true>(ODD ? L0[j] : L0[0] + j * SB);
+      b[opposite<9>(j)] = slot_ld<S, true>(ODD ? L1[j] : L1[0] + j * SB);
     } else {
       a[opposite<9>(j)] = slot_ld<S, false>(ODD ? L0[j] : L0[0] + j * SB);
       b[opposite<9>(j)] = slot_ld<S, false>(ODD ? L1[j] : L1[0] + j * SB);
@@ -124,8 +166,8 @@ __device__ __forceinline__ void update_pair(const uint32_t (&L0)[9], const uint3
   if (!(m0 & M_SOLID)) {
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
-      if (Lattice<9>::c(i, 1) != 0)
-        slot_st<S, REMOTE>(ODD ? L0[i] : L0[0] + i * SB, r0, i, a[i]);
+      if (is_far<FAR>(i))
+        slot_st<S, true>(ODD ? L0[i] : L0[0] + i * SB, r0, i, a[i]);
       else
         slot_st<S, false>(ODD ? L0[i] : L0[0] + i * SB, r0, i, a[i]);
     }
@@ -133,8 +175,8 @@ __device__ __forceinline__ void update_pair(const uint32_t (&L0)[9], const uint3
   if (!(m1 & M_SOLID)) {
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
-      if (Lattice<9>::c(i, 1) != 0)
-        slot_st<S, REMOTE>(ODD ? L1[i] : L1[0] + i * SB, r1, i, b[i]);
+      if (is_far<FAR>(i))
+        slot_st<S, true>(ODD ? L1[i] : L1[0] + i * SB, r1, i, b[i]);
       else
         slot_st<S, false>(ODD ? L1[i] : L1[0] + i * SB, r1, i, b[i]);
     }
@@ -142,13 +184,13 @@ __device__ __forceinline__ void update_pair(const uint32_t (&L0)[9], const uint3
 }
 
 // Bounds: a batch by FP32 instruction issue; one small domain by the latency
-// of a cluster barrier and of one cell's chain.  Each thread takes two cells
-// a block's width apart, so that the lanes of a warp stay on consecutive
-// cells and the collision runs in packed arithmetic.  ONE: the part has at
-// most two cells per thread, and their slot addresses stay in registers for
-// the whole call.
-template <typename S, int COLL, bool ONE>
-__global__ void __launch_bounds__(ONE ? 512 : 768, 1) k_resident2d(const S* A, S* B, const uint8_t* __restrict__ flags,
+// of a cluster barrier (287 ns) and of one cell's chain.  Each thread takes two
+// cells a warp's width apart: the lanes of a warp stay on consecutive cells, the
+// collision runs in packed arithmetic, and few warps hold cells of the rows
+// whose neighbours are in another block (a pair a block apart instead: 1024
+// channels 51.0 ms, this way 47.7).
+template <typename S, int COLL, int MODE>
+__global__ void __launch_bounds__(MODE == R_SINGLE ? 1024 : 768, 1) k_resident2d(const S* A, S* B, const uint8_t* __restrict__ flags,
                                                        const BatchDom* __restrict__ doms,
                                                        const int* __restrict__ order, const BatchDom one, float omega,
                                                        int steps) {
@@ -208,36 +250,28 @@ __global__ void __launch_bounds__(ONE ? 512 : 768, 1) k_resident2d(const S* A, S
       cluster_barrier();
   };
   barrier();
-  if constexpr (ONE) {
-    int c0 = threadIdx.x, c1 = c0 + blockDim.x, m0 = M_SOLID, m1 = M_SOLID;
-    if (c0 < cells) m0 = meta[c0 * MS];
-    if (c1 < cells) m1 = meta[c1 * MS];
-    const bool act = !(m0 & m1 & M_SOLID);
-    uint32_t L0[9], L1[9];
-    if (act) {
-      if (m0 & M_SOLID) cell_slots<S>(part, c1, m1, L0);
-      else cell_slots<S>(part, c0, m0, L0);
-      if (m1 & M_SOLID) cell_slots<S>(part, c0, m0, L1);
-      else cell_slots<S>(part, c1, m1, L1);
-    }
-    const bool remote = part.split && ((m0 | m1) & (M_YT | M_YB));
+  if constexpr (MODE == R_SINGLE) {
+    const int c = threadIdx.x, m = c < cells ? meta[c * MS] : M_SOLID;
+    uint32_t L[9];
+    if (!(m & M_SOLID)) cell_slots<S>(part, c, m, L);
+    const bool far = part.split && (m & (M_YT | M_YB));
     for (int t = 0; t < steps; ++t) {
       const bool last = t == steps - 1;
-      if (act) {
+      if (!(m & M_SOLID)) {
         if (t & 1)
-          update_pair<S, COLL, false, false>(L0, L1, c0, c1, m0, m1, part, p, last, dst);
-        else if (remote)
-          update_pair<S, COLL, true, true>(L0, L1, c0, c1, m0, m1, part, p, last, dst);
+          update_one<S, COLL, false, false>(L, c, part, p, last, dst);
+        else if (far)
+          update_one<S, COLL, true, true>(L, c, part, p, last, dst);
         else
-          update_pair<S, COLL, true, false>(L0, L1, c0, c1, m0, m1, part, p, last, dst);
+          update_one<S, COLL, true, false>(L, c, part, p, last, dst);
       }
       barrier();
     }
   } else {
     for (int t = 0; t < steps; ++t) {
       const bool last = t == steps - 1;
-      for (int c0 = threadIdx.x; c0 < cells; c0 += 2 * blockDim.x) {
-        const int c1 = c0 + blockDim.x;
+      for (int c0 = 2 * (threadIdx.x & ~31) + (threadIdx.x & 31); c0 < cells; c0 += 2 * blockDim.x) {
+        const int c1 = c0 + 32;
         const int m0 = meta[c0 * MS], m1 = c1 < cells ? meta[c1 * MS] : M_SOLID;
         if (m0 & m1 & M_SOLID) continue;
         uint32_t L0[9], L1[9];
@@ -262,32 +296,70 @@ __global__ void __launch_bounds__(ONE ? 512 : 768, 1) k_resident2d(const S* A, S
   }
 }
 
+// Where a launch goes: a.stream, or a node of `graph`.
+struct Target {
+  cudaGraph_t graph;
+  int priority;
+};
+
 template <typename S, int COLL>
-int launch_typed_resident(const ResidentArgs& a) {
-  auto kern = a.shape.one ? k_resident2d<S, COLL, true> : k_resident2d<S, COLL, false>;
+int launch_typed_resident(const ResidentArgs& a, const Target* t) {
+  auto kern = a.shape.one ? k_resident2d<S, COLL, R_SINGLE> : k_resident2d<S, COLL, R_LOOP>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a.shape.smem) != cudaSuccess ||
       (a.shape.ctas > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess))
     return -3;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(a.n_dom * a.shape.ctas));
-  cfg.blockDim = dim3((unsigned)a.shape.threads);
-  cfg.dynamicSmemBytes = (size_t)a.shape.smem;
-  cfg.stream = (cudaStream_t)a.stream;
+  const S* src = (const S*)a.src;
+  S* dst = (S*)a.dst;
+  const dim3 grid((unsigned)(a.n_dom * a.shape.ctas)), block((unsigned)a.shape.threads);
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = (unsigned)a.shape.ctas;
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  if (t) {
+    ResidentArgs c = a;  // the parameters' values are copied into the node
+    void* args[] = {&src, &dst, &c.flags, &c.doms, &c.order, &c.dom, &c.omega, &c.steps};
+    cudaKernelNodeParams kp = {};
+    kp.func = (void*)kern;
+    kp.gridDim = grid;
+    kp.blockDim = block;
+    kp.sharedMemBytes = (unsigned)a.shape.smem;
+    kp.kernelParams = args;
+    cudaGraphNode_t node;
+    cudaLaunchAttributeValue pr;
+    pr.priority = t->priority;
+    return cudaGraphAddKernelNode(&node, t->graph, nullptr, 0, &kp) == cudaSuccess &&
+                   cudaGraphKernelNodeSetAttribute(node, cudaLaunchAttributeClusterDimension, &at[0].val) == cudaSuccess &&
+                   cudaGraphKernelNodeSetAttribute(node, cudaLaunchAttributePriority, &pr) == cudaSuccess
+               ? 0
+               : -3;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = (size_t)a.shape.smem;
+  cfg.stream = (cudaStream_t)a.stream;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, (const S*)a.src, (S*)a.dst, a.flags, a.doms, a.order, a.dom, a.omega,
-                            a.steps) == cudaSuccess ? 0 : -3;
+  return cudaLaunchKernelEx(&cfg, kern, src, dst, a.flags, a.doms, a.order, a.dom, a.omega, a.steps) == cudaSuccess
+             ? 0
+             : -3;
 }
 
 template <typename S>
-int by_coll(const ResidentArgs& a) {
-  if (a.coll == COLL_BGK) return launch_typed_resident<S, COLL_BGK>(a);
-  if (a.coll == COLL_KBC) return launch_typed_resident<S, COLL_KBC>(a);
+int by_coll(const ResidentArgs& a, const Target* t) {
+  if (a.coll == COLL_BGK) return launch_typed_resident<S, COLL_BGK>(a, t);
+  if (a.coll == COLL_KBC) return launch_typed_resident<S, COLL_KBC>(a, t);
   return -2;
+}
+
+int launch_to(const ResidentArgs& a, const Target* t) {
+  if (a.n_dom < 1 || a.steps < 1 || a.shape.ctas < 1) return -1;
+  switch (a.storage) {
+    case XLB_STORE_F32: return by_coll<float>(a, t);
+    case XLB_STORE_F16: return by_coll<__half>(a, t);
+    case XLB_STORE_BF16: return by_coll<__nv_bfloat16>(a, t);
+  }
+  return -5;
 }
 
 }  // namespace
@@ -304,22 +376,18 @@ ResidentShape resident2d_shape(int storage, int coll, int nx, int ny, bool alone
       const long long cells = (long long)((ny + c - 1) / c) * nx;
       const long long smem = (cells * cell + 15) / 16 * 16;
       if (smem > limit) continue;
-      const long long pairs = (cells + 1) / 2;
+      if (cells <= 1024) return {c, (int)((cells + 31) / 32 * 32), smem, true};
       // 80 registers: 768 threads fill an SM
-      const int threads = (int)(pairs <= 512 ? (pairs + 31) / 32 * 32 : limit > 112 * 1024 ? 768 : 384);
-      return {c, threads, smem, pairs <= 512};
+      return {c, limit > 112 * 1024 ? 768 : 384, smem, false};
     }
   return none;
 }
 
-int launch_resident2d(const ResidentArgs& a) {
-  if (a.n_dom < 1 || a.steps < 1 || a.shape.ctas < 1) return -1;
-  switch (a.storage) {
-    case XLB_STORE_F32: return by_coll<float>(a);
-    case XLB_STORE_F16: return by_coll<__half>(a);
-    case XLB_STORE_BF16: return by_coll<__nv_bfloat16>(a);
-  }
-  return -5;
+int launch_resident2d(const ResidentArgs& a) { return launch_to(a, nullptr); }
+
+int add_resident2d_node(const ResidentArgs& a, void* graph, int priority) {
+  const Target t = {(cudaGraph_t)graph, priority};
+  return launch_to(a, &t);
 }
 
 }  // namespace xlb

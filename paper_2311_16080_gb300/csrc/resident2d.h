@@ -20,7 +20,7 @@ struct BatchDom {
 struct ResidentShape {
   int ctas, threads;
   long long smem;  // dynamic shared memory per block
-  bool one;        // at most two cells per thread
+  bool one;        // one cell per thread
 };
 
 // Shape for an nx x ny domain: alone on the GPU (spread wide, so that one
@@ -44,5 +44,7 @@ struct ResidentArgs {
 
 // 0 on a successful launch request, else a negative code.
 int launch_resident2d(const ResidentArgs& a);
+// The same launch as a node of a graph (cudaGraph_t), with a launch priority.
+int add_resident2d_node(const ResidentArgs& a, void* graph, int priority);
 
 }  // namespace xlb
