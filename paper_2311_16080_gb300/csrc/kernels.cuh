@@ -199,17 +199,35 @@ __device__ __forceinline__ uint32_t x_rule_dirs(uint32_t fc) {
 
 // Pull with the rules of the x-face planes (16-bit storage without FWALL
 // faces), the address chosen before the load so that a warp that meets an
-// x-face still issues one round of loads.
-template <int Q, typename S>
+// x-face still issues one round of loads.  PAIRS: with the two planes of a pair
+// (i, opp(i)) at hand, which is cheaper (128 x 83 x 61 FP16 13.9 -> 13.1 us, 161 x
+// 130 x 127 BF16 59.7 -> 58.1) but for FP16 on the flat mapping, where the
+// kernel's other path lost registers to it (161 x 130 x 127 42.8 -> 44.4).
+template <int Q, typename S, bool PAIRS>
 __device__ __forceinline__ void pull_x_faces(const S* src, const StepParams& p, const Nbr& nb, int self,
                                              uint32_t fc, uint32_t xr, float (&df)[Q]) {
-  const S* base = src;
+  if constexpr (PAIRS) {
+    df[0] = Store<S>::ld(src + self);
 #pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    const S* a = base + src_index<Q>(nb, i);
-    if (Lattice<Q>::c(i, 0) != 0 && (xr >> i & 1)) a = src + (long long)opposite<Q>(i) * p.plane + self;
-    df[i] = Store<S>::ld(a);
-    base += p.plane;
+    for (int i = 1; i < Q; ++i) {
+      if (opposite<Q>(i) > i) {
+        const int k = opposite<Q>(i);
+        const S* pi = src + (long long)i * p.plane;
+        const S* pk = src + (long long)k * p.plane;
+        const bool bi = Lattice<Q>::c(i, 0) != 0 && (xr >> i & 1), bk = Lattice<Q>::c(i, 0) != 0 && (xr >> k & 1);
+        df[i] = Store<S>::ld((bi ? pk : pi) + (bi ? self : src_index<Q>(nb, i)));
+        df[k] = Store<S>::ld((bk ? pi : pk) + (bk ? self : src_index<Q>(nb, k)));
+      }
+    }
+  } else {
+    const S* base = src;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      const S* a = base + src_index<Q>(nb, i);
+      if (Lattice<Q>::c(i, 0) != 0 && (xr >> i & 1)) a = src + (long long)opposite<Q>(i) * p.plane + self;
+      df[i] = Store<S>::ld(a);
+      base += p.plane;
+    }
   }
   if (p.face[0] <= WALL && p.face[1] <= WALL) return;
   if (xr) {
@@ -357,7 +375,7 @@ __global__ void __launch_bounds__(ROW_BLOCK, MinBlocks<Q, S, COLL>::value)
     } else {
       const uint32_t xr = (fc & FC_XN) ? x_rule_dirs<Q>(fc) : 0u;
       if (__any_sync(__activemask(), xr))
-        pull_x_faces<Q, S>(src, p, nb, c.self, fc, xr, df);
+        pull_x_faces<Q, S, !FLAT || std::is_same<S, __nv_bfloat16>::value>(src, p, nb, c.self, fc, xr, df);
       else
         pull_plain<Q, S>(src, p, nb, df);
     }

@@ -224,14 +224,22 @@ __device__ __forceinline__ bool pull_periodic(const S* src, const StepParams& p,
     at[5] = (zm == lz ? dir_bits<Q>(2, 1) : 0u) | (z == lz ? dir_bits<Q>(2, 0) : 0u) | (zp == lz ? dir_bits<Q>(2, -1) : 0u);
   }
   const FaceDirs d = face_dirs(p, at);
-  // all loads first (addresses chosen branch-free), adjustments after, so
-  // the Q loads stay in flight together
+  // all loads first (addresses chosen branch-free, the two planes of a pair
+  // (i, opp(i)) at hand), adjustments after, so the Q loads stay in flight
+  // together
+  df[0] = Store<S>::ld(src + self);
 #pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    const int own = (Lattice<Q>::c(i, 0) == -1 && outlet) ? self - 1 : self;
-    const S* a = (d.own >> i & 1) ? src + (long long)opposite<Q>(i) * p.plane + own : base + src_index<Q>(nb, i);
-    df[i] = Store<S>::ld(a);
-    base += p.plane;
+  for (int i = 1; i < Q; ++i) {
+    if (opposite<Q>(i) > i) {
+      const int k = opposite<Q>(i);
+      const S* pi = src + (long long)i * p.plane;
+      const S* pk = src + (long long)k * p.plane;
+      const bool bi = d.own >> i & 1, bk = d.own >> k & 1;
+      const int si = (Lattice<Q>::c(i, 0) == -1 && outlet) ? self - 1 : self;
+      const int sk = (Lattice<Q>::c(k, 0) == -1 && outlet) ? self - 1 : self;
+      df[i] = Store<S>::ld((bi ? pk : pi) + (bi ? si : src_index<Q>(nb, i)));
+      df[k] = Store<S>::ld((bk ? pi : pk) + (bk ? sk : src_index<Q>(nb, k)));
+    }
   }
   if (d.lid | d.eq) {
 #pragma unroll
