@@ -496,6 +496,14 @@ static int launch_init(xlb_ctx* c, void* dst) {
   return dispatch(c, OP_INIT, a);
 }
 
+static void free_bz(xlb_ctx* c) {
+  if (c->bz) cudaFree(c->bz);
+  if (c->bz_q) cudaFree(c->bz_q);
+  c->bz = nullptr;
+  c->bz_q = nullptr;
+  c->n_bz = 0;
+}
+
 // The six boundary planes of a mask, gathered on the device into one compact
 // host buffer (the x-planes are strided in the mask): plane f (x = 0,
 // x = nx - 1, y = 0, ..., z = nz - 1) holds its cells at a + n1 * b, (a, b)
@@ -915,6 +923,7 @@ int xlb_set_mask(xlb_ctx* c, const uint8_t* mask) {
   if (c->link_cells) cudaFree(c->link_cells);
   if (c->link_q) cudaFree(c->link_q);
   c->link_q = nullptr;  // wall distances belong to the old link table
+  free_bz(c);
   if (c->fix_side) cudaFree(c->fix_side);
   c->fix_side = nside;
   if (c->fix) cudaFree(c->fix);
@@ -1040,13 +1049,13 @@ int xlb_set_wall_distances(xlb_ctx* c, int64_t n, const int64_t* cell, const int
   if (r) return r;
   if (c->link_q) CK(cudaFree(c->link_q));
   c->link_q = nullptr;
-  if (c->bz) CK(cudaFree(c->bz));
-  if (c->bz_q) CK(cudaFree(c->bz_q));
-  c->bz = nullptr;
-  c->bz_q = nullptr;
-  c->n_bz = 0;
+  free_bz(c);
+  ++c->epoch;
+  if (n > 0) CK(cudaMalloc(&c->link_q, sizeof(float) * hq.size()));
+  if (n > 0) CK(cudaMemcpy(c->link_q, hq.data(), sizeof(float) * hq.size(), cudaMemcpyHostToDevice));
   if (n > 0 && c->Q == 9) {
-    // the same by cell, for the tiled kernel
+    // the same by cell, for the tiled kernel (which is not used without them:
+    // no memory for them is no error)
     std::vector<uint8_t> fl((size_t)c->N);
     CK(cudaMemcpy(fl.data(), c->flags, fl.size(), cudaMemcpyDeviceToHost));
     std::vector<int> row((size_t)c->N, 0);
@@ -1075,15 +1084,21 @@ int xlb_set_wall_distances(xlb_ctx* c, int64_t n, const int64_t* cell, const int
     }
     for (size_t r0 = 0; r0 < bits.size() / 2; ++r0) memcpy(rq.data() + 18 * r0, bits.data() + 2 * r0, 8);
     c->n_bz = (int64_t)rq.size() / 18;
-    CK(cudaMalloc(&c->bz, sizeof(int) * row.size()));
-    CK(cudaMalloc(&c->bz_q, sizeof(float) * rq.size()));
-    CK(cudaMemcpy(c->bz, row.data(), sizeof(int) * row.size(), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(c->bz_q, rq.data(), sizeof(float) * rq.size(), cudaMemcpyHostToDevice));
+    cudaError_t e = cudaMalloc(&c->bz, sizeof(int) * row.size());
+    if (e == cudaSuccess) e = cudaMalloc(&c->bz_q, sizeof(float) * rq.size());
+    if (e == cudaErrorMemoryAllocation) {
+      cudaGetLastError();
+      free_bz(c);
+    } else {
+      if (e == cudaSuccess) e = cudaMemcpy(c->bz, row.data(), sizeof(int) * row.size(), cudaMemcpyHostToDevice);
+      if (e == cudaSuccess) e = cudaMemcpy(c->bz_q, rq.data(), sizeof(float) * rq.size(), cudaMemcpyHostToDevice);
+      if (e != cudaSuccess) {
+        free_bz(c);
+        return cuda_fail(c, e, "wall distances by cell");
+      }
+    }
   }
-  if (n > 0) CK(cudaMalloc(&c->link_q, sizeof(float) * hq.size()));
-  if (n > 0) CK(cudaMemcpy(c->link_q, hq.data(), sizeof(float) * hq.size(), cudaMemcpyHostToDevice));
   if (!hl.empty()) CK(cudaMemcpy(c->links, hl.data(), sizeof(int2) * hl.size(), cudaMemcpyHostToDevice));
-  ++c->epoch;
   return XLB_OK;
 }
 
@@ -1224,9 +1239,10 @@ static bool tile_ok(xlb_ctx* c) {
 // n updates of the post-collision state in buf[*cur], launched (or captured)
 // on the ctx stream; *cur becomes the buffer that holds the result.  The tiled
 // kernel needs no ghost values; those of the last state are written at the end.
-static int run_updates(xlb_ctx* c, int* cur, int64_t n) {
+// keep: they end in the buffer that n single updates end in.
+static int run_updates(xlb_ctx* c, int* cur, int64_t n, bool keep) {
   int r = XLB_OK;
-  if (n < 2 || c->prof || !tile_ok(c)) {
+  if (n < (keep ? 3 : 2) || c->prof || !tile_ok(c)) {
     for (int64_t k = 0; k < n; ++k) {
       r = launch_step(c, c->buf[*cur], c->buf[*cur ^ 1]);
       if (r) return r;
@@ -1244,8 +1260,9 @@ static int run_updates(xlb_ctx* c, int* cur, int64_t n) {
   a.bz_q = c->bz_q;
   a.plan = c->tile;
   a.stream = c->stream;
-  for (int64_t left = n; left > 0;) {
-    const int64_t launches = (left + c->tile.halo - 1) / c->tile.halo;
+  int64_t launches = (n + c->tile.halo - 1) / c->tile.halo;
+  if (keep && (n - launches) % 2) ++launches;
+  for (int64_t left = n; left > 0; --launches) {
     a.steps = (int)((left + launches - 1) / launches);
     a.src = c->buf[*cur];
     a.dst = c->buf[*cur ^ 1];
@@ -1276,7 +1293,7 @@ static int step_graph(xlb_ctx* c, int from, cudaGraphExec_t* out) {
   if (cs != cudaStreamCaptureStatusNone) return fail(c, XLB_ERR_STATE, "the ctx stream is already capturing");
   CK(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
   int cur = from;
-  const int r = run_updates(c, &cur, c->graph_g);
+  const int r = run_updates(c, &cur, c->graph_g, false);
   cudaGraph_t g = nullptr;
   const cudaError_t e = cudaStreamEndCapture(c->stream, &g);
   if (r != XLB_OK || e != cudaSuccess) {
@@ -1323,7 +1340,11 @@ static int step_resident(xlb_ctx* c, int64_t room, int64_t* done) {
   if (c->Q != 9 || c->coll == XLB_COLL_NONE || room < RESIDENT_MIN || c->has_inlet_outlet || c->has_lid_eq ||
       c->link_q)
     return XLB_OK;
-  if (c->res.ctas < 0) c->res = resident2d_shape(c->storage, c->coll, (int)c->nx, (int)c->ny, true);
+  if (c->res.ctas < 0) {
+    c->res = resident2d_shape(c->storage, c->coll, (int)c->nx, (int)c->ny, true);
+    // (a process given a part of the GPU may have no room for such a cluster)
+    if (c->res.ctas > 0 && resident2d_clusters(c->res, c->storage, c->coll) < 1) c->res.ctas = 0;
+  }
   if (c->res.ctas == 0) return XLB_OK;
   // With one cell per thread an update costs 0.6 us and 0.9 us more for each
   // 1024 cells a block (128^2 on 16 blocks: 1.5 us; KBC twice that); with more
@@ -1335,7 +1356,6 @@ static int step_resident(xlb_ctx* c, int64_t room, int64_t* done) {
   ResidentArgs a;
   memset(&a, 0, sizeof a);
   a.src = c->buf[c->cur];
-  a.dst = c->buf[c->cur ^ 1];
   a.flags = c->has_mask ? c->flags : nullptr;
   a.dom.nx = (int)c->nx;
   a.dom.ny = (int)c->ny;
@@ -1349,13 +1369,14 @@ static int step_resident(xlb_ctx* c, int64_t room, int64_t* done) {
   a.coll = c->coll;
   a.omega = (float)c->omega;
   a.steps = (int)std::min(room, RESIDENT_MAX);
+  a.dst = c->buf[c->cur ^ (a.steps & 1)];  // where as many single updates end
   a.shape = c->res;
   a.stream = c->stream;
   const int r = launch_resident2d(a);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(c, e, "resident kernel launch");
   if (r) return fail(c, XLB_ERR_CUDA, "resident kernel launch rejected (code %d)", r);
-  c->cur ^= 1;
+  c->cur ^= a.steps & 1;
   *done = a.steps;
   return boundary_pass(c, nullptr, c->buf[c->cur]);
 }
@@ -1369,19 +1390,21 @@ static int step_last_segment(xlb_ctx* c, int64_t room, int64_t* done) {
   if (!c->tape_open || !c->kind_h) return XLB_OK;
   const int64_t s = (c->tape_T - 1) / c->tape_k, t0 = s * c->tape_k;
   if (c->t < t0 || c->t < 1) return XLB_OK;
+  if (t0 == 0 && c->init_epoch != c->epoch) return XLB_OK;  // (the adjoint starts from the initial fields)
   if (c->t != std::max<int64_t>(t0, 1) && c->t != c->seg_next) return XLB_OK;  // (updates taken elsewhere: recomputed)
   auto slot = [&](int64_t t) { return c->slots[(size_t)(t - t0)]; };
   const size_t bytes = state_bytes_raw(c);
   // the first state of the segment, or of this call
   CK(cudaMemcpyAsync(slot(c->t), c->buf[c->cur], bytes, cudaMemcpyDeviceToDevice, c->stream));
   const int64_t n = std::min(room, c->tape_T - c->t);
+  const int to = c->cur ^ (int)(n & 1);
   for (int64_t k = 0; k < n; ++k) {
     const int64_t t = c->t + k;
     const bool out = k + 1 == n;
-    const int r = launch_step(c, slot(t), out ? c->buf[c->cur ^ 1] : slot(t + 1));
+    const int r = launch_step(c, slot(t), out ? c->buf[to] : slot(t + 1));
     if (r) return r;
   }
-  c->cur ^= 1;
+  c->cur = to;
   c->seg_next = c->t + n;
   if (c->seg_next == c->tape_T) c->seg_loaded = s;
   *done = n;
@@ -1394,6 +1417,11 @@ int xlb_step(xlb_ctx* c, int64_t n) {
   if (!c->has_init && c->t == 0 && !c->kind_h) return fail(c, XLB_ERR_STATE, "xlb_init (or xlb_state_set) first");
   if (c->tape_open && c->t + n > c->tape_T)
     return fail(c, XLB_ERR_STATE, "stepping past the tape length %lld", (long long)c->tape_T);
+  // In a caller's capture n updates end where n single ones would, so that
+  // replays of an even number go on from each other.
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (n > 1) CK(cudaStreamIsCapturing(c->stream, &cs));
+  const bool keep = cs != cudaStreamCaptureStatusNone;
   for (int64_t k = 0; k < n; ++k) {
     int r;
     if (c->kind_h && !c->prof) {
@@ -1430,7 +1458,7 @@ int xlb_step(xlb_ctx* c, int64_t n) {
       // up to the next checkpoint of an open tape
       m = n - k;
       if (c->tape_open) m = std::min(m, c->tape_k - c->t % c->tape_k);
-      r = run_updates(c, &c->cur, m);
+      r = run_updates(c, &c->cur, m, keep);
     }
     if (r) return r;
     c->t += m;

@@ -340,8 +340,8 @@ static void by_storage(int storage, F&& f) {
 }
 
 // Group the domains by the launch shape they need (blocks per cluster, one or
-// two blocks per SM); `ord`: largest first.
-static bool group_domains(xlb_batch* b, const std::vector<int>& ord) {
+// two blocks per SM) and append that order to `ord`, which is largest first.
+static void group_domains(xlb_batch* b, std::vector<int>& ord) {
   std::map<std::pair<int, int>, std::vector<int>, std::greater<std::pair<int, int>>> by;
   std::map<std::pair<int, int>, ResidentShape> shape;
   std::vector<int> all, rest;
@@ -374,8 +374,7 @@ static bool group_domains(xlb_batch* b, const std::vector<int>& ord) {
   }
   b->n_rest = (int)rest.size();
   all.insert(all.end(), rest.begin(), rest.end());
-  return cudaMalloc(&b->res_order, sizeof(int) * all.size()) == cudaSuccess &&
-         cudaMemcpy(b->res_order, all.data(), sizeof(int) * all.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+  ord.insert(ord.end(), all.begin(), all.end());
 }
 
 static unsigned grid_of(long long n, int t) { return (unsigned)((n + t - 1) / t); }
@@ -391,7 +390,6 @@ void xlb_batch_destroy(xlb_batch* b) {
     if (b->buf[k]) cudaFree(b->buf[k]);
   if (b->doms) cudaFree(b->doms);
   if (b->order) cudaFree(b->order);
-  if (b->res_order) cudaFree(b->res_order);
   if (b->start) cudaFree(b->start);
   if (b->flags) cudaFree(b->flags);
   if (b->counter) cudaFree(b->counter);
@@ -457,7 +455,7 @@ int xlb_batch_create(xlb_batch** out, int n_domains, const int32_t* nx, const in
   for (int k = 0; k < 2; ++k)
     if (cudaMalloc(&b->buf[k], b->esize * (size_t)off) != cudaSuccess) return bail(XLB_ERR_OOM);
   if (cudaMalloc(&b->doms, sizeof(BatchDom) * n_domains) != cudaSuccess ||
-      cudaMalloc(&b->order, sizeof(int) * n_domains) != cudaSuccess ||
+      cudaMalloc(&b->order, sizeof(int) * 2 * n_domains) != cudaSuccess ||
       cudaMalloc(&b->start, sizeof(int) * (n_domains + 1)) != cudaSuccess ||
       cudaMalloc(&b->flags, (size_t)foff) != cudaSuccess || cudaMalloc(&b->counter, 4 * sizeof(int)) != cudaSuccess)
     return bail(XLB_ERR_OOM);
@@ -467,12 +465,13 @@ int xlb_batch_create(xlb_batch** out, int n_domains, const int32_t* nx, const in
   std::stable_sort(ord.begin(), ord.end(), [&](int a, int c) {
     return (long long)nx[a] * ny[a] > (long long)nx[c] * ny[c];
   });
+  group_domains(b, ord);
   if (cudaMemcpy(b->doms, b->hdoms.data(), sizeof(BatchDom) * n_domains, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(b->order, ord.data(), sizeof(int) * n_domains, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(b->order, ord.data(), sizeof(int) * ord.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(b->start, b->hstart.data(), sizeof(int) * (n_domains + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemset(b->counter, 0, 4 * sizeof(int)) != cudaSuccess || cudaMemset(b->flags, 0, (size_t)foff) != cudaSuccess)
     return bail(XLB_ERR_CUDA);
-  if (!group_domains(b, ord)) return bail(XLB_ERR_CUDA);
+  b->res_order = b->order + n_domains;
   *out = b;
   return XLB_OK;
 }
@@ -591,7 +590,9 @@ int xlb_batch_step(xlb_batch* b, int64_t n) {
     if (b->graph) cudaGraphDestroy(b->graph);
     b->graph_exec = nullptr;
     b->graph = nullptr;
-    BCK(cudaGraphCreate(&b->graph, 0));
+    // (an empty capture: a stream that is capturing already, or cannot, is refused)
+    BCK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
+    BCK(cudaStreamEndCapture(b->stream, &b->graph));
     // no node of one group depends on another's; larger clusters first, since
     // they need several free SMs at once
     int lo = 0, hi = 0;

@@ -296,10 +296,12 @@ __global__ void __launch_bounds__(MODE == R_SINGLE ? 1024 : 768, 1) k_resident2d
   }
 }
 
-// Where a launch goes: a.stream, or a node of `graph`.
+// Where a launch goes instead of a.stream: a node of `graph`, or nowhere, only
+// counting the clusters that fit the GPU.
 struct Target {
   cudaGraph_t graph;
   int priority;
+  int* clusters;
 };
 
 template <typename S, int COLL>
@@ -315,6 +317,14 @@ int launch_typed_resident(const ResidentArgs& a, const Target* t) {
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = (unsigned)a.shape.ctas;
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = (size_t)a.shape.smem;
+  cfg.stream = (cudaStream_t)a.stream;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (t && t->clusters) return cudaOccupancyMaxActiveClusters(t->clusters, kern, &cfg) == cudaSuccess ? 0 : -3;
   if (t) {
     ResidentArgs c = a;  // the parameters' values are copied into the node
     void* args[] = {&src, &dst, &c.flags, &c.doms, &c.order, &c.dom, &c.omega, &c.steps};
@@ -333,13 +343,6 @@ int launch_typed_resident(const ResidentArgs& a, const Target* t) {
                ? 0
                : -3;
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = (size_t)a.shape.smem;
-  cfg.stream = (cudaStream_t)a.stream;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, src, dst, a.flags, a.doms, a.order, a.dom, a.omega, a.steps) == cudaSuccess
              ? 0
              : -3;
@@ -386,8 +389,21 @@ ResidentShape resident2d_shape(int storage, int coll, int nx, int ny, bool alone
 int launch_resident2d(const ResidentArgs& a) { return launch_to(a, nullptr); }
 
 int add_resident2d_node(const ResidentArgs& a, void* graph, int priority) {
-  const Target t = {(cudaGraph_t)graph, priority};
+  const Target t = {(cudaGraph_t)graph, priority, nullptr};
   return launch_to(a, &t);
+}
+
+int resident2d_clusters(const ResidentShape& shape, int storage, int coll) {
+  ResidentArgs a = {};
+  a.n_dom = a.steps = 1;
+  a.storage = storage;
+  a.coll = coll;
+  a.shape = shape;
+  int n = 0;
+  const Target t = {nullptr, 0, &n};
+  if (launch_to(a, &t) == 0) return n;
+  cudaGetLastError();
+  return 0;
 }
 
 }  // namespace xlb

@@ -27,6 +27,9 @@ struct ResidentShape {
 // domain finishes early) or one of many (packed, so that all of them do).
 ResidentShape resident2d_shape(int storage, int coll, int nx, int ny, bool alone);
 
+// Clusters of that shape the GPU holds at once (0: it cannot launch one).
+int resident2d_clusters(const ResidentShape& shape, int storage, int coll);
+
 struct ResidentArgs {
   const void* src;        // post-collision populations (stored deviations)
   void* dst;              // the same after `steps` updates (may be src)
