@@ -79,17 +79,17 @@ __device__ __forceinline__ bool cell_of_grid(const StepParams& p, CellIdx& c) {
   return true;
 }
 
-// Blocks per SM the forward kernels are compiled for (register budget).
+// Blocks per SM the forward kernels are compiled for (register budget).  KBC is
+// bound by the latency of its ~1000 instructions a cell; 512 x 256 x 256 sphere,
+// k MLUPS for 5 / 6 / 7 / 8 blocks (96 / 80 / 72 / 64 registers): FP32 25.1 /
+// 26.7 / 27.4 / 28.3, FP16 27.2 / 28.9 / 30.0 / 29.3, BF16 23.9 / 24.1 / 24.8 / 23.3.
 #ifndef XLB_MINB_Q19_16
 #define XLB_MINB_Q19_16 9
-#endif
-#ifndef XLB_MINB_KBC
-#define XLB_MINB_KBC 6
 #endif
 template <int Q, typename S, int COLL>
 struct MinBlocks {
   static constexpr int value =
-      (COLL == 2) ? XLB_MINB_KBC : (Q == 27 ? 8 : (Q == 19 ? (sizeof(S) == 2 ? XLB_MINB_Q19_16 : 9) : 12));
+      (COLL == 2) ? (sizeof(S) == 4 ? 8 : 7) : (Q == 27 ? 8 : (Q == 19 ? (sizeof(S) == 2 ? XLB_MINB_Q19_16 : 9) : 12));
 };
 
 // Face types, per axis, of the coordinates v - 1, v and v + 1 (periodic) of

@@ -38,6 +38,7 @@ __device__ __forceinline__ F2 vset<F2>(float x) {
 
 __device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float vneg(float a) { return -a; }  // (a modifier of the operand that uses it)
 __device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ float vrcp(float a) { return 1.0f / a; }
@@ -59,6 +60,7 @@ __device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c) {
 }
 // a - b = fma(b, -1, a): one rounding, like the subtraction
 __device__ __forceinline__ F2 vsub(F2 a, F2 b) { return vfma(b, pack2(-1.0f, -1.0f), a); }
+__device__ __forceinline__ F2 vneg(F2 a) { return vmul(a, pack2(-1.0f, -1.0f)); }
 __device__ __forceinline__ F2 vrcp(F2 a) {
   float x, y;
   unpack2(a, x, y);
@@ -73,22 +75,17 @@ __device__ __forceinline__ F2 vdiv_fast(F2 a, F2 b) {
   unpack2(b, z, w);
   return pack2(__fdividef(x, z), __fdividef(y, w));
 }
-__device__ __forceinline__ float vdiv(float a, float b) { return __fdiv_rn(a, b); }
-__device__ __forceinline__ F2 vdiv(F2 a, F2 b) {
-  float x, y, z, w;
-  unpack2(a, x, y);
-  unpack2(b, z, w);
-  return pack2(__fdiv_rn(x, z), __fdiv_rn(y, w));
+// b < lim ? x : c - a / b per lane; no division where none is used
+__device__ __forceinline__ float vsub_div_unless_less(float x, float c, float a, float b, float lim) {
+  return b < lim ? x : __fsub_rn(c, __fdiv_rn(a, b));
 }
-// a < b ? x : y per lane
-__device__ __forceinline__ float vless(float a, float b, float x, float y) { return a < b ? x : y; }
-__device__ __forceinline__ F2 vless(F2 a, F2 b, F2 x, F2 y) {
-  float a0, a1, b0, b1, x0, x1, y0, y1;
+__device__ __forceinline__ F2 vsub_div_unless_less(F2 x, float c, F2 a, F2 b, F2 lim) {
+  float x0, x1, a0, a1, b0, b1, l0, l1;
+  unpack2(x, x0, x1);
   unpack2(a, a0, a1);
   unpack2(b, b0, b1);
-  unpack2(x, x0, x1);
-  unpack2(y, y0, y1);
-  return pack2(a0 < b0 ? x0 : y0, a1 < b1 ? x1 : y1);
+  unpack2(lim, l0, l1);
+  return pack2(vsub_div_unless_less(x0, c, a0, b0, l0), vsub_div_unless_less(x1, c, a1, b1, l1));
 }
 
 }  // namespace xlb

@@ -420,7 +420,7 @@ __device__ __forceinline__ void add_force(T (&df)[Q], T rho, T ir, const T (&u)[
   for (int i = 1; i < Q; ++i) {
     if (opposite<Q>(i) > i) {
       const T cu = vdot<Q>(i, u), cv = vdot<Q>(i, v);
-      const T e = vfma(vset<T>(4.5f), vfma(cv, cv, vmul(vmul(cu, vset<T>(-1.0f)), cu)), dsq), o = vsub(cv, cu);
+      const T e = vfma(vset<T>(4.5f), vfma(cv, cv, vmul(vneg(cu), cu)), dsq), o = vsub(cv, cu);
       const T wr = vmul(vset<T>(weight<Q>(i)), rho);
       df[i] = vfma(wr, vfma(vset<T>(3.0f), o, e), df[i]);
       df[opposite<Q>(i)] = vfma(wr, vfma(vset<T>(-3.0f), o, e), df[opposite<Q>(i)]);
@@ -456,7 +456,7 @@ __device__ __forceinline__ void collide_bgk(T (&df)[Q], const StepParams& p) {
   // df + omega (w x - df) as df - omega (df - w x), the same value
   const T nom = vset<T>(-p.omega);
   df[0] = vfma(nom, vfma(vset<T>(-weight<Q>(0)), vfma(rho, b0, drho), df[0]), df[0]);
-  const T r3 = vmul(rho, vset<T>(3.0f)), n3 = vmul(rho, vset<T>(-3.0f));
+  const T r3 = vmul(rho, vset<T>(3.0f)), n3 = vneg(r3);
 #pragma unroll
   for (int i = 1; i < Q; ++i) {
     if (opposite<Q>(i) > i) {
@@ -500,7 +500,6 @@ __device__ __forceinline__ T kbc_ds(int i, const T (&hd)[3], const T (&qo)[3], c
 template <int Q, typename T>
 __device__ __forceinline__ void collide_kbc(T (&df)[Q], const StepParams& p) {
   constexpr int D = Lattice<Q>::D;
-  const T mone = vset<T>(-1.0f);
   T drho, j[3], M[6];
   moments_kbc<Q>(df, drho, j, M);
   const T rho = vadd(vset<T>(1.0f), drho), ir = vrcp(rho);
@@ -509,7 +508,7 @@ __device__ __forceinline__ void collide_kbc(T (&df)[Q], const StepParams& p) {
   for (int a = 0; a < D; ++a) u[a] = vmul(j[a], ir);
   const T usq = vnorm2<Q>(u);
   const T b0 = vmul(vset<T>(-1.5f), usq);  // b of the rest direction (c = 0)
-  const T nrho = vmul(rho, mone);
+  const T nrho = vneg(rho);
   T nru[3], P[3], S;
 #pragma unroll
   for (int a = 0; a < D; ++a) {
@@ -524,7 +523,7 @@ __device__ __forceinline__ void collide_kbc(T (&df)[Q], const StepParams& p) {
   for (int k = 0; k < (D == 3 ? 3 : 1); ++k) {
     const int a = k == 2 ? 1 : 0, b = k == 0 ? 1 : 2;
     qo[k] = vmul(vset<T>(0.25f), vfma(nru[a], u[b], M[3 + k]));
-    nqo[k] = vmul(qo[k], mone);
+    nqo[k] = vneg(qo[k]);
   }
   // <a|b> = sum a_i b_i / f_i^eq with f_i^eq = w_i rho (1 + b +- a); the
   // common 1/rho cancels in gamma, and one reciprocal serves a pair:
@@ -545,7 +544,7 @@ __device__ __forceinline__ void collide_kbc(T (&df)[Q], const StepParams& p) {
       df[i] = fi;
       df[k] = fk;
       const T X = vadd(vset<T>(1.0f), bq);
-      const T rc = vdiv_fast(vset<T>(1.0f / weight<Q>(i)), vfma(X, X, vmul(vmul(a3, mone), a3)));
+      const T rc = vdiv_fast(vset<T>(1.0f / weight<Q>(i)), vfma(X, X, vmul(vneg(a3), a3)));
       const T ri = vmul(vsub(X, a3), rc), rk = vmul(vadd(X, a3), rc);
       T hi = fi, hk = fk;
       if (nnz<Q>(i) < 3) {
@@ -558,12 +557,13 @@ __device__ __forceinline__ void collide_kbc(T (&df)[Q], const StepParams& p) {
     }
   }
   const float beta = 0.5f * p.omega, ib = 1.0f / beta;
-  const T g = vsub(vset<T>(ib), vdiv(vmul(vset<T>(2.0f - ib), sh), hh));
-  const T gamma = vless(hh, vmul(vset<T>(1e-20f), rho), vset<T>(2.0f), g);
+  // (a uniform stream takes no division: 0 / 0 would cost it 6% of the update)
+  const T gamma = vsub_div_unless_less(vset<T>(2.0f), ib, vmul(vset<T>(2.0f - ib), sh), hh,
+                                       vmul(vset<T>(1e-20f), rho));
   const T a1 = vfma(vset<T>(-beta), gamma, vset<T>(1.0f));
   const T na2 = vmul(vset<T>(-beta), vsub(vset<T>(2.0f), gamma));
   df[0] = vfma(a1, df[0], e0);
-  const T r3 = vmul(rho, vset<T>(3.0f)), n3 = vmul(rho, vset<T>(-3.0f));
+  const T r3 = vmul(rho, vset<T>(3.0f)), n3 = vneg(r3);
 #pragma unroll
   for (int i = 1; i < Q; ++i) {
     if (opposite<Q>(i) > i) {
