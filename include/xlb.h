@@ -133,10 +133,13 @@ int xlb_set_mask(xlb_ctx* ctx, const uint8_t* mask);
  * cells of FWALL face planes and the cells of those inlet / outlet planes,
  * whose source cell is WALL, LID or EQ off the face planes; n_fix = number
  * of the other INLET and OUTLET cells plus the FWALL cells off the face
- * planes.  After each update a boundary pass writes, for every link, the
- * value the rule prescribes into the source cell's slot for that direction
- * (a ghost value, so the next update can pull every cell as if periodic)
- * and stores the fix-up cells, recomputed beside the bulk pass. */
+ * planes.  A boundary pass writes, for every link, the value the rule
+ * prescribes into the source cell's slot for that direction (a ghost value,
+ * so the next update can pull every cell as if periodic) and stores the
+ * fix-up cells, recomputed beside the bulk pass.  It follows each update,
+ * or only the last of a call where the updates apply the rules themselves
+ * (several D2Q9 updates in one launch; 16-bit storage whose only links lie
+ * on the x-faces). */
 int xlb_boundary_links(const xlb_ctx* ctx, int64_t* n_links, int64_t* n_fix);
 
 /* Zou-He inlet velocity per cell (a velocity profile, e.g. the Poiseuille
@@ -230,7 +233,9 @@ int xlb_step(xlb_ctx* ctx, int64_t n);
  * first use and captured again after any change of the mask, boundary
  * values, force or kernel variant; the first update after xlb_init and any
  * remainder of fewer than g updates are launched directly.  g = 0 (the
- * default) launches every update.  Results are identical either way.  The
+ * default) launches every update, or several D2Q9 updates at a time.  A
+ * small D2Q9 lattice that runs as one launch for all the updates of a call
+ * does so whatever g.  Results are identical either way.  The
  * capture needs the ctx stream idle and not capturing, with no other thread
  * queuing work on it during xlb_step; graphs are not used while a tape is
  * open or profiling is on.  XLB_ERR_ARG for g outside [0, 100000]. */
@@ -364,10 +369,10 @@ int xlb_tape_release(xlb_ctx* ctx);
  *   XLB_KERNEL_VEC2:   the same with 2 cells per thread and 32-bit words
  *     (nx even);
  *   XLB_KERNEL_AUTO:   the default, the fastest measured: FP16 runs VEC on
- *     lattices without boundary planes and VEC2 with them (D3Q19: VEC from 8 M
+ *     lattices without boundary planes and VEC2 with them (D3Q19: VEC from 3 M
  *     cells, DIRECT between 16,384 and 3 M cells where the x-faces are the
- *     only links), BF16 DIRECT (VEC on D3Q19 lattices of 500,000 cells or more
- *     without boundary planes), FP32 DIRECT.
+ *     only links), BF16 DIRECT (D3Q19: VEC from 100,000 cells without boundary
+ *     planes, from 8 M with them), FP32 DIRECT.
  * A mask with an FWALL face plane always runs DIRECT. */
 enum { XLB_KERNEL_AUTO = 0, XLB_KERNEL_DIRECT = 1, XLB_KERNEL_VEC = 2, XLB_KERNEL_VEC2 = 3 };
 
@@ -400,23 +405,26 @@ int xlb_batch_set_masks(xlb_batch* b, const uint8_t* masks, const float* forces)
  * interleaved u_x, u_y) concatenated like the masks, or NULL (1 and 0). */
 int xlb_batch_init(xlb_batch* b, const float* rho, const float* u);
 
-/* Advance every domain n steps in one persistent launch: each CTA takes
- * domains from a queue, largest first, and runs all n steps of one domain
- * before the next.  The launch is captured in a CUDA graph on first use and
- * replayed while n and the launch shape stay the same. */
+/* Advance every domain n steps in one graph launch: domains that fit the
+ * shared memory of a thread-block cluster stay there for all n steps (n >= 8);
+ * for the others, and for fewer steps, each CTA takes domains from a queue,
+ * largest first, and runs all n steps of one domain before the next.  The
+ * graph is built on first use and replayed while n and the launch shape stay
+ * the same; XLB_ERR_CUDA on a stream that is capturing. */
 int xlb_batch_step(xlb_batch* b, int64_t n);
 
 /* The same n steps with one ordinary launch per domain and step (the
  * baseline the persistent launch replaces). */
 int xlb_batch_step_per_domain(xlb_batch* b, int64_t n);
 
-/* Launch shape of xlb_batch_step: threads per CTA (32..1024, a multiple of
+/* Launch shape of xlb_batch_step's queue: threads per CTA (32..1024, a multiple of
  * 32) and resident CTAs per SM (1..32, capped by occupancy). */
 int xlb_batch_set_launch(xlb_batch* b, int threads, int ctas_per_sm);
 
-/* Autotuner: time every candidate shape over sample_steps updates on a saved
- * copy of the state (restored afterwards), keep the fastest, append it to the
- * cache file (NULL: no cache; a matching line skips the timing). */
+/* Autotuner of the queue: time every candidate shape over sample_steps updates
+ * of all the domains on a saved copy of the state (restored afterwards), keep
+ * the fastest, append it to the cache file (NULL: no cache; a matching line
+ * skips the timing). */
 int xlb_batch_tune(xlb_batch* b, int sample_steps, const char* cache_path, int* best_threads, int* best_ctas);
 
 /* rho (total cells) and u (2 per cell) of every domain's post-stream state;

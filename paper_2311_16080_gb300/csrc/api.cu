@@ -3,13 +3,17 @@
 // State machine of a ctx:
 //  - xlb_init writes f_0 (post-stream populations) and marks the buffer as
 //    "pre-collision" (kind_h = 0).  The first step after that is a local
-//    collision (h_0 = C(f_0)); every later step is one fused stream-collide
-//    launch h_t = C(S_bc(h_{t-1})).  The stored buffer after t steps is
+//    collision (h_0 = C(f_0), formed from the initial fields while they still
+//    describe the state); every later step is a fused stream-collide update
+//    h_t = C(S_bc(h_{t-1})): a launch each, or several in one launch of the
+//    resident or the tiled D2Q9 kernel.  The stored buffer after t steps is
 //    h_{t-1}, and the observables of f_t = S_bc(h_{t-1}) are computed by a pull
 //    inside the readout kernels.  (S_bc C)^n = S_bc (C S_bc)^(n-1) C, so this is
 //    the same sequence of operations as Eqs. 1-2 applied n times.
 //  - A tape records h_{sk-1} at every time sk < T; the adjoint recomputes one
-//    segment of k states from its checkpoint before walking it backwards.
+//    segment of k states from its checkpoint before walking it backwards.  The
+//    states of the last segment stay in the tape slots as the forward pass
+//    takes them.
 #include <cuda_runtime.h>
 #include <stdarg.h>
 #include <stdio.h>
@@ -306,12 +310,13 @@ static bool has_fwall_face(const xlb_ctx* c) {
 // The bulk variant an update launches: the requested one where it can run
 // this ctx, and for AUTO the fastest measured on D3Q19 lattices (us per update,
 // one / two / four cells per thread):
-//   FP16 without boundary planes   256^3 253 / 232 / 223, 64^3 5.4 / 5.0 / 4.9
-//   FP16 cavity                    256^3 289 / 263 / 259, 160^3 74 / 73 / 74,
-//                                  132 x 100 x 90 23 / 25 / 27, 64^3 8 / 12 / 13
-//   BF16 without boundary planes   256^3 297 / 312 / 292, 160^3 82 / 80 / 76,
-//                                  64^3 6.2 / 6.6 / 6.8
-//   BF16 cavity                    one cell throughout; FP32 too.
+//   FP16 without boundary planes   256^3 249 / 221 / 194, 64^3 5.4 / 4.6 / 4.3
+//   FP16 cavity                    256^3 275 / 257 / 231, 160^3 73 / 72 / 67,
+//                                  128^3 37 / 40 / 40, 64^3 8 / 13 / 13
+//   BF16 without boundary planes   256^3 302 / 303 / 262, 160^3 80 / 79 / 69,
+//                                  64^3 6.2 / 6.4 / 5.9
+//   BF16 cavity                    256^3 324 / 344 / 314, 160^3 87 / 95 / 94
+//   FP32                           one cell throughout.
 // One cell per thread gains on the cavities because it serves the x-faces
 // itself (x_pull) and then needs no boundary pass; lattices of a few thousand
 // cells, where launches decide, keep two.  Masks with FWALL faces always run
@@ -325,10 +330,10 @@ static int bulk_variant(const xlb_ctx* c) {
   for (int f = 0; f < 6; ++f) faces |= c->face[f] != 0;
   if (c->has_mask && c->n_links > 0) faces = true;  // boundary planes served by ghost links
   if (c->storage == XLB_STORE_BF16)
-    return !faces && c->Q == 19 && c->N >= 500000 && vec_possible(c, 4) ? XLB_KERNEL_VEC : XLB_KERNEL_DIRECT;
+    return c->Q == 19 && c->N >= (faces ? 8000000 : 100000) && vec_possible(c, 4) ? XLB_KERNEL_VEC : XLB_KERNEL_DIRECT;
   if (!faces && vec_possible(c, 4)) return XLB_KERNEL_VEC;
   if (faces && c->Q == 19) {
-    if (c->N >= 8000000 && vec_possible(c, 4)) return XLB_KERNEL_VEC;
+    if (c->N >= 3000000 && vec_possible(c, 4)) return XLB_KERNEL_VEC;
     if (c->x_pull && c->N >= 16384 && c->N < 3000000) return XLB_KERNEL_DIRECT;
   }
   if (vec_possible(c, 2)) return XLB_KERNEL_VEC2;

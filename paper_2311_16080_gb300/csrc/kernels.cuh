@@ -622,9 +622,13 @@ __global__ void __launch_bounds__(ROW_BLOCK) k_fix_recompute(const S* __restrict
 // box).  Stores are V-wide.  Needs
 // nx % V == 0; no FWALL faces.
 
+// Blocks per SM (register budget).  The kernel waits for its loads (V = 4) or
+// issues (V = 2): a 256^3 FP16 D3Q19 periodic box, k MLUPS, for 2 / 3 / 4 / 5 / 6
+// blocks of V = 4: 76.5 / 75.2 / 86.3 / 72.3 / 54.3 (from 5 on it spills); for
+// 5 / 6 / 7 / 8 / 9 of V = 2: 68.3 / 71.8 / 75.9 / 71.9 / 65.7.
 template <int Q, typename S, int COLL, int V>
 struct VecMinBlocks {
-  static constexpr int value = (COLL == 2) ? 5 : (Q * V > 64 ? 3 : (Q * V > 32 ? 6 : 8));
+  static constexpr int value = COLL == 2 ? 5 : Q == 19 ? (V == 4 ? 4 : 7) : (V == 4 ? 6 : 8);
 };
 
 template <int Q, typename S, int COLL, int V>
