@@ -2,11 +2,14 @@
 // simulations advanced together).  Thousands of D2Q9 domains of different
 // sizes, each periodic in x and y unless its mask says otherwise, with WALL
 // cells (halfway bounce-back) and a per-domain body force, advance in one
-// persistent launch: every CTA takes domains from an atomic queue (largest
-// first) and runs all requested steps of a domain before taking the next,
-// with a CTA barrier between steps.  A domain's state therefore stays in the
-// caches of one SM while it is being advanced.  The launch and its queue
-// reset are captured in a CUDA graph and replayed.
+// graph launch.  For 8 steps or more a domain whose populations fit the shared
+// memory of a cluster runs on the resident kernel, grouped with the domains of
+// the same cluster size and footprint (12.0 M cells in 1024 domains, 500 steps:
+// 76.1 ms on the queue alone, 40.7 ms resident).  The others, and all of them
+// for fewer steps, are taken by persistent CTAs from an atomic queue (largest
+// first), which run all requested steps of a domain before the next, with a
+// CTA barrier between steps.  The graph (one node per group, the queue's reset
+// and launch) is kept while the step count and the launch shape stay the same.
 //
 // Per domain: populations f[i][y][x] (deviations f_i - w_i, like the single
 // lattice) in two buffers, a flag byte per cell (type | FLAG_SLOW when a WALL
