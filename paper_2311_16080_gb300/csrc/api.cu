@@ -1058,7 +1058,12 @@ int xlb_set_wall_distances(xlb_ctx* c, int64_t n, const int64_t* cell, const int
   ++c->epoch;
   if (n > 0) CK(cudaMalloc(&c->link_q, sizeof(float) * hq.size()));
   if (n > 0) CK(cudaMemcpy(c->link_q, hq.data(), sizeof(float) * hq.size(), cudaMemcpyHostToDevice));
-  if (n > 0 && c->Q == 9) {
+  // The tiled kernel updates the outlet column by itself, without the rows of
+  // a cell with Bouzidi links: no tables, and so no tiles, where an OUTLET cell
+  // owns such a link (a body that reaches the column before it).
+  bool outlet_link = false;
+  for (int64_t k = 0; k < n && c->x_outlet; ++k) outlet_link |= cell[k] % c->nx == c->nx - 1;
+  if (n > 0 && c->Q == 9 && !outlet_link) {
     // the same by cell, for the tiled kernel (which is not used without them:
     // no memory for them is no error)
     std::vector<uint8_t> fl((size_t)c->N);

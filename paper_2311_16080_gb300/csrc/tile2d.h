@@ -26,7 +26,9 @@ struct Tile2dArgs {
   int storage, coll;
   const void* src;       // post-collision populations
   void* dst;             // the same `steps` updates later (another buffer)
-  const int* bz;         // per cell 0 or 1 + its row in bz_q (rows < 65535), or null
+  // per cell 0 or 1 + its row in bz_q (rows < 65535), or null; 0 for OUTLET
+  // cells, which the kernel updates without a row
+  const int* bz;
   // 9 pairs per row.  Pair i of a link in direction i with wall distance q:
   // {2q, 1 - 2q} or {1/(2q), 1 - 1/(2q)} (q >= 1/2); {1, 0}, the halfway rule as
   // q = 1/2, for a distance below 1/2 where the cell behind is not FLUID.  Pair
