@@ -69,6 +69,7 @@ struct xlb_ctx {
   int inlet_axis = 0, inlet_sign = 1;  // inward normal of the INLET boundary
   bool has_inlet_outlet = false;  // INLET, OUTLET or FWALL cells (no adjoint)
   bool has_lid_eq = false;        // LID or EQ cells
+  bool outlet_walled = false;     // an OUTLET cell whose neighbour at x - 1 is a WALL cell
   float* init_fields = nullptr;  // (1 + D) * N: rho0, u0 (component-major)
   bool has_init = false;
   uint64_t init_epoch = 0;  // buf[cur] is f_0 of init_fields under this epoch's parameters (0: it is not)
@@ -774,7 +775,7 @@ int xlb_set_mask(xlb_ctx* c, const uint8_t* mask) {
     dmask = (uint8_t*)mask;
   }
   uint8_t* nf = nullptr;
-  bool new_io = false, new_le = false, new_x_inlet = false, new_x_outlet = false;
+  bool new_io = false, new_le = false, new_ow = false, new_x_inlet = false, new_x_outlet = false;
   int new_face[6] = {0, 0, 0, 0, 0, 0};
   CK(cudaMalloc(&nf, n));
   CK(cudaMemsetAsync(c->err_word, 0, sizeof(int), c->stream));
@@ -819,6 +820,7 @@ int xlb_set_mask(xlb_ctx* c, const uint8_t* mask) {
     }
     new_io = (hw[2] & 1) != 0;
     new_le = (hw[2] & 2) != 0;
+    new_ow = (hw[2] & 4) != 0;
     detect_faces(pl, c->nx, c->ny, c->nz, new_face);
     bool fw_face = false;  // (the bulk instance for FWALL faces has no inflow / outflow planes)
     for (int f = 0; f < 6; ++f) fw_face |= new_face[f] == XLB_CELL_FWALL;
@@ -940,6 +942,7 @@ int xlb_set_mask(xlb_ctx* c, const uint8_t* mask) {
   c->n_fix = nfx;
   c->has_inlet_outlet = new_io;
   c->has_lid_eq = new_le;
+  c->outlet_walled = new_ow;
   for (int f = 0; f < 6; ++f) c->face[f] = new_face[f];
   c->x_linked = new_x_linked;
   c->x_pull = new_x_pull;
@@ -1235,10 +1238,12 @@ static double single_update_us(const xlb_ctx* c) {
 }
 
 // Whether the tiled D2Q9 kernel may take this ctx's updates: FLUID and WALL
-// cells, inflow and outflow planes together (the lattice then ends at them),
+// cells, inflow and outflow planes together (the lattice then ends at them; the
+// cells before an OUTLET cell hand it what they pull, so they must not be WALL),
 // Bouzidi links.
 static bool tile_ok(xlb_ctx* c) {
   if (c->Q != 9 || c->coll == XLB_COLL_NONE || c->has_lid_eq || c->n_fix > 0 || has_fwall_face(c)) return false;
+  if (c->outlet_walled) return false;
   if (c->x_inlet != c->x_outlet || (c->x_inlet && (c->inlet_axis != 0 || c->inlet_sign != 1))) return false;
   if (c->link_q && !c->bz) return false;
   if (c->tile.halo < 0) c->tile = tile2d_plan(c->storage, c->coll, (int)c->nx, (int)c->ny);

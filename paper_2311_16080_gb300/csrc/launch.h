@@ -67,7 +67,8 @@ long long cell_blocks(const StepParams& p);
 
 // Mask preparation: validates codes (< 7), writes flag bytes; err_word[0] is
 // set to 1 on an invalid code, bit 0 of err_word[2] where an INLET, OUTLET or
-// FWALL cell occurs, bit 1 where a LID or EQ cell does.  Q picks the stencil used for the FLAG_SLOW test.
+// FWALL cell occurs, bit 1 where a LID or EQ cell does, bit 2 where an OUTLET
+// cell has a WALL cell at x - 1.  Q picks the stencil used for the FLAG_SLOW test.
 int launch_mask_prepare(int Q, const uint8_t* mask, uint8_t* flags, int nx, int ny, int nz, int* err_word,
                         void* stream);
 // The six boundary planes of a device mask into `out` (compact, plane by

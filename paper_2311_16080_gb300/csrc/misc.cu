@@ -34,7 +34,7 @@ __device__ __forceinline__ void cell_xyz(long long cell, int nx, int ny, bool sm
 // flags = type | FLAG_SLOW where a fluid-like cell has a WALL / LID / EQ cell
 // in its Q-stencil, or is an INLET / OUTLET / FWALL cell.  Codes >= 7 set
 // err[0]; an INLET, OUTLET or FWALL cell anywhere sets bit 0 of err[2], a LID
-// or EQ cell bit 1.
+// or EQ cell bit 1, an OUTLET cell beside a WALL cell at x - 1 bit 2.
 template <int Q>
 __global__ void k_mask_prepare(const uint8_t* __restrict__ mask, uint8_t* __restrict__ flags, int nx, int ny,
                                int nz, int* err) {
@@ -63,6 +63,7 @@ __global__ void k_mask_prepare(const uint8_t* __restrict__ mask, uint8_t* __rest
       }
       int slow = (t == INLET || t == OUTLET || t == FWALL);
       seen |= slow | (t == LID || t == EQ ? 2 : 0);
+      if (t == OUTLET && x > 0 && mask[cell - 1] == WALL) seen |= 4;
       if (fluid_like(t) && !slow) {
         const int xs[3] = {x == 0 ? nx - 1 : x - 1, x, x == nx - 1 ? 0 : x + 1};
 #pragma unroll

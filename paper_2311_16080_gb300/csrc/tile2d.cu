@@ -15,8 +15,9 @@
 //     q <  1/2: f_j = 2q h_i(x) + (1 - 2q) f_i(x) when x pulls;
 //     q >= 1/2: h_i(x) / (2q) + (1 - 1/(2q)) h_j(x) is formed when x collides
 //               and left in the slot that x will read;
-//   OUTLET: the cell x - 1 leaves the populations it pulls with c_x = -1 in a
-//   stash, and the outlet column is updated after a barrier of its own.
+//   OUTLET: the cell x - 1 (no WALL cell) leaves the populations it pulls with
+//   c_x = -1 in a stash, and the outlet column is updated after a barrier of its
+//   own.
 #include <cuda_runtime.h>
 
 #include <type_traits>

@@ -78,3 +78,24 @@ def test_wall_distances_of_outlet_cells(storage):
     assert _links(m, O.OUTLET)
     a, b = _sims(m, storage, links)
     _compare(a, b, m)
+
+
+@pytest.mark.parametrize("storage", STORAGES)
+@pytest.mark.parametrize("body", [lambda x, y: (x >= 410) & (abs(y - 75) <= 3),  # a plate that ends at the outlet
+                                  lambda x, y: (y <= 1) | (y >= 148),           # walls two cells thick
+                                  lambda x, y: (x == 418) & (y == 40)],         # one cell
+                         ids=["plate", "thick", "cell"])
+def test_wall_before_the_outlet(body, storage):
+    """An OUTLET cell whose neighbour at x - 1 is a WALL cell."""
+    m = _channel(body)
+    a, b = _sims(m, storage)
+    _compare(a, b, m)
+
+
+@pytest.mark.parametrize("storage", STORAGES)
+def test_body_one_cell_off_the_outlet(storage):
+    """The nearest body that leaves the OUTLET plane's neighbours FLUID."""
+    m = _channel(lambda x, y: (x >= 410) & (x <= 417) & (abs(y - 75) <= 3))
+    links = _links(m, O.FLUID)
+    a, b = _sims(m, storage, links)
+    _compare(a, b, m)
