@@ -139,7 +139,7 @@ int xlb_set_mask(xlb_ctx* ctx, const uint8_t* mask);
  * fix-up cells, recomputed beside the bulk pass.  It follows each update,
  * or only the last of a call where the updates apply the rules themselves
  * (several D2Q9 updates in one launch; 16-bit storage whose only links lie
- * on the x-faces). */
+ * on the x-faces and carry no wall distances). */
 int xlb_boundary_links(const xlb_ctx* ctx, int64_t* n_links, int64_t* n_fix);
 
 /* Zou-He inlet velocity per cell (a velocity profile, e.g. the Poiseuille
@@ -186,9 +186,10 @@ int xlb_set_inlet_normal(xlb_ctx* ctx, int axis, int sign);
  * Unlisted WALL links keep halfway bounce-back (q = 1/2).  Arrays are host
  * memory; the list replaces any earlier one (n = 0 clears it) and acts from
  * the next step on; a new mask clears it.  XLB_ERR_ARG (nothing changed) if
- * a link is not a ghost link of the mask (the cell is not FLUID, the
- * neighbour is not WALL, or the neighbour lies on a boundary face plane) or
- * a q is outside [0, 1]; XLB_ERR_STATE before a mask or while a tape is open. */
+ * a link is not a ghost link of the mask (the neighbour is not WALL, the cell
+ * owns no links, or the neighbour lies on a boundary face plane that is handled
+ * by coordinates: with 16-bit storage the x-face planes have links and take
+ * distances) or a q is outside [0, 1]; XLB_ERR_STATE before a mask or while a tape is open. */
 int xlb_set_wall_distances(xlb_ctx* ctx, int64_t n, const int64_t* cell, const int32_t* dir, const float* q);
 
 /* Momentum-exchange force on the WALL cells off the boundary faces (Mei et
@@ -371,7 +372,7 @@ int xlb_tape_release(xlb_ctx* ctx);
  *   XLB_KERNEL_AUTO:   the default, the fastest measured: FP16 runs VEC on
  *     lattices without boundary planes and VEC2 with them (D3Q19: VEC from 3 M
  *     cells, DIRECT between 16,384 and 3 M cells where the x-faces are the
- *     only links), BF16 DIRECT (D3Q19: VEC from 100,000 cells without boundary
+ *     only links and carry no wall distances), BF16 DIRECT (D3Q19: VEC from 100,000 cells without boundary
  *     planes, from 8 M with them), FP32 DIRECT.
  * A mask with an FWALL face plane always runs DIRECT. */
 enum { XLB_KERNEL_AUTO = 0, XLB_KERNEL_DIRECT = 1, XLB_KERNEL_VEC = 2, XLB_KERNEL_VEC2 = 3 };

@@ -60,7 +60,7 @@ struct xlb_ctx {
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int face[6] = {0, 0, 0, 0, 0, 0};  // described boundary faces (StepParams::face)
   bool x_linked = false;             // the x-faces' sources are served by ghost links
-  bool x_pull = false;               // ... which are the only ones: one cell per thread serves them itself
+  bool x_pull = false;               // ... which are the only ones (pulls_x_faces)
   bool x_inlet = false;              // the x = 0 plane is INLET, served by the bulk pass
   bool x_outlet = false;             // the x = nx - 1 plane is OUTLET, served by the bulk pass
   float* link_q = nullptr;  // Bouzidi wall distance per link (LINK_BZ entries), or null
@@ -308,6 +308,11 @@ static bool has_fwall_face(const xlb_ctx* c) {
   return false;
 }
 
+// Whether the bulk pass with one cell per thread serves the x-faces itself and
+// needs no boundary pass.  Not while links carry wall distances: a WALL x-face's
+// links may, and only the boundary pass knows which.
+static bool pulls_x_faces(const xlb_ctx* c) { return c->x_pull && !c->link_q; }
+
 // The bulk variant an update launches: the requested one where it can run
 // this ctx, and for AUTO the fastest measured on D3Q19 lattices (us per update,
 // one / two / four cells per thread):
@@ -319,7 +324,7 @@ static bool has_fwall_face(const xlb_ctx* c) {
 //   BF16 cavity                    256^3 324 / 344 / 314, 160^3 87 / 95 / 94
 //   FP32                           one cell throughout.
 // One cell per thread gains on the cavities because it serves the x-faces
-// itself (x_pull) and then needs no boundary pass; lattices of a few thousand
+// itself (pulls_x_faces) and then needs no boundary pass; lattices of a few thousand
 // cells, where launches decide, keep two.  Masks with FWALL faces always run
 // one cell per thread.
 static int bulk_variant(const xlb_ctx* c) {
@@ -335,7 +340,7 @@ static int bulk_variant(const xlb_ctx* c) {
   if (!faces && vec_possible(c, 4)) return XLB_KERNEL_VEC;
   if (faces && c->Q == 19) {
     if (c->N >= 3000000 && vec_possible(c, 4)) return XLB_KERNEL_VEC;
-    if (c->x_pull && c->N >= 16384 && c->N < 3000000) return XLB_KERNEL_DIRECT;
+    if (pulls_x_faces(c) && c->N >= 16384 && c->N < 3000000) return XLB_KERNEL_DIRECT;
   }
   if (vec_possible(c, 2)) return XLB_KERNEL_VEC2;
   return XLB_KERNEL_DIRECT;
@@ -398,7 +403,7 @@ static int launch_step(xlb_ctx* c, const void* src, void* dst) {
   a.dst = dst;
   a.vec_width = bulk_variant(c) == XLB_KERNEL_VEC2 ? 2 : 4;
   a.p.has_mask = 0;  // bulk pass: every cell pulled as if periodic
-  const bool x_pull = c->x_pull && !vec;
+  const bool x_pull = pulls_x_faces(c) && !vec;
   if (x_pull) a.p.x_linked = 0;
   cudaEvent_t* pe = prof_begin(c, 0);
   const bool side = c->has_mask && c->n_fix > 0 && c->fix_side && c->aux;
@@ -430,7 +435,7 @@ static int launch_step(xlb_ctx* c, const void* src, void* dst) {
 }
 
 // The ghost values of the links alone, once per call where the updates need
-// none (x_pull with one cell per thread): the wall force and the vector
+// none (pulls_x_faces): the wall force and the vector
 // kernels read them.
 static int write_links(xlb_ctx* c, void* dst) {
   LaunchArgs a = base_args(c);
@@ -1481,7 +1486,7 @@ int xlb_step(xlb_ctx* c, int64_t n) {
     r = record_checkpoint(c);
     if (r) return r;
   }
-  if (c->x_pull && !use_vec(c) && c->kind_h && n > 0) return write_links(c, c->buf[c->cur]);
+  if (pulls_x_faces(c) && !use_vec(c) && c->kind_h && n > 0) return write_links(c, c->buf[c->cur]);
   return XLB_OK;
 }
 
