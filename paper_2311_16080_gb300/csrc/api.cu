@@ -436,7 +436,7 @@ static int launch_step(xlb_ctx* c, const void* src, void* dst) {
 
 // The ghost values of the links alone, once per call where the updates need
 // none (pulls_x_faces): the wall force and the vector
-// kernels read them.
+// kernels read them (those that replay a tape's checkpoints among them).
 static int write_links(xlb_ctx* c, void* dst) {
   LaunchArgs a = base_args(c);
   a.src = dst;
@@ -1877,6 +1877,12 @@ static int load_segment(xlb_ctx* c, int64_t s) {
     j0 = 2;
   } else {
     CK(cudaMemcpyAsync(c->slots[0], c->ckpt[s - 1], state_bytes_raw(c), cudaMemcpyDeviceToDevice, c->stream));
+    // a checkpoint recorded within a call of updates that need no links has
+    // none; the vector kernels (xlb_set_kernel since then) read them
+    if (pulls_x_faces(c) && use_vec(c)) {
+      r = write_links(c, c->slots[0]);
+      if (r) return r;
+    }
     j0 = 1;
   }
   for (int64_t j = j0; j <= jmax; ++j) {
