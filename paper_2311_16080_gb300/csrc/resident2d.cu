@@ -15,6 +15,11 @@
 namespace xlb {
 namespace {
 
+// Dynamic shared memory a block may take.  The kernels are allowed all of it,
+// whatever a launch needs: that attribute belongs to the function, which other
+// threads launch with other sizes.
+constexpr int RESIDENT_SMEM = 220 * 1024;
+
 // meta word of a cell: bits 0-7: x + c_j is a WALL cell (j = 1..8)
 constexpr int M_SOLID = 1 << 8;                       // the cell itself is a WALL cell
 constexpr int M_XL = 1 << 9, M_XR = 1 << 10;          // x = 0 / x = nx - 1
@@ -307,7 +312,7 @@ struct Target {
 template <typename S, int COLL>
 int launch_typed_resident(const ResidentArgs& a, const Target* t) {
   auto kern = a.shape.one ? k_resident2d<S, COLL, R_SINGLE> : k_resident2d<S, COLL, R_LOOP>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a.shape.smem) != cudaSuccess ||
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, RESIDENT_SMEM) != cudaSuccess ||
       (a.shape.ctas > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess))
     return -3;
   const S* src = (const S*)a.src;
@@ -373,7 +378,8 @@ ResidentShape resident2d_shape(int storage, int coll, int nx, int ny, bool alone
   const long long cell = storage == XLB_STORE_F32 ? 9 * 4 + 2 : 10 * 2;  // Slots<S>, meta included
   // many domains: two blocks per SM where eight blocks' worth of that is
   // enough, else one
-  for (long long limit = alone ? 220 * 1024 : 112 * 1024; limit <= 220 * 1024; limit += 108 * 1024)
+  constexpr long long HALF = 112 * 1024;
+  for (long long limit = alone ? RESIDENT_SMEM : HALF; limit <= RESIDENT_SMEM; limit += RESIDENT_SMEM - HALF)
     for (int ctas = alone ? 16 : 1; ctas <= (alone ? 16 : 8); ++ctas) {
       const int c = ctas > ny ? ny : ctas;
       const long long cells = (long long)((ny + c - 1) / c) * nx;
@@ -381,7 +387,7 @@ ResidentShape resident2d_shape(int storage, int coll, int nx, int ny, bool alone
       if (smem > limit) continue;
       if (cells <= 1024) return {c, (int)((cells + 31) / 32 * 32), smem, true};
       // 80 registers: 768 threads fill an SM
-      return {c, limit > 112 * 1024 ? 768 : 384, smem, false};
+      return {c, limit > HALF ? 768 : 384, smem, false};
     }
   return none;
 }
