@@ -19,12 +19,11 @@
 #include <string.h>
 
 #include <algorithm>
-#include <functional>
-#include <map>
 #include <string>
 #include <vector>
 
 #include "../../include/xlb.h"
+#include "batch_groups.h"
 #include "lbm_device.cuh"
 #include "resident2d.h"
 
@@ -284,12 +283,6 @@ __global__ void k_batch_flags(const BatchDom* __restrict__ doms, const int* __re
 
 using namespace xlb;
 
-// Domains that one launch of the resident kernel advances.
-struct Bucket {
-  ResidentShape shape;
-  int first = 0, count = 0;  // its domains in res_order
-};
-
 struct xlb_batch {
   int n = 0, storage = 0, esize = 4;
   double omega = 1.0;
@@ -340,44 +333,6 @@ static void by_storage(int storage, F&& f) {
   if (storage == XLB_STORE_F32) f(float());
   if (storage == XLB_STORE_F16) f(__half());
   if (storage == XLB_STORE_BF16) f(__nv_bfloat16());
-}
-
-// Group the domains by the launch shape they need (blocks per cluster, one or
-// two blocks per SM) and append that order to `ord`, which is largest first.
-static void group_domains(xlb_batch* b, std::vector<int>& ord) {
-  std::map<std::pair<int, int>, std::vector<int>, std::greater<std::pair<int, int>>> by;
-  std::map<std::pair<int, int>, ResidentShape> shape;
-  std::vector<int> all, rest;
-  for (int d : ord) {
-    const ResidentShape s = resident2d_shape(b->storage, COLL_BGK, b->hdoms[d].nx, b->hdoms[d].ny, false);
-    if (s.ctas == 0) {
-      rest.push_back(d);
-      continue;
-    }
-    const std::pair<int, int> key(s.ctas, !s.one && s.threads > 512);
-    by[key].push_back(d);
-    auto it = shape.find(key);
-    if (it == shape.end()) {
-      shape[key] = s;
-      continue;
-    }
-    ResidentShape& m = it->second;
-    // one cell per thread only where that serves every domain of the group
-    m.threads = m.one == s.one ? std::max(m.threads, s.threads) : (m.one ? s.threads : m.threads);
-    m.one = m.one && s.one;
-    m.smem = std::max(m.smem, s.smem);
-  }
-  for (auto& g : by) {  // larger clusters first
-    Bucket k;
-    k.shape = shape[g.first];
-    k.first = (int)all.size();
-    k.count = (int)g.second.size();
-    b->buckets.push_back(k);
-    all.insert(all.end(), g.second.begin(), g.second.end());
-  }
-  b->n_rest = (int)rest.size();
-  all.insert(all.end(), rest.begin(), rest.end());
-  ord.insert(ord.end(), all.begin(), all.end());
 }
 
 static unsigned grid_of(long long n, int t) { return (unsigned)((n + t - 1) / t); }
@@ -468,7 +423,13 @@ int xlb_batch_create(xlb_batch** out, int n_domains, const int32_t* nx, const in
   std::stable_sort(ord.begin(), ord.end(), [&](int a, int c) {
     return (long long)nx[a] * ny[a] > (long long)nx[c] * ny[c];
   });
-  group_domains(b, ord);
+  DomainGroups groups = group_domains(
+      ord,
+      [&](int d) { return resident2d_shape(storage, COLL_BGK, nx[d], ny[d], false); },
+      [&](const ResidentShape& s) { return resident2d_clusters(s, storage, COLL_BGK) >= 1; });
+  b->buckets = groups.buckets;
+  b->n_rest = groups.n_rest;
+  ord.insert(ord.end(), groups.order.begin(), groups.order.end());
   if (cudaMemcpy(b->doms, b->hdoms.data(), sizeof(BatchDom) * n_domains, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(b->order, ord.data(), sizeof(int) * ord.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(b->start, b->hstart.data(), sizeof(int) * (n_domains + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
