@@ -533,8 +533,8 @@ int xlb_batch_step(xlb_batch* b, int64_t n) {
     if (--n == 0) return XLB_OK;
   }
   // Domains that fit a cluster run on the resident kernel, the others (and
-  // all of them for a single update, which the resident kernel's load and
-  // store of the whole state would not shorten) on the queue.
+  // all of them for fewer updates than pay for the resident kernel's load and
+  // store of the whole state) on the queue.
   const bool queue = b->queue_only || n < BATCH_RESIDENT_MIN;
   const int n_queue = queue ? b->n : b->n_rest;
   const int* q_order = queue ? b->order : b->res_order + (b->n - b->n_rest);
@@ -546,7 +546,7 @@ int xlb_batch_step(xlb_batch* b, int64_t n) {
   });
   const int per_sm = std::max(1, std::min(occ, b->ctas_per_sm));
   const int grid = std::min(n_queue, per_sm * b->num_sms);
-  // (re)build the graph (queue reset and persistent launch, and one branch per
+  // (re)build the graph (queue reset and persistent launch, and one node per
   // group of resident domains) when its shape changes
   if (!b->graph_exec || b->graph_steps != (int)n || b->graph_threads != b->threads || b->graph_grid != grid ||
       b->graph_cur != b->cur || b->graph_queue != queue) {
@@ -557,11 +557,8 @@ int xlb_batch_step(xlb_batch* b, int64_t n) {
     // (an empty capture: a stream that is capturing already, or cannot, is refused)
     BCK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
     BCK(cudaStreamEndCapture(b->stream, &b->graph));
-    // no node of one group depends on another's; larger clusters first, since
-    // they need several free SMs at once
-    int lo = 0, hi = 0;
-    BCK(cudaDeviceGetStreamPriorityRange(&lo, &hi));
-    int prio = hi;
+    // no node depends on another group's; larger clusters first, since they need
+    // several free SMs at once
     if (!queue)
       for (const Bucket& k : b->buckets) {
         ResidentArgs a;
@@ -577,11 +574,10 @@ int xlb_batch_step(xlb_batch* b, int64_t n) {
         a.omega = (float)b->omega;
         a.steps = (int)n;
         a.shape = k.shape;
-        if (add_resident2d_node(a, b->graph, prio) != 0) {
+        if (add_resident2d_node(a, b->graph) != 0) {
           cudaGetLastError();
           return bfail(b, XLB_ERR_CUDA, "resident kernel rejected");
         }
-        if (prio < lo) ++prio;
       }
     if (n_queue > 0) {
       cudaGraphNode_t reset, node;

@@ -305,7 +305,6 @@ __global__ void __launch_bounds__(MODE == R_SINGLE ? 1024 : 768, 1) k_resident2d
 // counting the clusters that fit the GPU.
 struct Target {
   cudaGraph_t graph;
-  int priority;
   int* clusters;
 };
 
@@ -340,11 +339,8 @@ int launch_typed_resident(const ResidentArgs& a, const Target* t) {
     kp.sharedMemBytes = (unsigned)a.shape.smem;
     kp.kernelParams = args;
     cudaGraphNode_t node;
-    cudaLaunchAttributeValue pr;
-    pr.priority = t->priority;
     return cudaGraphAddKernelNode(&node, t->graph, nullptr, 0, &kp) == cudaSuccess &&
-                   cudaGraphKernelNodeSetAttribute(node, cudaLaunchAttributeClusterDimension, &at[0].val) == cudaSuccess &&
-                   cudaGraphKernelNodeSetAttribute(node, cudaLaunchAttributePriority, &pr) == cudaSuccess
+                   cudaGraphKernelNodeSetAttribute(node, cudaLaunchAttributeClusterDimension, &at[0].val) == cudaSuccess
                ? 0
                : -3;
   }
@@ -394,8 +390,8 @@ ResidentShape resident2d_shape(int storage, int coll, int nx, int ny, bool alone
 
 int launch_resident2d(const ResidentArgs& a) { return launch_to(a, nullptr); }
 
-int add_resident2d_node(const ResidentArgs& a, void* graph, int priority) {
-  const Target t = {(cudaGraph_t)graph, priority, nullptr};
+int add_resident2d_node(const ResidentArgs& a, void* graph) {
+  const Target t = {(cudaGraph_t)graph, nullptr};
   return launch_to(a, &t);
 }
 
@@ -406,7 +402,7 @@ int resident2d_clusters(const ResidentShape& shape, int storage, int coll) {
   a.coll = coll;
   a.shape = shape;
   int n = 0;
-  const Target t = {nullptr, 0, &n};
+  const Target t = {nullptr, &n};
   if (launch_to(a, &t) == 0) return n;
   cudaGetLastError();
   return 0;

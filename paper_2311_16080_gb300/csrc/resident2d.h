@@ -47,7 +47,7 @@ struct ResidentArgs {
 
 // 0 on a successful launch request, else a negative code.
 int launch_resident2d(const ResidentArgs& a);
-// The same launch as a node of a graph (cudaGraph_t), with a launch priority.
-int add_resident2d_node(const ResidentArgs& a, void* graph, int priority);
+// The same launch as a node of a graph (cudaGraph_t).
+int add_resident2d_node(const ResidentArgs& a, void* graph);
 
 }  // namespace xlb
