@@ -108,6 +108,9 @@ struct xlb_ctx {
   int* bz = nullptr;
   float* bz_q = nullptr;
   int64_t n_bz = 0;  // cells with Bouzidi links
+  // updates have been queued (or captured) that leave WALL cells' slots as the
+  // buffer had them, but for the ghost values
+  bool loose_walls = false;
   // graph replay of the update (xlb_set_step_graph): g updates per graph, one
   // executable graph per starting buffer, each valid for one parameter epoch
   int64_t graph_g = 0;
@@ -1280,6 +1283,7 @@ static int run_updates(xlb_ctx* c, int* cur, int64_t n, bool keep) {
   a.bz_q = c->bz_q;
   a.plan = c->tile;
   a.stream = c->stream;
+  c->loose_walls = true;
   int64_t launches = (n + c->tile.halo - 1) / c->tile.halo;
   if (keep && (n - launches) % 2) ++launches;
   for (int64_t left = n; left > 0; --launches) {
@@ -1396,6 +1400,7 @@ static int step_resident(xlb_ctx* c, int64_t room, int64_t* done) {
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(c, e, "resident kernel launch");
   if (r) return fail(c, XLB_ERR_CUDA, "resident kernel launch rejected (code %d)", r);
+  c->loose_walls = true;
   c->cur ^= a.steps & 1;
   *done = a.steps;
   return boundary_pass(c, nullptr, c->buf[c->cur]);
@@ -1659,9 +1664,25 @@ int xlb_state_bytes(const xlb_ctx* c, size_t* bytes) {
   return XLB_OK;
 }
 
+// Before the stored bytes are handed out: WALL cells' slots that no update of
+// the resident and the tiled kernel writes hold whatever the buffer had (at
+// first, old device memory).  They become the rest state with the ghost values
+// of the present one.  (Done here, not in the kernels: carrying the slots over
+// in each launch cost the 1761 x 330 cylinder 4 to 7% of an update.)
+static int settle_walls(xlb_ctx* c) {
+  if (!c->loose_walls || !c->kind_h || !c->has_mask) return XLB_OK;
+  if (launch_clear_walls(c->buf[c->cur], c->esize, c->flags, c->Q, c->N, c->plane, c->stream) != 0)
+    return fail(c, XLB_ERR_CUDA, "clearing of WALL cells rejected");
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(c, e, "clearing of WALL cells");
+  return boundary_pass(c, nullptr, c->buf[c->cur]);
+}
+
 int xlb_state_get(xlb_ctx* c, void* buf, size_t bytes) {
   if (!c || !buf) return XLB_ERR_ARG;
   if (bytes < 64 + state_bytes_raw(c)) return fail(c, XLB_ERR_ARG, "buffer too small");
+  const int r = settle_walls(c);
+  if (r) return r;
   StateHeader h;
   memset(&h, 0, sizeof h);
   memcpy(h.magic, "XLBSTAT1", 8);
@@ -1704,6 +1725,8 @@ int xlb_state_set(xlb_ctx* c, const void* buf, size_t bytes) {
 
 int xlb_populations(xlb_ctx* c, void** ptr, int64_t* plane) {
   if (!c || !ptr || !plane) return XLB_ERR_ARG;
+  const int r = settle_walls(c);
+  if (r) return r;
   c->init_epoch = 0;  // the caller may write through the pointer
   *ptr = c->buf[c->cur];
   *plane = c->plane;

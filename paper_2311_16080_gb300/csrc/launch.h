@@ -101,9 +101,12 @@ int launch_pred_write(int Q, const int* face, bool x_in, bool x_out, const uint8
                       const long long* offs, int2* links, int* cells, void* stream);
 // *flag is set to 1 if some link's source (cells: launch_link_cells) lies off
 // the face planes among x = 0 (face0) and x = nx - 1 (face1).
+int launch_links_off_x(const int2* cells, long long n, int nx, bool face0, bool face1, int* flag, void* stream);
+// The Q slots of every WALL cell become the rest state, as an initialisation
+// leaves them (esize: bytes per stored population).
+int launch_clear_walls(void* f, int esize, const uint8_t* flags, int Q, long long n, long long plane, void* stream);
 // Per link {cell x, dir i | ...}: the source cell x - c_i (periodic) and the
 // cell x + c_i when it is FLUID, else -1 (the boundary pass's Bouzidi partner).
-int launch_links_off_x(const int2* cells, long long n, int nx, bool face0, bool face1, int* flag, void* stream);
 int launch_link_cells(int Q, const int2* links, long long n, const uint8_t* flags, int nx, int ny, int nz,
                       int2* cells, void* stream);
 

@@ -329,6 +329,27 @@ int launch_links_off_x(const int2* cells, long long n, int nx, bool face0, bool 
   return 0;
 }
 
+template <typename T>
+__global__ void k_clear_walls(T* __restrict__ f, const uint8_t* __restrict__ flags, int Q, long long n,
+                              long long plane) {
+  for (long long cell = blockIdx.x * 256LL + threadIdx.x; cell < n; cell += (long long)gridDim.x * 256)
+    if ((flags[cell] & FLAG_TYPE) == WALL)
+      for (int i = 0; i < Q; ++i) f[i * plane + cell] = T(0);
+}
+
+int launch_clear_walls(void* f, int esize, const uint8_t* flags, int Q, long long n, long long plane, void* stream) {
+  const long long b = (n + 255) / 256;
+  const unsigned grid = (unsigned)(b < 152 * 32 ? b : 152 * 32);
+  cudaStream_t s = (cudaStream_t)stream;
+  if (esize == 4)
+    k_clear_walls<<<grid, 256, 0, s>>>((uint32_t*)f, flags, Q, n, plane);
+  else if (esize == 2)
+    k_clear_walls<<<grid, 256, 0, s>>>((uint16_t*)f, flags, Q, n, plane);
+  else
+    return -1;
+  return 0;
+}
+
 int launch_link_cells(int Q, const int2* links, long long n, const uint8_t* flags, int nx, int ny, int nz,
                       int2* cells, void* stream) {
   if (n <= 0) return 0;
