@@ -56,7 +56,8 @@ enum { XLB_COLL_NONE = 0, XLB_COLL_BGK = 1, XLB_COLL_KBC = 2 };
  * BF16 rounds stochastically (up with probability equal to the discarded
  * fraction), from random bits hashed from the cell index and the cell's FP32
  * values, so that results are reproducible and identical in every kernel
- * variant; ghost values of boundary links round to nearest even. */
+ * variant; ghost values of boundary links likewise, from bits hashed from the
+ * slot they are written to and the value. */
 enum { XLB_STORE_F32 = 0, XLB_STORE_F16 = 1, XLB_STORE_BF16 = 2 };
 
 /* Cell types of the mask (Section 3.5).  For a fluid-like or FWALL cell x

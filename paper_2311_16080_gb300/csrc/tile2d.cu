@@ -45,6 +45,19 @@ constexpr int M_WALLS = 0xff;
 // but packed in a list that a few warps work off beside it
 constexpr int M_LISTED = M_INLET | M_BEFORE | M_BZ;
 
+// The lattice's slot (direction j, cell) that the ghost value of the link from
+// cell `self` in direction i = opp(j) is written to: BF16 rounds it by that
+// number.  The wall may lie across a periodic seam.
+template <typename S>
+__device__ __forceinline__ uint32_t ghost_slot(const StepParams& p, int self, int i, int j) {
+  if (!std::is_same<S, __nv_bfloat16>::value) return 0u;  // (no key)
+  const int y = self / p.nx, x = self - y * p.nx;
+  int xw = x + Lattice<9>::c(i, 0), yw = y + Lattice<9>::c(i, 1);
+  xw = xw < 0 ? p.nx - 1 : (xw == p.nx ? 0 : xw);
+  yw = yw < 0 ? p.ny - 1 : (yw == p.ny ? 0 : yw);
+  return (uint32_t)((long long)j * p.plane + xw + p.nx * yw);
+}
+
 // A value as a ghost slot (k of the lattice) would store it.
 template <typename S>
 __device__ __forceinline__ float ghost_round(uint32_t slot, float v) {
@@ -87,8 +100,7 @@ __device__ __forceinline__ void special_pull(const StepParams& p, int m, int row
     for (int i = 1; i < 9; ++i) {
       const int j = opposite<9>(i);
       const float2 w = __ldg(q + i);
-      const int wall = self + Lattice<9>::c(i, 0) + p.nx * Lattice<9>::c(i, 1);
-      const float v = ghost_round<S>((uint32_t)((long long)j * p.plane + wall), __fmaf_rn(w.x, f[j], __fmul_rn(w.y, f[i])));
+      const float v = ghost_round<S>(ghost_slot<S>(p, self, i, j), __fmaf_rn(w.x, f[j], __fmul_rn(w.y, f[i])));
       g[j] = (low >> i & 1) ? v : f[j];
     }
 #pragma unroll
@@ -118,9 +130,8 @@ __device__ __forceinline__ void special_push(const StepParams& p, int self, cons
   for (int i = 1; i < 9; ++i) {
     const int j = opposite<9>(i);
     const float2 w = __ldg(q + i);
-    const int wall = self + Lattice<9>::c(i, 0) + p.nx * Lattice<9>::c(i, 1);
     S s;
-    st_ghost<S>(&s, (uint32_t)((long long)j * p.plane + wall), __fmaf_rn(w.x, h[i], __fmul_rn(w.y, h[j])));
+    st_ghost<S>(&s, ghost_slot<S>(p, self, i, j), __fmaf_rn(w.x, h[i], __fmul_rn(w.y, h[j])));
     if (high >> i & 1) {
       if constexpr (sizeof(S) == 4) {
         asm volatile("st.shared.f32 [%0], %1;" ::"r"(a + i * SB), "f"(s) : "memory");
