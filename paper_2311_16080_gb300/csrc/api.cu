@@ -490,9 +490,10 @@ static int launch_collide_local(xlb_ctx* c, void* buf) {
 }
 
 // The first update: from the initial fields where the state is still f_0 as
-// xlb_init left it, else a local collision of the stored state.
-static int launch_first(xlb_ctx* c, void* buf) {
-  if (c->init_epoch != c->epoch || c->coll == XLB_COLL_NONE) return launch_collide_local(c, buf);
+// xlb_init left it, else a local collision of the stored state.  So too in a
+// caller's capture: its replays may find another state there.
+static int launch_first(xlb_ctx* c, void* buf, bool captured) {
+  if (captured || c->init_epoch != c->epoch || c->coll == XLB_COLL_NONE) return launch_collide_local(c, buf);
   LaunchArgs a = base_args(c);
   a.dst = buf;
   a.rho = c->init_fields;
@@ -1445,8 +1446,8 @@ int xlb_step(xlb_ctx* c, int64_t n) {
   // In a caller's capture n updates end where n single ones would, so that
   // replays of an even number go on from each other.
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (n > 1) CK(cudaStreamIsCapturing(c->stream, &cs));
-  const bool keep = cs != cudaStreamCaptureStatusNone;
+  if (n > 1 || (n > 0 && !c->kind_h)) CK(cudaStreamIsCapturing(c->stream, &cs));
+  const bool captured = cs != cudaStreamCaptureStatusNone;
   for (int64_t k = 0; k < n; ++k) {
     int r;
     if (c->kind_h && !c->prof) {
@@ -1477,13 +1478,13 @@ int xlb_step(xlb_ctx* c, int64_t n) {
     }
     int64_t m = 1;
     if (!c->kind_h) {
-      r = launch_first(c, c->buf[c->cur]);
+      r = launch_first(c, c->buf[c->cur], captured);
       c->kind_h = 1;
     } else {
       // up to the next checkpoint of an open tape
       m = n - k;
       if (c->tape_open) m = std::min(m, c->tape_k - c->t % c->tape_k);
-      r = run_updates(c, &c->cur, m, keep);
+      r = run_updates(c, &c->cur, m, captured);
     }
     if (r) return r;
     c->t += m;
