@@ -73,6 +73,7 @@ struct xlb_ctx {
   float* init_fields = nullptr;  // (1 + D) * N: rho0, u0 (component-major)
   bool has_init = false;
   uint64_t init_epoch = 0;  // buf[cur] is f_0 of init_fields under this epoch's parameters (0: it is not)
+  bool handed_out = false;  // a pointer to buf[cur] (xlb_populations) that is valid until the next update
   int kind_h = 0;
   int64_t t = 0;
   // boundary values and force
@@ -1221,7 +1222,7 @@ int xlb_init(xlb_ctx* c, const float* rho, const float* u) {
   c->init_epoch = 0;
   int r = launch_init(c, c->buf[c->cur]);
   if (r) return r;
-  c->init_epoch = c->epoch;
+  c->init_epoch = c->handed_out ? 0 : c->epoch;  // (its holder may write over f_0)
   c->kind_h = 0;
   c->t = 0;
   return XLB_OK;
@@ -1443,6 +1444,7 @@ int xlb_step(xlb_ctx* c, int64_t n) {
   if (!c->has_init && c->t == 0 && !c->kind_h) return fail(c, XLB_ERR_STATE, "xlb_init (or xlb_state_set) first");
   if (c->tape_open && c->t + n > c->tape_T)
     return fail(c, XLB_ERR_STATE, "stepping past the tape length %lld", (long long)c->tape_T);
+  if (n > 0) c->handed_out = false;
   // In a caller's capture n updates end where n single ones would, so that
   // replays of an even number go on from each other.
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -1729,6 +1731,7 @@ int xlb_populations(xlb_ctx* c, void** ptr, int64_t* plane) {
   const int r = settle_walls(c);
   if (r) return r;
   c->init_epoch = 0;  // the caller may write through the pointer
+  c->handed_out = true;
   *ptr = c->buf[c->cur];
   *plane = c->plane;
   return XLB_OK;
