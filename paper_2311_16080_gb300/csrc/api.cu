@@ -1023,6 +1023,102 @@ int xlb_set_inlet_normal(xlb_ctx* c, int axis, int sign) {
   return XLB_OK;
 }
 
+// Time of one D2Q9 update launched by itself, as measured on lattices of 128^2
+// to 601 x 599 cells: 2.1 us, 1.55 us replayed from a graph, or the cells' time;
+// a boundary pass 2.4 us more, 3.3 us in 16-bit storage.
+static double single_update_us(const xlb_ctx* c, bool graph) {
+  const double rate = c->coll == XLB_COLL_KBC ? 69e3 : c->storage == XLB_STORE_BF16 ? 60e3 : 108e3;  // cells per us
+  const double us = std::max(graph ? 1.55 : 2.1, 1.1 + (double)c->N / rate);
+  return us + (c->n_links > 0 ? (c->esize == 2 ? 3.3 : 2.4) : 0.0);
+}
+
+// Whether the tiled D2Q9 kernel may take updates of a lattice with this mask, for
+// n_bz cells with Bouzidi links: FLUID and WALL cells, inflow and outflow planes
+// together (the lattice then ends at them; the cells before an OUTLET cell hand
+// it what they pull, so they must not be WALL).  graph: single updates would be
+// replayed from a graph.
+static bool tile_fits(xlb_ctx* c, int64_t n_bz, bool graph) {
+  if (c->Q != 9 || c->coll == XLB_COLL_NONE || c->has_lid_eq || c->n_fix > 0 || has_fwall_face(c)) return false;
+  if (c->outlet_walled || c->x_inlet != c->x_outlet) return false;
+  if (c->tile.halo < 0) c->tile = tile2d_plan(c->storage, c->coll, (int)c->nx, (int)c->ny);
+  if (c->tile.halo < 2 || n_bz + 2 * (c->tile.by + 2 * c->tile.halo) > TILE_LIST) return false;
+  return c->tile.us < 0.95 * single_update_us(c, graph);
+}
+
+// Whether it may take this ctx's updates now.
+static bool tile_ok(xlb_ctx* c) {
+  if (c->x_inlet && (c->inlet_axis != 0 || c->inlet_sign != 1)) return false;
+  if (c->link_q && !c->bz) return false;
+  return tile_fits(c, c->n_bz, c->graph_g > 0);
+}
+
+// The wall distances by cell, for the tiled kernel (Tile2dArgs::bz, bz_q): entry k
+// of the list is link link[k] of the table.  None where that kernel can never take
+// this lattice's updates, and none without the memory, which is no error: the
+// updates are then launched one by one.
+static int build_bz(xlb_ctx* c, int64_t n, const int64_t* cell, const int32_t* dir, const size_t* link,
+                    const float* q) {
+  if (!tile_fits(c, 0, false)) return XLB_OK;
+  // the cells' rows
+  std::vector<int> cells;
+  std::vector<int> row((size_t)n);
+  {
+    std::vector<int64_t> by((size_t)n);
+    for (int64_t k = 0; k < n; ++k) by[(size_t)k] = k;
+    std::sort(by.begin(), by.end(), [&](int64_t a, int64_t b) { return cell[a] < cell[b]; });
+    for (int64_t k : by) {
+      if (cells.empty() || cells.back() != (int)cell[k]) cells.push_back((int)cell[k]);
+      row[(size_t)k] = (int)cells.size() - 1;
+    }
+  }
+  if (!tile_fits(c, (int64_t)cells.size(), false)) return XLB_OK;
+  // The kernel updates the outlet column by itself, without rows: no tiles where an
+  // OUTLET cell owns such a link (a body that reaches the column before it).
+  for (int x : cells)
+    if (c->x_outlet && x % c->nx == c->nx - 1) return XLB_OK;
+  std::vector<int2> partner((size_t)c->n_links);
+  CK(cudaMemcpy(partner.data(), c->link_cells, sizeof(int2) * partner.size(), cudaMemcpyDeviceToHost));
+  std::vector<float> rq(18 * cells.size(), 0.0f);
+  std::vector<uint32_t> bits(2 * cells.size(), 0u);
+  for (int64_t k = 0; k < n; ++k) {
+    const bool behind = partner[link[k]].y >= 0;  // x + c_j is FLUID
+    const float qk = q[k] < 0.5f && !behind ? 0.5f : q[k];
+    const float w = qk < 0.5f ? 2.0f * qk : 0.5f / qk;
+    float* pair = rq.data() + 18 * (size_t)row[(size_t)k] + 2 * dir[k];
+    pair[0] = w;
+    pair[1] = 1.0f - w;
+    uint32_t* b = bits.data() + 2 * (size_t)row[(size_t)k];
+    b[0] &= ~(1u << dir[k]);
+    b[1] &= ~(1u << dir[k]);
+    b[qk < 0.5f ? 0 : 1] |= 1u << dir[k];
+  }
+  for (size_t r = 0; r < cells.size(); ++r) memcpy(rq.data() + 18 * r, bits.data() + 2 * r, 8);
+  int* list = nullptr;
+  cudaError_t e = cudaMalloc(&c->bz, sizeof(int) * (size_t)c->N);
+  if (e == cudaSuccess) e = cudaMalloc(&c->bz_q, sizeof(float) * rq.size());
+  if (e == cudaSuccess) e = cudaMalloc(&list, sizeof(int) * cells.size());
+  const bool room = e != cudaErrorMemoryAllocation;
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->bz, 0, sizeof(int) * (size_t)c->N, c->stream);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(list, cells.data(), sizeof(int) * cells.size(), cudaMemcpyHostToDevice, c->stream);
+  if (e == cudaSuccess) {
+    launch_number_cells(list, (int)cells.size(), c->bz, c->stream);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(c->bz_q, rq.data(), sizeof(float) * rq.size(), cudaMemcpyHostToDevice, c->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+  if (list) cudaFree(list);
+  if (e != cudaSuccess) {
+    free_bz(c);
+    if (room) return cuda_fail(c, e, "wall distances by cell");
+    cudaGetLastError();
+    return XLB_OK;
+  }
+  c->n_bz = (int64_t)cells.size();
+  return XLB_OK;
+}
+
 int xlb_set_wall_distances(xlb_ctx* c, int64_t n, const int64_t* cell, const int32_t* dir, const float* q) {
   if (!c) return XLB_ERR_ARG;
   if (n < 0 || (n > 0 && (!cell || !dir || !q))) return fail(c, XLB_ERR_ARG, "n < 0 or a null array");
@@ -1043,6 +1139,7 @@ int xlb_set_wall_distances(xlb_ctx* c, int64_t n, const int64_t* cell, const int
     }
   }
   std::vector<float> hq(hl.size(), 0.f);
+  std::vector<size_t> link(c->Q == 9 ? (size_t)n : 0);  // of the table, per entry of the list (build_bz)
   for (int64_t k = 0; k < n; ++k) {
     const int i = dir[k];
     if (i < 1 || i >= c->Q) return fail(c, XLB_ERR_ARG, "link %lld: direction %d out of range", (long long)k, i);
@@ -1061,6 +1158,7 @@ int xlb_set_wall_distances(xlb_ctx* c, int64_t n, const int64_t* cell, const int
     const size_t idx = (size_t)(e - hl.data());
     hl[idx].y |= LINK_BZ;
     hq[idx] = q[k];
+    if (c->Q == 9) link[(size_t)k] = idx;
   }
   // the new rule acts from the next step on (like xlb_set_bc)
   int r = materialize_post_stream(c);
@@ -1071,58 +1169,8 @@ int xlb_set_wall_distances(xlb_ctx* c, int64_t n, const int64_t* cell, const int
   ++c->epoch;
   if (n > 0) CK(cudaMalloc(&c->link_q, sizeof(float) * hq.size()));
   if (n > 0) CK(cudaMemcpy(c->link_q, hq.data(), sizeof(float) * hq.size(), cudaMemcpyHostToDevice));
-  // The tiled kernel updates the outlet column by itself, without the rows of
-  // a cell with Bouzidi links: no tables, and so no tiles, where an OUTLET cell
-  // owns such a link (a body that reaches the column before it).
-  bool outlet_link = false;
-  for (int64_t k = 0; k < n && c->x_outlet; ++k) outlet_link |= cell[k] % c->nx == c->nx - 1;
-  if (n > 0 && c->Q == 9 && !outlet_link) {
-    // the same by cell, for the tiled kernel (which is not used without them:
-    // no memory for them is no error)
-    std::vector<uint8_t> fl((size_t)c->N);
-    CK(cudaMemcpy(fl.data(), c->flags, fl.size(), cudaMemcpyDeviceToHost));
-    std::vector<int> row((size_t)c->N, 0);
-    std::vector<float> rq;  // Tile2dArgs::bz_q
-    std::vector<uint32_t> bits;
-    for (int64_t k = 0; k < n; ++k) {
-      const int j = lattice_opposite(9, dir[k]);
-      int& r0 = row[(size_t)cell[k]];
-      if (!r0) {
-        rq.insert(rq.end(), 18, 0.0f);
-        bits.insert(bits.end(), 2, 0u);
-        r0 = (int)(rq.size() / 18);
-      }
-      const int64_t x = (cell[k] % c->nx + Lattice<9>::c(j, 0) + c->nx) % c->nx;
-      const int64_t y = (cell[k] / c->nx + Lattice<9>::c(j, 1) + c->ny) % c->ny;
-      const bool behind = (fl[(size_t)(x + c->nx * y)] & FLAG_TYPE) == XLB_CELL_FLUID;
-      const float qk = q[k] < 0.5f && !behind ? 0.5f : q[k];
-      const float w = qk < 0.5f ? 2.0f * qk : 0.5f / qk;
-      float* pair = rq.data() + 18 * (size_t)(r0 - 1) + 2 * dir[k];
-      pair[0] = w;
-      pair[1] = 1.0f - w;
-      uint32_t* b = bits.data() + 2 * (size_t)(r0 - 1);
-      b[0] &= ~(1u << dir[k]);
-      b[1] &= ~(1u << dir[k]);
-      b[qk < 0.5f ? 0 : 1] |= 1u << dir[k];
-    }
-    for (size_t r0 = 0; r0 < bits.size() / 2; ++r0) memcpy(rq.data() + 18 * r0, bits.data() + 2 * r0, 8);
-    c->n_bz = (int64_t)rq.size() / 18;
-    cudaError_t e = cudaMalloc(&c->bz, sizeof(int) * row.size());
-    if (e == cudaSuccess) e = cudaMalloc(&c->bz_q, sizeof(float) * rq.size());
-    if (e == cudaErrorMemoryAllocation) {
-      cudaGetLastError();
-      free_bz(c);
-    } else {
-      if (e == cudaSuccess) e = cudaMemcpy(c->bz, row.data(), sizeof(int) * row.size(), cudaMemcpyHostToDevice);
-      if (e == cudaSuccess) e = cudaMemcpy(c->bz_q, rq.data(), sizeof(float) * rq.size(), cudaMemcpyHostToDevice);
-      if (e != cudaSuccess) {
-        free_bz(c);
-        return cuda_fail(c, e, "wall distances by cell");
-      }
-    }
-  }
   if (!hl.empty()) CK(cudaMemcpy(c->links, hl.data(), sizeof(int2) * hl.size(), cudaMemcpyHostToDevice));
-  return XLB_OK;
+  return n > 0 && c->Q == 9 ? build_bz(c, n, cell, dir, link.data(), q) : XLB_OK;
 }
 
 int xlb_wall_force(xlb_ctx* c, double* out) {
@@ -1236,29 +1284,6 @@ static int record_checkpoint(xlb_ctx* c) {
       CK(cudaMemcpyAsync(c->ckpt[s], c->buf[c->cur], state_bytes_raw(c), cudaMemcpyDeviceToDevice, c->stream));
   }
   return XLB_OK;
-}
-
-// Time of one D2Q9 update launched by itself, as measured on lattices of 128^2
-// to 601 x 599 cells: 2.1 us, 1.55 us replayed from a graph, or the cells' time;
-// a boundary pass 2.4 us more, 3.3 us in 16-bit storage.
-static double single_update_us(const xlb_ctx* c) {
-  const double rate = c->coll == XLB_COLL_KBC ? 69e3 : c->storage == XLB_STORE_BF16 ? 60e3 : 108e3;  // cells per us
-  const double us = std::max(c->graph_g > 0 ? 1.55 : 2.1, 1.1 + (double)c->N / rate);
-  return us + (c->n_links > 0 ? (c->esize == 2 ? 3.3 : 2.4) : 0.0);
-}
-
-// Whether the tiled D2Q9 kernel may take this ctx's updates: FLUID and WALL
-// cells, inflow and outflow planes together (the lattice then ends at them; the
-// cells before an OUTLET cell hand it what they pull, so they must not be WALL),
-// Bouzidi links.
-static bool tile_ok(xlb_ctx* c) {
-  if (c->Q != 9 || c->coll == XLB_COLL_NONE || c->has_lid_eq || c->n_fix > 0 || has_fwall_face(c)) return false;
-  if (c->outlet_walled) return false;
-  if (c->x_inlet != c->x_outlet || (c->x_inlet && (c->inlet_axis != 0 || c->inlet_sign != 1))) return false;
-  if (c->link_q && !c->bz) return false;
-  if (c->tile.halo < 0) c->tile = tile2d_plan(c->storage, c->coll, (int)c->nx, (int)c->ny);
-  if (c->tile.halo < 2 || c->n_bz + 2 * (c->tile.by + 2 * c->tile.halo) > TILE_LIST) return false;
-  return c->tile.us < 0.95 * single_update_us(c);
 }
 
 // n updates of the post-collision state in buf[*cur], launched (or captured)
@@ -1378,7 +1403,7 @@ static int step_resident(xlb_ctx* c, int64_t room, int64_t* done) {
   if (!c->res.one) return XLB_OK;
   const double cells = (double)((c->ny + c->res.ctas - 1) / c->res.ctas * c->nx);
   const double us = 0.6 + 0.9 * cells / 1024.0 * (c->coll == XLB_COLL_KBC ? 2.0 : 1.0);
-  if (us > single_update_us(c) || (tile_ok(c) && us > c->tile.us)) return XLB_OK;
+  if (us > single_update_us(c, c->graph_g > 0) || (tile_ok(c) && us > c->tile.us)) return XLB_OK;
   ResidentArgs a;
   memset(&a, 0, sizeof a);
   a.src = c->buf[c->cur];

@@ -102,6 +102,8 @@ int launch_pred_write(int Q, const int* face, bool x_in, bool x_out, const uint8
 // *flag is set to 1 if some link's source (cells: launch_link_cells) lies off
 // the face planes among x = 0 (face0) and x = nx - 1 (face1).
 int launch_links_off_x(const int2* cells, long long n, int nx, bool face0, bool face1, int* flag, void* stream);
+// number[cells[k]] = k + 1 for k < n.
+void launch_number_cells(const int* cells, int n, int* number, void* stream);
 // The Q slots of every WALL cell become the rest state, as an initialisation
 // leaves them (esize: bytes per stored population).
 int launch_clear_walls(void* f, int esize, const uint8_t* flags, int Q, long long n, long long plane, void* stream);

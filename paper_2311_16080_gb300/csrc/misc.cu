@@ -329,6 +329,15 @@ int launch_links_off_x(const int2* cells, long long n, int nx, bool face0, bool 
   return 0;
 }
 
+__global__ void k_number_cells(const int* __restrict__ cells, int n, int* __restrict__ number) {
+  const int k = blockIdx.x * 256 + threadIdx.x;
+  if (k < n) number[cells[k]] = k + 1;
+}
+
+void launch_number_cells(const int* cells, int n, int* number, void* stream) {
+  if (n > 0) k_number_cells<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(cells, n, number);
+}
+
 template <typename T>
 __global__ void k_clear_walls(T* __restrict__ f, const uint8_t* __restrict__ flags, int Q, long long n,
                               long long plane) {
