@@ -190,7 +190,8 @@ int xlb_set_inlet_normal(xlb_ctx* ctx, int axis, int sign);
  * a link is not a ghost link of the mask (the neighbour is not WALL, the cell
  * owns no links, or the neighbour lies on a boundary face plane that is handled
  * by coordinates: with 16-bit storage the x-face planes have links and take
- * distances) or a q is outside [0, 1]; XLB_ERR_STATE before a mask or while a tape is open. */
+ * distances) or a q is outside [0, 1]; XLB_ERR_STATE before a mask or while a
+ * tape is open. */
 int xlb_set_wall_distances(xlb_ctx* ctx, int64_t n, const int64_t* cell, const int32_t* dir, const float* q);
 
 /* Momentum-exchange force on the WALL cells off the boundary faces (Mei et
@@ -373,15 +374,19 @@ int xlb_tape_release(xlb_ctx* ctx);
  *   XLB_KERNEL_AUTO:   the default, the fastest measured: FP16 runs VEC on
  *     lattices without boundary planes and VEC2 with them (D3Q19: VEC from 3 M
  *     cells, DIRECT between 16,384 and 3 M cells where the x-faces are the
- *     only links and carry no wall distances), BF16 DIRECT (D3Q19: VEC from 100,000 cells without boundary
- *     planes, from 8 M with them), FP32 DIRECT.
+ *     only links and carry no wall distances), BF16 DIRECT (D3Q19: VEC from
+ *     100,000 cells without boundary planes, from 8 M with them), FP32 DIRECT.
+ *     With AUTO a D2Q9 call of several updates may also take many of them in
+ *     one launch (a kernel that keeps the lattice, or tiles of it, on the SMs);
+ *     any other choice launches every update by itself.
  * A mask with an FWALL face plane always runs DIRECT. */
 enum { XLB_KERNEL_AUTO = 0, XLB_KERNEL_DIRECT = 1, XLB_KERNEL_VEC = 2, XLB_KERNEL_VEC2 = 3 };
 
 /* Choose the variant (XLB_ERR_UNSUPPORTED if it cannot run this ctx). */
 int xlb_set_kernel(xlb_ctx* ctx, int variant);
 
-/* The variant the next update launches (DIRECT, VEC or VEC2). */
+/* The variant the next update launches where it is launched by itself (DIRECT,
+ * VEC or VEC2). */
 int xlb_get_kernel(const xlb_ctx* ctx, int* variant);
 
 /* ---- batched small 2D domains (Section 6 batching) --------------------- */

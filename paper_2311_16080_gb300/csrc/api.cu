@@ -1045,8 +1045,10 @@ static bool tile_fits(xlb_ctx* c, int64_t n_bz, bool graph) {
   return c->tile.us < 0.95 * single_update_us(c, graph);
 }
 
-// Whether it may take this ctx's updates now.
+// Whether it may take this ctx's updates now.  (A variant that the caller has
+// chosen takes them one by one.)
 static bool tile_ok(xlb_ctx* c) {
+  if (c->variant != XLB_KERNEL_AUTO) return false;
   if (c->x_inlet && (c->inlet_axis != 0 || c->inlet_sign != 1)) return false;
   if (c->link_q && !c->bz) return false;
   return tile_fits(c, c->n_bz, c->graph_g > 0);
@@ -1388,8 +1390,8 @@ constexpr int64_t RESIDENT_MIN = 2, RESIDENT_MAX = 20000;
 
 static int step_resident(xlb_ctx* c, int64_t room, int64_t* done) {
   *done = 0;
-  if (c->Q != 9 || c->coll == XLB_COLL_NONE || room < RESIDENT_MIN || c->has_inlet_outlet || c->has_lid_eq ||
-      c->link_q)
+  if (c->Q != 9 || c->coll == XLB_COLL_NONE || c->variant != XLB_KERNEL_AUTO || room < RESIDENT_MIN ||
+      c->has_inlet_outlet || c->has_lid_eq || c->link_q)
     return XLB_OK;
   if (c->res.ctas < 0) {
     c->res = resident2d_shape(c->storage, c->coll, (int)c->nx, (int)c->ny, true);
