@@ -1399,10 +1399,9 @@ static int step_resident(xlb_ctx* c, int64_t room, int64_t* done) {
     if (c->res.ctas > 0 && resident2d_clusters(c->res, c->storage, c->coll) < 1) c->res.ctas = 0;
   }
   if (c->res.ctas == 0) return XLB_OK;
-  // With one cell per thread an update costs 0.6 us and 0.9 us more for each
-  // 1024 cells a block (128^2 on 16 blocks: 1.5 us; KBC twice that); with more
-  // the tiles are faster (256 x 128: 3.5 us against 2.0).
-  if (!c->res.one) return XLB_OK;
+  // An update costs 0.6 us and 0.9 us more for each 1024 cells a block (128^2 on
+  // 16 blocks: 1.5 us; KBC twice that).  (Lattices with more cells a block than
+  // threads are not taken: the tiles are faster, 256 x 128 2.0 us against 3.5.)
   const double cells = (double)((c->ny + c->res.ctas - 1) / c->res.ctas * c->nx);
   const double us = 0.6 + 0.9 * cells / 1024.0 * (c->coll == XLB_COLL_KBC ? 2.0 : 1.0);
   if (us > single_update_us(c, c->graph_g > 0) || (tile_ok(c) && us > c->tile.us)) return XLB_OK;

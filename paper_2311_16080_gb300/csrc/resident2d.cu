@@ -310,7 +310,11 @@ struct Target {
 
 template <typename S, int COLL>
 int launch_typed_resident(const ResidentArgs& a, const Target* t) {
-  auto kern = a.shape.one ? k_resident2d<S, COLL, R_SINGLE> : k_resident2d<S, COLL, R_LOOP>;
+  // (more than one cell per thread: the domains of a batch, which is BGK)
+  if (COLL != COLL_BGK && !a.shape.one) return -2;
+  auto kern = k_resident2d<S, COLL, R_SINGLE>;
+  if constexpr (COLL == COLL_BGK)
+    if (!a.shape.one) kern = k_resident2d<S, COLL, R_LOOP>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, RESIDENT_SMEM) != cudaSuccess ||
       (a.shape.ctas > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess))
     return -3;
@@ -372,18 +376,22 @@ ResidentShape resident2d_shape(int storage, int coll, int nx, int ny, bool alone
   const ResidentShape none = {0, 0, 0, false};
   if (coll != COLL_BGK && coll != COLL_KBC) return none;
   const long long cell = storage == XLB_STORE_F32 ? 9 * 4 + 2 : 10 * 2;  // Slots<S>, meta included
+  auto fit = [&](int ctas, long long limit, bool one) {
+    const int c = ctas > ny ? ny : ctas;
+    const long long cells = (long long)((ny + c - 1) / c) * nx;
+    const long long smem = (cells * cell + 15) / 16 * 16;
+    if (smem > limit || (one && cells > 1024)) return none;
+    if (cells <= 1024) return ResidentShape{c, (int)((cells + 31) / 32 * 32), smem, true};
+    // 80 registers: 768 threads fill an SM
+    return ResidentShape{c, limit == RESIDENT_SMEM ? 768 : 384, smem, false};
+  };
+  if (alone) return fit(16, RESIDENT_SMEM, true);
   // many domains: two blocks per SM where eight blocks' worth of that is
   // enough, else one
-  constexpr long long HALF = 112 * 1024;
-  for (long long limit = alone ? RESIDENT_SMEM : HALF; limit <= RESIDENT_SMEM; limit += RESIDENT_SMEM - HALF)
-    for (int ctas = alone ? 16 : 1; ctas <= (alone ? 16 : 8); ++ctas) {
-      const int c = ctas > ny ? ny : ctas;
-      const long long cells = (long long)((ny + c - 1) / c) * nx;
-      const long long smem = (cells * cell + 15) / 16 * 16;
-      if (smem > limit) continue;
-      if (cells <= 1024) return {c, (int)((cells + 31) / 32 * 32), smem, true};
-      // 80 registers: 768 threads fill an SM
-      return {c, limit > HALF ? 768 : 384, smem, false};
+  for (long long limit : {112 * 1024, RESIDENT_SMEM})
+    for (int ctas = 1; ctas <= 8; ++ctas) {
+      const ResidentShape s = fit(ctas, limit, false);
+      if (s.ctas > 0) return s;
     }
   return none;
 }

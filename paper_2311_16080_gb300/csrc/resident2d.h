@@ -23,8 +23,9 @@ struct ResidentShape {
   bool one;        // one cell per thread
 };
 
-// Shape for an nx x ny domain: alone on the GPU (spread wide, so that one
-// domain finishes early) or one of many (packed, so that all of them do).
+// Shape for an nx x ny domain: alone on the GPU (spread wide and with one cell
+// per thread, so that the domain finishes early) or one of many (packed, so that
+// all of them do).
 ResidentShape resident2d_shape(int storage, int coll, int nx, int ny, bool alone);
 
 // Clusters of that shape the GPU holds at once (0: it cannot launch one).
