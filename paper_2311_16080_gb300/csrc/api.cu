@@ -105,7 +105,7 @@ struct xlb_ctx {
   int variant = 0;
   ResidentShape res = {-1, 0, 0, false};  // launch shape of the resident kernel (ctas < 0: not asked yet)
   // the tiled D2Q9 kernel: its plan, and the cells with Bouzidi links (Tile2dArgs)
-  Tile2dPlan tile = {0, 0, 0, 0, -1, 0.f};  // halo < 0: not asked yet
+  Tile2dPlan tile = {0, 0, 0, 0, -1, 0.f, 0};  // halo < 0: not asked yet
   int* bz = nullptr;
   float* bz_q = nullptr;
   int64_t n_bz = 0;  // cells with Bouzidi links
@@ -1023,35 +1023,98 @@ int xlb_set_inlet_normal(xlb_ctx* c, int axis, int sign) {
   return XLB_OK;
 }
 
-// Time of one D2Q9 update launched by itself, as measured on lattices of 128^2
-// to 601 x 599 cells: 2.1 us, 1.55 us replayed from a graph, or the cells' time;
-// a boundary pass 2.4 us more, 3.3 us in 16-bit storage.
+// How a D2Q9 call takes its updates is decided by what n of them cost each way, in
+// us as measured over lattices of 32^2 to 1200 x 1000 cells, three storage types,
+// BGK and KBC, with and without walls, calls of 2 to 48 updates.  With these lines
+// the way taken is on average within 0.5% of the better one; a choice by the cost
+// of one update of many made calls of 2 to 6 up to 2.5 times as slow as single
+// launches (1200 x 1000 FP16: 14.2 us launched one by one, 30.2 in tiles).
+
+// A boundary pass: after each single update (but where those serve the x-faces
+// themselves), and once where many end.
+static double link_pass_us(const xlb_ctx* c) {
+  if (c->n_links == 0) return 0.0;
+  return c->esize == 2 ? 4.2 : c->coll == XLB_COLL_KBC ? 3.0 : 2.6;
+}
+
+// One of several updates launched one by one: 2.0 us, 1.4 (FP16, with two or four
+// cells per thread, 1.7) replayed from a graph, or the cells' time.
 static double single_update_us(const xlb_ctx* c, bool graph) {
-  const double rate = c->coll == XLB_COLL_KBC ? 69e3 : c->storage == XLB_STORE_BF16 ? 60e3 : 108e3;  // cells per us
-  const double us = std::max(graph ? 1.55 : 2.1, 1.1 + (double)c->N / rate);
-  return us + (c->n_links > 0 ? (c->esize == 2 ? 3.3 : 2.4) : 0.0);
+  double fixed = 1.4, rate = 130e3;  // us, cells per us
+  if (c->coll == XLB_COLL_KBC)
+    fixed = 1.6, rate = 88e3;
+  else if (c->storage == XLB_STORE_BF16)
+    fixed = 1.5, rate = 105e3;
+  else if (c->esize == 2)
+    fixed = bulk_variant(c) == XLB_KERNEL_VEC ? 1.2 : 1.4, rate = bulk_variant(c) == XLB_KERNEL_VEC ? 185e3 : 140e3;
+  const double least = !graph ? 2.0 : c->storage == XLB_STORE_F16 ? 1.7 : 1.4;
+  const double links = pulls_x_faces(c) && !use_vec(c) ? 0.0 : link_pass_us(c) * (graph ? 0.9 : 1.0);
+  return std::max(least, fixed + (double)c->N / rate - (graph ? 0.3 : 0.0)) + links;
+}
+
+// n updates launched one by one (graph: all of them within a graph).
+static double single_updates_us(const xlb_ctx* c, int64_t n, bool graph) {
+  const int64_t g = c->graph_g;
+  if (graph || g == 0 || c->tape_open) return (double)n * single_update_us(c, graph);
+  return (double)(n / g) * (3.2 + (double)g * single_update_us(c, true)) + (double)(n % g) * single_update_us(c, false);
+}
+
+// The ghost values of the state that several updates in one launch end in.
+static double last_ghosts_us(const xlb_ctx* c) {
+  bool faces = false;
+  for (int f = 0; f < 6; ++f) faces |= c->face[f] != 0;
+  return link_pass_us(c) + (faces && c->esize == 2 ? 3.8 : 0.0);
+}
+
+// n updates in tiles: a launch's load and store and each update by the cells of a
+// block's region.
+static double tile_us(const xlb_ctx* c, int64_t n) {
+  const Tile2dPlan& p = c->tile;
+  const double k = 1e-3 * (p.bx + 2 * p.halo) * (p.by + 2 * p.halo);
+  double launch = 3.4 + 1.63 * k, update = 0.45 + 0.48 * k;  // FP32 BGK
+  if (c->coll == XLB_COLL_KBC)
+    launch = 6.6 + 1.46 * k, update = std::max(0.3, 1.54 * k - 0.5);
+  else if (c->storage == XLB_STORE_F16)
+    launch = 3.9 + 1.3 * k, update = 0.25 + 0.585 * k;
+  else if (c->storage == XLB_STORE_BF16)
+    launch = 3.5 + 1.15 * k, update = 0.3 + 1.06 * k;
+  return p.waves * ((double)((n + p.halo - 1) / p.halo) * launch + (double)n * update) + last_ghosts_us(c);
+}
+
+// n updates in the shared memory of one cluster, by the cells of a block.
+static double resident_us(const xlb_ctx* c, int64_t n) {
+  const double k = (double)((c->ny + c->res.ctas - 1) / c->res.ctas * c->nx) / 1024.0;
+  double launch = 4.6 + 2.0 * k, update = 0.53 + 0.95 * k;  // FP32 BGK
+  if (c->coll == XLB_COLL_KBC)
+    launch = 4.2 + 1.5 * k, update = 0.77 + 1.28 * k;
+  else if (c->storage == XLB_STORE_F16)
+    launch = 4.7 + 0.9 * k, update = 0.57 + 0.72 * k;
+  else if (c->storage == XLB_STORE_BF16)
+    launch = 4.5 + 1.1 * k, update = 0.69 + 1.03 * k;
+  return launch + (double)n * update + last_ghosts_us(c);
 }
 
 // Whether the tiled D2Q9 kernel may take updates of a lattice with this mask, for
 // n_bz cells with Bouzidi links: FLUID and WALL cells, inflow and outflow planes
 // together (the lattice then ends at them; the cells before an OUTLET cell hand
-// it what they pull, so they must not be WALL).  graph: single updates would be
-// replayed from a graph.
-static bool tile_fits(xlb_ctx* c, int64_t n_bz, bool graph) {
+// it what they pull, so they must not be WALL).
+static bool tile_fits(xlb_ctx* c, int64_t n_bz) {
   if (c->Q != 9 || c->coll == XLB_COLL_NONE || c->has_lid_eq || c->n_fix > 0 || has_fwall_face(c)) return false;
   if (c->outlet_walled || c->x_inlet != c->x_outlet) return false;
   if (c->tile.halo < 0) c->tile = tile2d_plan(c->storage, c->coll, (int)c->nx, (int)c->ny);
   if (c->tile.halo < 2 || n_bz + 2 * (c->tile.by + 2 * c->tile.halo) > TILE_LIST) return false;
-  return c->tile.us < 0.95 * single_update_us(c, graph);
+  const int64_t many = 100 * c->tile.halo;  // (no call of fewer gains more)
+  return tile_us(c, many) < (double)many * single_update_us(c, false);
 }
 
-// Whether it may take this ctx's updates now.  (A variant that the caller has
-// chosen takes them one by one.)
-static bool tile_ok(xlb_ctx* c) {
+// Whether it may take n updates of this ctx now, and gains by it (graph: they are
+// queued into a graph).  (A variant that the caller has chosen takes them one by
+// one.)
+static bool tile_ok(xlb_ctx* c, int64_t n, bool graph) {
   if (c->variant != XLB_KERNEL_AUTO) return false;
   if (c->x_inlet && (c->inlet_axis != 0 || c->inlet_sign != 1)) return false;
   if (c->link_q && !c->bz) return false;
-  return tile_fits(c, c->n_bz, c->graph_g > 0);
+  return tile_fits(c, c->n_bz) && tile_us(c, n) < single_updates_us(c, n, graph);
 }
 
 // The wall distances by cell, for the tiled kernel (Tile2dArgs::bz, bz_q): entry k
@@ -1060,7 +1123,7 @@ static bool tile_ok(xlb_ctx* c) {
 // updates are then launched one by one.
 static int build_bz(xlb_ctx* c, int64_t n, const int64_t* cell, const int32_t* dir, const size_t* link,
                     const float* q) {
-  if (!tile_fits(c, 0, false)) return XLB_OK;
+  if (!tile_fits(c, 0)) return XLB_OK;
   // the cells' rows
   std::vector<int> cells;
   std::vector<int> row((size_t)n);
@@ -1073,7 +1136,7 @@ static int build_bz(xlb_ctx* c, int64_t n, const int64_t* cell, const int32_t* d
       row[(size_t)k] = (int)cells.size() - 1;
     }
   }
-  if (!tile_fits(c, (int64_t)cells.size(), false)) return XLB_OK;
+  if (!tile_fits(c, (int64_t)cells.size())) return XLB_OK;
   // The kernel updates the outlet column by itself, without rows: no tiles where an
   // OUTLET cell owns such a link (a body that reaches the column before it).
   for (int x : cells)
@@ -1291,10 +1354,11 @@ static int record_checkpoint(xlb_ctx* c) {
 // n updates of the post-collision state in buf[*cur], launched (or captured)
 // on the ctx stream; *cur becomes the buffer that holds the result.  The tiled
 // kernel needs no ghost values; those of the last state are written at the end.
-// keep: they end in the buffer that n single updates end in.
-static int run_updates(xlb_ctx* c, int* cur, int64_t n, bool keep) {
+// keep: they end in the buffer that n single updates end in.  graph: they are
+// captured into a graph.
+static int run_updates(xlb_ctx* c, int* cur, int64_t n, bool keep, bool graph) {
   int r = XLB_OK;
-  if (n < (keep ? 3 : 2) || c->prof || !tile_ok(c)) {
+  if (n < (keep ? 3 : 2) || c->prof || !tile_ok(c, n, graph)) {
     for (int64_t k = 0; k < n; ++k) {
       r = launch_step(c, c->buf[*cur], c->buf[*cur ^ 1]);
       if (r) return r;
@@ -1346,7 +1410,7 @@ static int step_graph(xlb_ctx* c, int from, cudaGraphExec_t* out) {
   if (cs != cudaStreamCaptureStatusNone) return fail(c, XLB_ERR_STATE, "the ctx stream is already capturing");
   CK(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
   int cur = from;
-  const int r = run_updates(c, &cur, c->graph_g, false);
+  const int r = run_updates(c, &cur, c->graph_g, false, true);
   cudaGraph_t g = nullptr;
   const cudaError_t e = cudaStreamEndCapture(c->stream, &g);
   if (r != XLB_OK || e != cudaSuccess) {
@@ -1388,7 +1452,7 @@ int xlb_set_step_graph(xlb_ctx* c, int64_t steps_per_graph) {
 // ctx or call does not qualify).
 constexpr int64_t RESIDENT_MIN = 2, RESIDENT_MAX = 20000;
 
-static int step_resident(xlb_ctx* c, int64_t room, int64_t* done) {
+static int step_resident(xlb_ctx* c, int64_t room, bool captured, int64_t* done) {
   *done = 0;
   if (c->Q != 9 || c->coll == XLB_COLL_NONE || c->variant != XLB_KERNEL_AUTO || room < RESIDENT_MIN ||
       c->has_inlet_outlet || c->has_lid_eq || c->link_q)
@@ -1399,12 +1463,10 @@ static int step_resident(xlb_ctx* c, int64_t room, int64_t* done) {
     if (c->res.ctas > 0 && resident2d_clusters(c->res, c->storage, c->coll) < 1) c->res.ctas = 0;
   }
   if (c->res.ctas == 0) return XLB_OK;
-  // An update costs 0.6 us and 0.9 us more for each 1024 cells a block (128^2 on
-  // 16 blocks: 1.5 us; KBC twice that).  (Lattices with more cells a block than
-  // threads are not taken: the tiles are faster, 256 x 128 2.0 us against 3.5.)
-  const double cells = (double)((c->ny + c->res.ctas - 1) / c->res.ctas * c->nx);
-  const double us = 0.6 + 0.9 * cells / 1024.0 * (c->coll == XLB_COLL_KBC ? 2.0 : 1.0);
-  if (us > single_update_us(c, c->graph_g > 0) || (tile_ok(c) && us > c->tile.us)) return XLB_OK;
+  // (Lattices with more cells a block than threads are not taken: the tiles are
+  // faster, 256 x 128 2.0 us an update against 3.5.)
+  const double us = resident_us(c, room);
+  if (us >= single_updates_us(c, room, captured) || (tile_ok(c, room, captured) && us > tile_us(c, room))) return XLB_OK;
   ResidentArgs a;
   memset(&a, 0, sizeof a);
   a.src = c->buf[c->cur];
@@ -1484,7 +1546,7 @@ int xlb_step(xlb_ctx* c, int64_t n) {
       r = step_last_segment(c, room, &m);
       if (r) return r;
       if (c->tape_open) room = std::min(room, c->tape_k - c->t % c->tape_k);
-      if (m == 0) r = step_resident(c, room, &m);
+      if (m == 0) r = step_resident(c, room, captured, &m);
       if (r) return r;
       if (m > 0) {
         c->t += m;
@@ -1512,7 +1574,7 @@ int xlb_step(xlb_ctx* c, int64_t n) {
       // up to the next checkpoint of an open tape
       m = n - k;
       if (c->tape_open) m = std::min(m, c->tape_k - c->t % c->tape_k);
-      r = run_updates(c, &c->cur, m, captured);
+      r = run_updates(c, &c->cur, m, captured, captured);
     }
     if (r) return r;
     c->t += m;

@@ -408,11 +408,10 @@ int tile_by_coll(const Tile2dArgs& a) {
 
 // Tiles that a model of the kernel expects to take the least time per update:
 // waves of blocks over the SMs, 5 us a launch for load and store, and per update
-// 0.8 us and a time for each round of two cells per thread.  Measured per update
-// (FP32 BGK with walls) 300 x 200: 2.3 us, launched one by one 4.9, graph 4.1;
-// 601 x 599: 4.7, 7.6 and 7.0; the 1761 x 330 cylinder 7.5, graph 11.5.
+// 0.8 us and a time for each round of two cells per thread.  (It ranks plans; what
+// one takes is tile_us in api.cu.)
 Tile2dPlan tile2d_plan(int storage, int coll, int nx, int ny) {
-  Tile2dPlan best = {0, 0, 0, 0, 0, 0.f};
+  Tile2dPlan best = {0, 0, 0, 0, 0, 0.f, 0};
   const float over = 5.0f, per = coll == COLL_KBC ? 2.9f : storage == XLB_STORE_BF16 ? 1.8f : 0.85f;
   for (int tx = 1; tx <= nx && tx <= 152; ++tx) {
     const int bx = (nx + tx - 1) / tx;
@@ -422,7 +421,6 @@ Tile2dPlan tile2d_plan(int storage, int coll, int nx, int ny) {
       if ((ny + by - 1) / by != ty) continue;
       for (int h = 2; h <= 12; ++h) {
         if (bx + 2 * h > nx || by + 2 * h > ny) break;  // a cell at most once in a region
-        const long long cells = (long long)(bx + 2 * h) * (by + 2 * h);
         const long long smem = storage == XLB_STORE_F32 ? tile_smem<float>(bx, by, h) : tile_smem<__half>(bx, by, h);
         if (smem > TILE_SMEM) break;
         const int waves = (tx * ty + 151) / 152;
@@ -430,7 +428,7 @@ Tile2dPlan tile2d_plan(int storage, int coll, int nx, int ny) {
         const long long busy = (long long)(bx + 2 * h) * (by + h - 1);
         const float rounds = (float)((busy + 2 * TILE_THREADS - 1) / (2 * TILE_THREADS));
         const float us = waves * (over + h * (0.8f + rounds * per)) / h;
-        if (best.halo == 0 || us < best.us) best = {bx, by, tx, ty, h, us};
+        if (best.halo == 0 || us < best.us) best = {bx, by, tx, ty, h, us, waves};
       }
     }
   }

@@ -12,7 +12,8 @@ namespace xlb {
 // halo = 0: no plan.
 struct Tile2dPlan {
   int bx, by, tx, ty, halo;
-  float us;  // the model's time per update
+  float us;   // the time per update by which plans are compared
+  int waves;  // of blocks, one per SM
 };
 
 Tile2dPlan tile2d_plan(int storage, int coll, int nx, int ny);

@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 N = 40
 
 
-def _kernels(shape, storage, variant="auto", prepare=None, mask=None):
+def _kernels(shape, storage, variant="auto", prepare=None, mask=None, steps=N):
     st = torch.cuda.Stream()
     r, u = I.random_flow(shape, 2, seed=111, rho_amp=0.005, u_amp=0.02)
     if mask is None:
@@ -28,7 +28,7 @@ def _kernels(shape, storage, variant="auto", prepare=None, mask=None):
         prepare(s)
     s.init(r.astype(np.float32), u.astype(np.float32))
     s.step(1)
-    n = kernels_of(st.cuda_stream, lambda: s.step(N))
+    n = kernels_of(st.cuda_stream, lambda: s.step(steps))
     s.close()
     return n
 
@@ -52,3 +52,10 @@ def test_profiled_updates_are_launched_one_by_one():
 @pytest.mark.parametrize("shape", [(64, 68), (200, 320)])
 def test_a_chosen_variant_launches_every_update(shape, storage, variant):
     assert _kernels(shape, storage, variant) >= N
+
+
+# (us launched one by one / together: 4.6 / 9.2, 8.3 / 12.8, 28.3 / 42.9, 84.8 / 128.6)
+@pytest.mark.parametrize("shape,storage,n", [((128, 128), "f32", 2), ((599, 601), "f16", 2), ((1000, 1200), "f16", 4),
+                                             ((1000, 1200), "f16", 12), ((800, 900), "bf16", 24)])
+def test_calls_that_gain_nothing_launch_every_update(shape, storage, n):
+    assert _kernels(shape, storage, mask=np.zeros(shape, np.uint8), steps=n) == n
