@@ -939,8 +939,10 @@ __global__ void __launch_bounds__(ROW_BLOCK) k_readout(const S* f, const StepPar
       u[1] = p.eq_u[1];
       u[2] = Lattice<Q>::D == 3 ? p.eq_u[2] : 0.f;
     }
-    const double u0 = u[0], u1 = u[1], u2 = u[2];
-    acc[0] += 0.5 * (double)rho * (u0 * u0 + u1 * u1 + u2 * u2);
+    if (mode == RD_KE) {  // (the moments are the fluid-like cells' alone)
+      const double u0 = u[0], u1 = u[1], u2 = u[2];
+      acc[0] += 0.5 * (double)rho * (u0 * u0 + u1 * u1 + u2 * u2);
+    }
   }
   __shared__ double red[ROW_BLOCK / 32][4];
 #pragma unroll
