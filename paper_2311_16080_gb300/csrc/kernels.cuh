@@ -27,7 +27,7 @@ struct CellIdx {
 
 // a / n and its remainder, m = magic_of(n)
 __device__ __forceinline__ int divide(int a, int n, uint32_t m, int& rem) {
-  if (m == 0u) {  // n = 1
+  if (m == 1u) {  // n = 1
     rem = 0;
     return a;
   }

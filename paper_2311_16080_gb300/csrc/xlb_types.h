@@ -72,9 +72,11 @@ struct StepParams {
 };
 
 // Division of a cell or row index (below 2^31) by an extent n >= 2 as a
-// multiplication: the quotient's estimate is exact or one too large.  0 stands
-// for n = 1.
-inline uint32_t magic_of(int n) { return (uint32_t)(((1ULL << 32) + (unsigned)n - 1) / (unsigned)n); }
+// multiplication: the quotient's estimate is exact or one too large.  1 (which no
+// other extent has) stands for n = 1.
+inline uint32_t magic_of(int n) {
+  return n == 1 ? 1u : (uint32_t)(((1ULL << 32) + (unsigned)n - 1) / (unsigned)n);
+}
 
 // Ghost link entries are int2 {cell, dir | type << 8 | flags << 16}; LINK_BZ
 // marks a WALL link with a Bouzidi wall distance (in a parallel float array).
