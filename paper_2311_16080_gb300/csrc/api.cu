@@ -491,11 +491,26 @@ static int launch_collide_local(xlb_ctx* c, void* buf) {
   return r;
 }
 
+// Whether forming f_0 again from the initial fields beats reading it.  FP32 reads
+// (1 + D) values in place of Q (first update of 256^3 D3Q19 376 -> 250 us; D2Q9
+// gains once the state leaves L2, 4000^2 174 -> 139 us, 1000^2 10.3 -> 11.2), FP16
+// little (256^3 259 -> 237 us, 64^3 6.3 -> 7.2, D2Q9 4000^2 129 -> 141); BF16 would
+// round stochastically twice (256^3 330 -> 416 us).  Not beside scattered solid
+// cells, whose sectors are then written in part without having been read (5% of
+// them: 256^3 FP32 733 -> 852 us).
+static bool first_from_fields(const xlb_ctx* c) {
+  if (c->n_links >= c->N / 16) return false;
+  const size_t bytes = state_bytes_raw(c);
+  if (c->storage == XLB_STORE_F32) return c->Q != 9 || bytes > (128u << 20);
+  return c->storage == XLB_STORE_F16 && c->Q != 9 && bytes > (64u << 20);
+}
+
 // The first update: from the initial fields where the state is still f_0 as
 // xlb_init left it, else a local collision of the stored state.  So too in a
 // caller's capture: its replays may find another state there.
 static int launch_first(xlb_ctx* c, void* buf, bool captured) {
-  if (captured || c->init_epoch != c->epoch || c->coll == XLB_COLL_NONE) return launch_collide_local(c, buf);
+  if (captured || c->init_epoch != c->epoch || c->coll == XLB_COLL_NONE || !first_from_fields(c))
+    return launch_collide_local(c, buf);
   LaunchArgs a = base_args(c);
   a.dst = buf;
   a.rho = c->init_fields;
