@@ -938,6 +938,8 @@ __global__ void __launch_bounds__(ROW_BLOCK) k_readout(const S* f, const StepPar
       u[0] = p.eq_u[0];
       u[1] = p.eq_u[1];
       u[2] = Lattice<Q>::D == 3 ? p.eq_u[2] : 0.f;
+    } else {
+      continue;  // (its zeros would take the FP64 lines a second time per warp)
     }
     if (mode == RD_KE) {  // (the moments are the fluid-like cells' alone)
       const double u0 = u[0], u1 = u[1], u2 = u[2];
@@ -974,7 +976,8 @@ __global__ void __launch_bounds__(ROW_BLOCK, MinBlocks<Q, S, COLL_BGK>::value) k
   float rho = 0.f, u[3] = {0.f, 0.f, 0.f};
   if (fluid_like(t)) {
     float df[Q];
-    if (kind_h && !(fl & FLAG_SLOW)) {
+    // (chosen per warp: among scattered walls both ways would be taken)
+    if (kind_h && !__any_sync(__activemask(), fl & FLAG_SLOW)) {
       Nbr nb;
       make_nbr(nb, c.x, c.y, c.z, p.nx, p.ny, p.nz);
       pull_plain<Q, S>(f, p, nb, df);
