@@ -475,7 +475,10 @@ static int materialize_post_stream(xlb_ctx* c) {
   c->init_epoch = 0;
   const int coll = c->coll;
   c->coll = XLB_COLL_NONE;
-  const int r = launch_step(c, c->buf[c->cur], c->buf[c->cur ^ 1]);
+  int r = launch_step(c, c->buf[c->cur], c->buf[c->cur ^ 1]);
+  // (a new mask may turn x-face cells into fluid: what their slots hold does not
+  // depend on the kernel that has served the faces)
+  if (!r && pulls_x_faces(c)) r = write_links(c, c->buf[c->cur ^ 1]);
   c->coll = coll;
   if (r) return r;
   c->cur ^= 1;
@@ -526,6 +529,21 @@ static int launch_init(xlb_ctx* c, void* dst) {
   a.rho = c->init_fields;
   a.u = c->init_fields + c->N;
   return dispatch(c, OP_INIT, a);
+}
+
+// Before the stored bytes are handed out, or a new mask turns WALL cells into fluid:
+// slots of WALL cells that no update of the resident and the tiled kernel writes
+// hold whatever the buffer had (at first, old device memory).  They become the
+// rest state, with the ghost values of the present one where it has them.  (Done
+// here, not in the kernels: carrying the slots over in each launch cost the 1761 x
+// 330 cylinder 4 to 7% of an update.)
+static int settle_walls(xlb_ctx* c) {
+  if (!c->loose_walls || !c->has_mask) return XLB_OK;
+  if (launch_clear_walls(c->buf[c->cur], c->esize, c->flags, c->Q, c->N, c->plane, c->stream) != 0)
+    return fail(c, XLB_ERR_CUDA, "clearing of WALL cells rejected");
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(c, e, "clearing of WALL cells");
+  return c->kind_h ? boundary_pass(c, nullptr, c->buf[c->cur]) : XLB_OK;
 }
 
 static void free_bz(xlb_ctx* c) {
@@ -931,7 +949,8 @@ int xlb_set_mask(xlb_ctx* c, const uint8_t* mask) {
     }
   }
   {
-    const int r = materialize_post_stream(c);  // f_t under the old mask
+    int r = settle_walls(c);
+    if (!r) r = materialize_post_stream(c);  // f_t under the old mask
     if (r) {
       cudaFree(nf);
       if (nlinks) cudaFree(nlinks);
@@ -1769,20 +1788,6 @@ int xlb_state_bytes(const xlb_ctx* c, size_t* bytes) {
   if (!c || !bytes) return XLB_ERR_ARG;
   *bytes = 64 + state_bytes_raw(c);
   return XLB_OK;
-}
-
-// Before the stored bytes are handed out: WALL cells' slots that no update of
-// the resident and the tiled kernel writes hold whatever the buffer had (at
-// first, old device memory).  They become the rest state with the ghost values
-// of the present one.  (Done here, not in the kernels: carrying the slots over
-// in each launch cost the 1761 x 330 cylinder 4 to 7% of an update.)
-static int settle_walls(xlb_ctx* c) {
-  if (!c->loose_walls || !c->kind_h || !c->has_mask) return XLB_OK;
-  if (launch_clear_walls(c->buf[c->cur], c->esize, c->flags, c->Q, c->N, c->plane, c->stream) != 0)
-    return fail(c, XLB_ERR_CUDA, "clearing of WALL cells rejected");
-  const cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return cuda_fail(c, e, "clearing of WALL cells");
-  return boundary_pass(c, nullptr, c->buf[c->cur]);
 }
 
 int xlb_state_get(xlb_ctx* c, void* buf, size_t bytes) {
