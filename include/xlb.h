@@ -120,7 +120,9 @@ double xlb_omega_from_nu(double nu);
  * Codes >= 7 give XLB_ERR_ARG and leave the previous mask in place.  Between
  * steps, a new mask (like new boundary values from xlb_set_bc) acts from the
  * next step on: the current state keeps the boundaries it was streamed with.
- * XLB_ERR_STATE while a tape is open. */
+ * Solid cells that it turns into fluid start from the values their slots hold,
+ * which may depend on how the updates before were launched (xlb_init sets every
+ * cell).  XLB_ERR_STATE while a tape is open. */
 int xlb_set_mask(xlb_ctx* ctx, const uint8_t* mask);
 
 /* Sizes of the boundary tables of the current mask.  Whole face planes that
