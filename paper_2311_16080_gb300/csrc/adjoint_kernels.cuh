@@ -136,10 +136,7 @@ __device__ __forceinline__ void init_state(const float* rho0, const float* u0, l
   u[0] = u0[self];
   u[1] = u0[ucs + self];
   u[2] = Lattice<Q>::D == 3 ? u0[2 * ucs + self] : 0.f;
-  const float usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-  const float drho = rho - 1.0f;
-#pragma unroll
-  for (int i = 0; i < Q; ++i) df[i] = weight<Q>(i) * (drho + rho * eq_poly<Q>(i, u, usq));
+  init_deviations<Q>(rho, u, df);
   CellRound<S> rnd;
   rnd.begin((uint32_t)self, df);
 #pragma unroll

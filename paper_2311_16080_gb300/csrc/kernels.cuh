@@ -806,10 +806,7 @@ __device__ __forceinline__ void init_cell(const float* rho_in, const float* u_in
     u[1] = u_in[ucs + self];
     if (Lattice<Q>::D == 3) u[2] = u_in[2 * ucs + self];
   }
-  const float usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-  const float drho = rho - 1.0f;
-#pragma unroll
-  for (int i = 0; i < Q; ++i) df[i] = weight<Q>(i) * (drho + rho * eq_poly<Q>(i, u, usq));
+  init_deviations<Q>(rho, u, df);
 }
 
 // The first update after an initialisation, a local collision of f_0: f_0 is

@@ -98,6 +98,25 @@ __device__ __forceinline__ float eq_poly(int i, const float (&u)[3], float usq) 
   return cu * (3.0f + 4.5f * cu) - 1.5f * usq;
 }
 
+// Deviations f_i^eq(rho, u) - w_i of an initial state, before storage rounds them.
+// Every rounding is spelled out: the kernels that form f_0 (the initialisation, the
+// first update, the adjoint's first step) must agree to the bit, or 16-bit storage
+// rounds some values apart.
+template <int Q>
+__device__ __forceinline__ void init_deviations(float rho, const float (&u)[3], float (&df)[Q]) {
+  const float usq = __fmaf_rn(u[2], u[2], __fmaf_rn(u[1], u[1], __fmul_rn(u[0], u[0])));
+  const float drho = __fsub_rn(rho, 1.0f), b = __fmul_rn(1.5f, usq);
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    float cu = 0.f;
+#pragma unroll
+    for (int a = 0; a < Lattice<Q>::D; ++a)
+      if (Lattice<Q>::c(i, a)) cu = __fmaf_rn((float)Lattice<Q>::c(i, a), u[a], cu);
+    const float x = __fmaf_rn(cu, __fmaf_rn(4.5f, cu, 3.0f), -b);
+    df[i] = __fmul_rn(weight<Q>(i), __fmaf_rn(rho, x, drho));
+  }
+}
+
 // c_i . u
 template <int Q>
 __device__ __forceinline__ float cdot(int i, const float (&u)[3]) {
