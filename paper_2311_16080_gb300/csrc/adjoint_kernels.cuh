@@ -127,8 +127,8 @@ __device__ __forceinline__ void zero_out(float* aout, const StepParams& p, int s
   for (int i = 0; i < Q; ++i) aout[(long long)i * p.plane + self] = 0.f;
 }
 
-// f_0 of a fluid-like cell exactly as the forward initialisation stored it:
-// f^eq(rho0, u0) rounded through the storage type.
+// f_0 of a fluid-like cell as the forward initialisation stored it: f^eq(rho0, u0)
+// rounded through the storage type (before that, to the last FP32 bit or two).
 template <int Q, typename S>
 __device__ __forceinline__ void init_state(const float* rho0, const float* u0, long long ucs, int self,
                                            float (&df)[Q], float& rho, float (&u)[3]) {
@@ -136,7 +136,10 @@ __device__ __forceinline__ void init_state(const float* rho0, const float* u0, l
   u[0] = u0[self];
   u[1] = u0[ucs + self];
   u[2] = Lattice<Q>::D == 3 ? u0[2 * ucs + self] : 0.f;
-  init_deviations<Q>(rho, u, df);
+  const float usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+  const float drho = rho - 1.0f;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) df[i] = weight<Q>(i) * (drho + rho * eq_poly<Q>(i, u, usq));
   CellRound<S> rnd;
   rnd.begin((uint32_t)self, df);
 #pragma unroll

@@ -99,8 +99,8 @@ __device__ __forceinline__ float eq_poly(int i, const float (&u)[3], float usq) 
 }
 
 // Deviations f_i^eq(rho, u) - w_i of an initial state, before storage rounds them.
-// Every rounding is spelled out: the kernels that form f_0 (the initialisation, the
-// first update, the adjoint's first step) must agree to the bit, or 16-bit storage
+// Every rounding is spelled out: the kernels that form f_0 (the initialisation and
+// the first update, for every storage type) must agree to the bit, or 16-bit storage
 // rounds some values apart.
 template <int Q>
 __device__ __forceinline__ void init_deviations(float rho, const float (&u)[3], float (&df)[Q]) {
