@@ -59,7 +59,7 @@ struct xlb_ctx {
   cudaStream_t aux = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int face[6] = {0, 0, 0, 0, 0, 0};  // described boundary faces (StepParams::face)
-  bool x_linked = false;             // the x-faces' sources are served by ghost links
+  bool x_linked = false;             // the x-faces' sources have ghost links
   bool x_pull = false;               // ... which are the only ones (pulls_x_faces)
   bool x_inlet = false;              // the x = 0 plane is INLET, served by the bulk pass
   bool x_outlet = false;             // the x = nx - 1 plane is OUTLET, served by the bulk pass
@@ -873,10 +873,11 @@ int xlb_set_mask(xlb_ctx* c, const uint8_t* mask) {
   // With 16-bit storage the bulk pass is bound by instruction issue, and the
   // x-face rules would run in diverging lanes at both ends of every row: the
   // sources on WALL / LID / EQ x-face planes (outside the skipped y / z face
-  // rows) go to the ghost links instead, written by the boundary pass after
-  // each update.  The x-faces still take part in deriving the rule of the
-  // cells where planes meet.  Lattices with an FWALL x-face keep the rules in
-  // the pull.  (Two forms that write these values from the bulk pass itself
+  // rows) have ghost links instead, written by the boundary pass after each
+  // update; with one cell per thread the pull serves them after all where they
+  // are the only links (pulls_x_faces), which spares that pass.  The x-faces
+  // still take part in deriving the rule of the cells where planes meet.
+  // Lattices with an FWALL x-face keep the rules in the pull.  (Two forms that write these values from the bulk pass itself
   // measured slower on the FP16 256^3 cavity: ghost values held in each
   // row's face cell, 55.7 k against 59.9 k MLUPS, and ghost values pushed by
   // the cells next to the faces, 57.9 k against 58.7 k: both diverge the

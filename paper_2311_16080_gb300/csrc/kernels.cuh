@@ -123,9 +123,9 @@ __device__ __forceinline__ int fc_type(uint32_t fc, int axis, int k) { return (i
 template <bool FW>
 __device__ __forceinline__ uint32_t face_code(const StepParams& p, int x, int y, int z) {
   if (!p.has_faces) return 0u;
-  // a row two or more planes away from the y / z boundary planes (uniform
-  // over a warp, which covers one row) can only meet x-faces: their types
-  // follow from four compares per lane
+  // a row two or more planes away from the y / z boundary planes can only meet
+  // x-faces: their types follow from four compares per lane (uniform over a warp
+  // where rows fill whole blocks; on the flat mapping a warp may hold two rows)
   if (y > 1 && y < p.ny - 2 && (p.nz == 1 || (z > 1 && z < p.nz - 2))) {
     if ((p.face[0] | p.face[1]) == 0 || (x > 1 && x < p.nx - 2)) return 0u;
     const int tm = (x == 1 ? p.face[0] : 0) | (x == 0 ? p.face[1] : 0);           // x - 1
@@ -327,14 +327,15 @@ __device__ __forceinline__ void store_cell(S* dst, const StepParams& p, int self
 // Which mechanism delivers the rules of the boundary faces to the bulk pass:
 // with 16-bit storage the cells of y / z face rows are skipped and take
 // ghost values pushed by the rows next to them, and the sources on x-face
-// planes are ghost links (p.x_linked) or, with an FWALL x-face, take the
-// rules inside the pull (the kernel is bound by instruction issue: whole
-// warps skip or push, and at most the lanes at the ends of a row run face
-// logic); FP32 applies every face rule by coordinates
-// inside the pull (the kernel is bound by memory traffic, and the face logic
-// hides under it).  Both give the same pulled values; the readouts, the
-// boundary pass and the adjoint apply the face rules by coordinates and never
-// read face cells.
+// planes take the rules inside the pull, where they are the lattice's only links
+// without wall distances or belong to an FWALL x-face, and are ghost links
+// otherwise (p.x_linked; always with two or four cells per thread).  The kernel
+// is bound by instruction issue: whole warps skip or push, and at most the lanes
+// at the ends of a row run face logic.  FP32 applies every face rule by
+// coordinates inside the pull (the kernel is bound by memory traffic, and the
+// face logic hides under it).  Both give the same pulled values; the readouts,
+// the boundary pass and the adjoint apply the face rules by coordinates and
+// never read face cells.
 template <typename S>
 struct GhostFaces {
   static constexpr bool value = sizeof(S) == 2;

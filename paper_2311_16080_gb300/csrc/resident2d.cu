@@ -188,7 +188,9 @@ __device__ __forceinline__ void update_pair(const uint32_t (&L0)[9], const uint3
   }
 }
 
-// Bounds: a batch by FP32 instruction issue; one small domain by the latency
+// Bounds: a batch by FP32 instruction issue (608 domains of 60 x 44, one block
+// each: 128 instructions per cell and update, 0.58 issued per cycle and scheduler,
+// then math pipe and barrier stalls); one small domain by the latency
 // of a cluster barrier (287 ns) and of one cell's chain.  Each thread takes two
 // cells a warp's width apart: the lanes of a warp stay on consecutive cells, the
 // collision runs in packed arithmetic, and few warps hold cells of the rows

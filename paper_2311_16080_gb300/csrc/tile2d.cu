@@ -144,9 +144,11 @@ __device__ __forceinline__ void special_push(const StepParams& p, int self, cons
   }
 }
 
-// Bounds: FP32 instruction issue, as for the resident kernel (about 130
-// instructions per cell and update); the load and store of the tile and the
-// launch, some 4.5 us, are shared by the updates of a launch.
+// Bounds: FP32 instruction issue and the loads of a launch.  The 1761 x 330 cylinder,
+// 4 updates a launch: 227 instructions per lattice cell and update (of which the
+// ring and the meta words are some 100), 0.46 issued per cycle and scheduler; waits
+// for the tile's loads lead the stalls.  A launch costs 7 us on regions of 2,100
+// cells and 12 on 5,500, shared by its updates.
 template <typename S, int COLL>
 __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile2d(const S* A, S* B,
                                                             const StepParams p, const int* __restrict__ bz,

@@ -56,7 +56,8 @@ struct StepParams {
   int face[6];
   int has_faces;
   // 16-bit bulk passes: the sources on the x-face planes outside the skipped
-  // y / z face rows are served by ghost links, not by rules in the pull
+  // y / z face rows are read from ghost links in this launch, not served by
+  // rules in the pull
   int x_linked;
   // the x = 0 plane is INLET / the x = nx - 1 plane is OUTLET (outside the
   // y / z face planes): the bulk pass applies the inlet rule / the outflow
